@@ -497,7 +497,7 @@ extern "C" vne_status vne_quadrature_bounds(vne_ctx* ctx, const double* alpha, c
     double* dn = upload(ctx, "tb.n", nn);
     double* dout = ws_get_t<double>(ctx, "tb.out", 3 * (size_t)count);
     VNE_TRY_CUDA(ctx, launch_tridiag_bounds(da, db, dn, ds, count, m, count, lam_min, lam_max, grid, dout,
-                                            dout + count, dout + 2 * count, ctx->stream));
+                                            dout + count, dout + 2 * count, nullptr, ctx->stream));
     ctx->launches += 1;
     std::vector<double> h = download(ctx, dout, 3 * (size_t)count);
     std::copy(h.begin(), h.begin() + count, lower);

@@ -533,10 +533,9 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
             j = j1;
             m_run = j;
             if (j >= m) break;
-            VNE_TRY_CUDA(ctx, launch_tridiag_quad(alpha, beta, norm2, dscale, SK, j, SK, psi, st));
             VNE_TRY_CUDA(ctx, launch_tridiag_bounds(alpha, beta, norm2, dscale, SK, j, SK, ad->lam_min, ad->lam_max,
-                                                    ad->grid, est, est + SK, est + 2 * SK, st));
-            ctx->launches += 2;
+                                                    ad->grid, est, est + SK, est + 2 * SK, psi, st));
+            ctx->launches += 1;
             std::vector<double> hp = download(ctx, psi, SK), he = download(ctx, est + 2 * SK, SK);
             bool done = true;
             if (ad->abs)

@@ -166,17 +166,17 @@ __host__ __device__ inline bool symtri_qr_first_row(double* d, double* e, double
 // ---------------------------------------------------------------------------
 // Gauss quadrature psi = ||c||^2 sum_j u_{1j}^2 f(sigma theta_j) of the
 // leading unreduced block of T (Golub & Meurant, Matrices, Moments and
-// Quadrature, Ch. 6), one warp per tridiagonal with the eigenvalues spread
-// over the lanes.  GB300 retires FP64 instructions slowly and with long
-// latency, so one long sequential QR chain per column is the slowest possible
-// schedule; here every lane runs short independent chains:
+// Quadrature, Ch. 6), one CTA per tridiagonal with the eigenvalues spread
+// over the threads.  GB300 retires FP64 instructions slowly, so one long
+// sequential QR chain per column is the slowest possible schedule; here every
+// lane runs short independent chains:
 //  * theta_j by bisection on the Sturm count #{theta < z} (number of k with
 //    sign p_k(z) = sign p_{k-1}(z), p_k = det(z I - T_k) by the three-term
 //    recurrence, rescaled by powers of two every four steps; Wilkinson, The
-//    Algebraic Eigenvalue Problem, Ch. 5): FP32 halvings first narrow the
-//    Gershgorin interval, FP64 counts check the bracket, then FP64
-//    quadrisection with all of a lane's points evaluated as interleaved
-//    independent recurrences, a warp-uniform number of passes;
+//    Algebraic Eigenvalue Problem, Ch. 5): FP32 counts first narrow the
+//    Gershgorin interval, FP64 counts check the bracket, a bracket that holds
+//    one eigenvalue goes to Newton's iteration on p_n, others are searched on
+//    with FP64 counts (four trial points per pass and eigenvalue);
 //  * u_{1j}^2 from the eigenvector of the twisted factorisation
 //    T - theta I = N_r Delta_r N_r^T at the twist index r of smallest
 //    |gamma_r| (Parlett & Dhillon, Lin. Alg. Appl. 309, 2000): z_r = 1,
@@ -315,41 +315,8 @@ __device__ __forceinline__ int sturm_count_f32(const float* a, const float* b2, 
 }
 
 __device__ __forceinline__ double guard_pivot(double x, double pivmin) {
-    return fabs(x) < pivmin ? (x < 0.0 ? -pivmin : pivmin) : x;
-}
-
-// u_{1j}^2 by the twisted factorisation at an isolated eigenvalue th.
-// Dp / Rp: this lane's columns of the pivot scratch ([k][32] doubles).
-__device__ double twisted_weight(const double* a, const double* b, int n, double th, double pivmin, double* Dp,
-                                 double* Rp) {
-    double d = 0.0;
-    for (int k = 0; k < n; k++) {
-        d = guard_pivot((a[k] - th) - (k > 0 ? b[k - 1] * b[k - 1] / d : 0.0), pivmin);
-        Dp[k * 32] = d;
-    }
-    double r = 0.0, best = INFINITY;
-    int tw = n - 1;
-    for (int k = n - 1; k >= 0; k--) {
-        r = guard_pivot((a[k] - th) - (k + 1 < n ? b[k] * b[k] / r : 0.0), pivmin);
-        Rp[k * 32] = r;
-        const double gam = fabs(Dp[k * 32] + r - (a[k] - th));
-        if (gam < best) {
-            best = gam;
-            tw = k;
-        }
-    }
-    double s = 1.0, z = 1.0;
-    for (int k = tw - 1; k >= 0; k--) {
-        z = -b[k] * z / Dp[k * 32];
-        s = fma(z, z, s);
-    }
-    const double z1 = tw > 0 ? z : 1.0;
-    z = 1.0;
-    for (int k = tw + 1; k < n; k++) {
-        z = -b[k - 1] * z / Rp[k * 32];
-        s = fma(z, z, s);
-    }
-    return z1 * z1 / s;
+    // compared by their bits: an FP64 comparison would take a slot of the FP64 port
+    return absbits(x) < absbits(pivmin) ? copysign(pivmin, x == 0.0 ? 1.0 : x) : x;
 }
 
 // Point q of the K-point trapezoid rule on the circle z = c + rho e^{i phi}:
@@ -398,24 +365,71 @@ __device__ void quad_by_qr(const double* sa, const double* sb, int n, double sc,
     *out = ok ? norm2 * s : nan("");
 }
 
-// Shared state of the spectral kernels for one tridiagonal (one warp).
+// Shapes of the spectral kernels.  FP64 bounds them: GB300 issues one FP64
+// instruction per warp and sub-partition in 64 cycles whatever its
+// independence (measured: 0.5 lane operations per cycle for one warp, 1.7 per
+// SM; a division takes 9, a reciprocal 6, a logarithm 32 such slots), while
+// FP32, integer and conversion instructions run at full rate.  One warp per
+// tridiagonal therefore leaves three of an SM's four FP64 issue ports idle
+// and pays for every lane loop in full, so a CTA of 4 MAXM threads takes one
+// tridiagonal: four lanes per eigenvalue in the searches (one trial point
+// each), one lane in Newton's iteration, two lanes in the twisted
+// factorisation (top-down and bottom-up pivots at the same time).
+// Measured (a CTA per tridiagonal against one warp): 104 quadratures of order
+// 50 in 0.10 ms (0.59); 3072 of order 40 in 1.30 ms (2.38); one Krylov check
+// of a server (quadrature and 512 grid points of Theorem 4.4, some hundred
+// columns of order 3 to 9) in 0.071 ms (0.320 in two kernels).
+template <int MAXM>
+struct TqCfg {
+    static constexpr int NT = 4 * MAXM;                 // threads per CTA
+    static constexpr int NW = NT / 32;
+    static constexpr int RB = MAXM < 64 ? MAXM : 64;    // eigenvectors per pass of the pivot scratch
+    static constexpr int LD = RB + 1;                   // row stride of the scratch (conflict-free both ways)
+    static constexpr int kSmem = 2 * MAXM * LD * (int)sizeof(double);
+};
+
+// Shared state of the spectral kernels for one tridiagonal (one CTA).
 template <int MAXM>
 struct TqShared {
-    double a[MAXM], b[MAXM], b2[MAXM + 1];  // scaled block, b2[k] = beta_{k-1}^2
+    double a[MAXM], b[MAXM], b2[MAXM + 1];  // scaled block, b2[k] = beta_{k-1}^2, b2[n] = 0
     double th[MAXM], bw[MAXM];              // eigenvalues (ascending), bracket widths
+    double z1[MAXM], zn[MAXM], nrm[MAXM];   // first / last entry and squared norm of the twisted eigenvectors
+    double c0[MAXM], c1[MAXM];              // per-eigenvalue terms of the final sums
+    double k0[MAXM / 2], k1[MAXM / 2], k2[MAXM / 2];  // per-cluster terms
     float a32[MAXM], b2_32[MAXM + 1];
     double cc[MAXM / 2], rho[MAXM / 2], half[MAXM / 2];  // clusters: centre, circle radius, half-width
     int gfirst[MAXM + 1], glast[MAXM], cl_of_group[MAXM];
-    int ngroups, ncl, fallback, n;
-    double span, s2, pivmin;
+    int clo[MAXM], chi[MAXM];  // Sturm counts at the ends of the brackets (searches)
+    int ngroups, ncl, fallback, n, finite;
+    double span, s2, pivmin, glo, ghi;
+    float pivmin32;
+    unsigned long long gmin, gmax;
 };
 
+// Choose the sub-interval of [lo, hi] that holds eigenvalue j from the counts
+// of four ascending interior points, one per lane of the quad (all four lanes
+// of the quad end with the same bracket).
+__device__ __forceinline__ void quad_choose(int j, int lane, double z, int cnt, double& lo, double& hi, int& clo,
+                                            int& chi) {
+    const int base = lane & 28;
+    const unsigned above = (__ballot_sync(0xffffffffu, cnt > j) >> base) & 15u;
+    const int i = above ? __ffs(above) - 1 : 4;  // first point above eigenvalue j
+    const double zu = __shfl_sync(0xffffffffu, z, base + (i < 4 ? i : 3));
+    const int cu = __shfl_sync(0xffffffffu, cnt, base + (i < 4 ? i : 3));
+    const double zl = __shfl_sync(0xffffffffu, z, base + (i > 0 ? i - 1 : 0));
+    const int cl = __shfl_sync(0xffffffffu, cnt, base + (i > 0 ? i - 1 : 0));
+    if (i < 4) hi = zu, chi = cu;
+    if (i > 0) lo = zl, clo = cl;
+}
+
 // Eigenvalues and their grouping for the leading unreduced block of
-// tridiagonal c (all 32 lanes call it).  Returns false if the block has a
-// non-finite entry.
+// tridiagonal c (every thread of the CTA calls it).  Returns false if the
+// block has a non-finite entry.
 template <int MAXM>
 __device__ bool tq_spectrum(const double* __restrict__ alpha, const double* __restrict__ beta, int c, int m, int ld,
-                            int lane, TqShared<MAXM>& S) {
+                            TqShared<MAXM>& S) {
+    constexpr int NT = TqCfg<MAXM>::NT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double* sa = S.a;
     double* sb = S.b;
     double* sb2 = S.b2;
@@ -423,191 +437,194 @@ __device__ bool tq_spectrum(const double* __restrict__ alpha, const double* __re
     double* sbw = S.bw;
     float* sa32 = S.a32;
     float* sb2_32 = S.b2_32;
-    // leading unreduced block: n = 1 + first j with beta_j == 0
-    int n = m;
-    for (int j0 = 0; j0 < m - 1; j0 += 32) {
-        const int j = j0 + lane;
-        const bool zero = j < m - 1 && beta[(size_t)j * ld + c] == 0.0;
-        const unsigned zb = __ballot_sync(0xffffffffu, zero);
-        if (zb) {
-            n = j0 + __ffs(zb);
-            break;
-        }
-    }
-    bool finite = true;
-    double glo = INFINITY, ghi = -INFINITY, bmax = 0.0;
-    for (int j = lane; j < n; j += 32) {
-        const double aj = alpha[(size_t)j * ld + c];
-        const double bj = (j + 1 < n) ? beta[(size_t)j * ld + c] : 0.0;
-        const double bp = (j > 0) ? beta[(size_t)(j - 1) * ld + c] : 0.0;
-        sa[j] = aj;
-        sb[j] = bj;
-        sb2[j + 1] = bj * bj;
-        finite = finite && isfinite(aj) && isfinite(bj);
-        const double r = fabs(bj) + fabs(bp);
-        glo = fmin(glo, aj - r);
-        ghi = fmax(ghi, aj + r);
-        bmax = fmax(bmax, bj * bj);
-    }
-    if (lane == 0) {
-        sb2[0] = 0.0;
-        sb2_32[0] = 0.f;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, off));
-        ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, off));
-        bmax = fmax(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
-    }
-    finite = __all_sync(0xffffffffu, finite);
-    __syncwarp();
-    if (!finite) return false;
-    // scale the block by the power of two s2 that brings its Gershgorin
-    // radius to [1, 2) (exact: eigenvalues scale by s2, weights do not), so
-    // the unnormalised Sturm recurrences stay far from overflow
-    const double s2 = pow2_rescale(absbits(fmax(fmax(fabs(glo), fabs(ghi)), DBL_MIN)));
-    for (int j = lane; j < n; j += 32) {
-        sa[j] *= s2;
-        sb[j] *= s2;
-        sb2[j + 1] *= s2 * s2;
-        sa32[j] = (float)sa[j];
-        sb2_32[j + 1] = (float)sb2[j + 1];
-    }
-    __syncwarp();
-    glo *= s2;
-    ghi *= s2;
-    bmax *= s2 * s2;
-    const double span = fmax(fmax(fabs(glo), fabs(ghi)), DBL_MIN);
-    glo -= 4.0 * DBL_EPSILON * span + DBL_MIN;
-    ghi += 4.0 * DBL_EPSILON * span + DBL_MIN;
-    const double pivmin = DBL_MIN * fmax(1.0, bmax);
-    // 1. eigenvalues, ascending: theta_j is the j-th smallest.  Lane l owns
-    //    j = l + 32 r, r < R (the last lanes carry a dummy root when n < 32 R,
-    //    so the warp stays converged).
-    constexpr int R = MAXM / 32;
-    double lo[R], hi[R];
-    int clo[R], chi[R];  // Sturm counts at lo and hi
-    {
-        // (a) FP32 bisection narrows each bracket to a few ulps of FP32
-        const float pivmin32 = FLT_MIN * fmaxf(1.f, (float)bmax);
-        const float glo32 = (float)glo, ghi32 = (float)ghi;
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            const int j = lane + 32 * r;
-            float l32 = glo32, h32 = ghi32;
-            if (j < n)
-                for (int it = 0; it < 26; it++) {
-                    const float z = 0.5f * (l32 + h32);
-                    if (sturm_count_f32(sa32, sb2_32, n, z, pivmin32) > j) h32 = z;
-                    else l32 = z;
-                }
-            const double w = 4e-6 * span + 8.0 * (double)FLT_EPSILON * fabs((double)h32);
-            lo[r] = fmax(glo, (double)l32 - w);
-            hi[r] = fmin(ghi, (double)h32 + w);
-        }
-        // (b) FP64 check of the brackets: count(lo) <= j < count(hi)
-        double zc[2 * R];
-        int cc[2 * R];
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            zc[2 * r] = lo[r];
-            zc[2 * r + 1] = hi[r];
-        }
-        sturm_counts<2 * R>(sa, sb2, n, zc, cc);
-        bool widened = false;
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            const int j = lane + 32 * r;
-            clo[r] = cc[2 * r];
-            chi[r] = cc[2 * r + 1];
-            if (j < n && !(clo[r] <= j && chi[r] > j)) {
-                lo[r] = glo;
-                hi[r] = ghi;
-                clo[r] = 0;
-                chi[r] = n;
-                widened = true;
+    if (warp == 0) {
+        // leading unreduced block: n = 1 + first j with beta_j == 0
+        int n = m;
+        for (int j0 = 0; j0 < m - 1; j0 += 32) {
+            const int j = j0 + lane;
+            const bool zero = j < m - 1 && beta[(size_t)j * ld + c] == 0.0;
+            const unsigned zb = __ballot_sync(0xffffffffu, zero);
+            if (zb) {
+                n = j0 + __ffs(zb);
+                break;
             }
         }
-        // (c) FP64 quadrisection (three interior points per root and pass)
-        //     down to ~3e-8 span: 4 passes from the FP32 bracket, 13 from the
-        //     Gershgorin interval
-        const int passes = __any_sync(0xffffffffu, widened) ? 13 : 4;
+        bool finite = true;
+        double glo = INFINITY, ghi = -INFINITY, bmax = 0.0;
+        for (int j = lane; j < n; j += 32) {
+            const double aj = alpha[(size_t)j * ld + c];
+            const double bj = (j + 1 < n) ? beta[(size_t)j * ld + c] : 0.0;
+            const double bp = (j > 0) ? beta[(size_t)(j - 1) * ld + c] : 0.0;
+            sa[j] = aj;
+            sb[j] = bj;
+            const double bj2 = bj * bj;
+            sb2[j + 1] = bj2;
+            finite = finite && isfinite(aj) && isfinite(bj);
+            const double r = fabs(bj) + fabs(bp);
+            glo = fmin(glo, aj - r);
+            ghi = fmax(ghi, aj + r);
+            bmax = fmax(bmax, bj2);
+        }
+        if (lane == 0) {
+            sb2[0] = 0.0;
+            sb2_32[0] = 0.f;
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, off));
+            ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, off));
+            bmax = fmax(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
+        }
+        finite = __all_sync(0xffffffffu, finite);
+        __syncwarp();
+        // scale the block by the power of two s2 that brings its Gershgorin
+        // radius to [1, 2) (exact: eigenvalues scale by s2, weights do not), so
+        // the unnormalised Sturm recurrences stay far from overflow
+        const double s2 = pow2_rescale(absbits(fmax(fmax(fabs(glo), fabs(ghi)), DBL_MIN)));
+        for (int j = lane; j < n; j += 32) {
+            sa[j] *= s2;
+            sb[j] *= s2;
+            sb2[j + 1] *= s2 * s2;
+            sa32[j] = (float)sa[j];
+            sb2_32[j + 1] = (float)sb2[j + 1];
+        }
+        if (lane == 0) {
+            glo *= s2;
+            ghi *= s2;
+            bmax *= s2 * s2;
+            const double span = fmax(fmax(fabs(glo), fabs(ghi)), DBL_MIN);
+            S.n = n;
+            S.finite = finite;
+            S.span = span;
+            S.s2 = s2;
+            S.glo = glo - (4.0 * DBL_EPSILON * span + DBL_MIN);
+            S.ghi = ghi + (4.0 * DBL_EPSILON * span + DBL_MIN);
+            S.pivmin = DBL_MIN * fmax(1.0, bmax);
+            S.pivmin32 = FLT_MIN * fmaxf(1.f, (float)bmax);
+        }
+    }
+    __syncthreads();
+    if (!S.finite) return false;
+    const int n = S.n;
+    const double span = S.span, glo = S.glo, ghi = S.ghi;
+    // 1. eigenvalues, ascending: theta_j is the j-th smallest; four lanes
+    //    search for it, each with one trial point per pass.  Warps without an
+    //    eigenvalue skip the arithmetic.
+    const int j = tid >> 2, q = tid & 3;
+    const bool busy = warp * 8 < n, live = j < n;
+    double lo = glo, hi = ghi;
+    int clo = 0, chi = n;
+    bool widened = false;
+    if (busy) {
+        // (a) FP32 search (factor 5 per pass) down to ~1e-6 of the span
+        const float pivmin32 = S.pivmin32;
+        float l32 = (float)glo, h32 = (float)ghi;
+        for (int it = 0; it < 9; it++) {
+            const float w = h32 - l32;
+            const float z = l32 + 0.2f * (float)(q + 1) * w;
+            const bool gt = sturm_count_f32(sa32, sb2_32, n, z, pivmin32) > j;
+            const unsigned above = (__ballot_sync(0xffffffffu, gt) >> (lane & 28)) & 15u;
+            const int i = above ? __ffs(above) - 1 : 4;
+            if (i < 4) h32 = l32 + 0.2f * (float)(i + 1) * w;
+            if (i > 0) l32 = l32 + 0.2f * (float)i * w;
+        }
+        const double wd = 4e-6 * span + 8.0 * (double)FLT_EPSILON * fabs((double)h32);
+        lo = fmax(glo, (double)l32 - wd);
+        hi = fmin(ghi, (double)h32 + wd);
+        // (b) FP64 counts at the ends and two interior points: the bracket is
+        //     trusted only if count(lo) <= j < count(hi)
+        double zc[1] = {q == 3 ? hi : fma((double)q * (1.0 / 3.0), hi - lo, lo)};
+        int cn[1];
+        sturm_counts<1>(sa, sb2, n, zc, cn);
+        const int c_lo = __shfl_sync(0xffffffffu, cn[0], lane & 28);
+        const int c_hi = __shfl_sync(0xffffffffu, cn[0], (lane & 28) + 3);
+        clo = c_lo;
+        chi = c_hi;
+        quad_choose(j, lane, zc[0], cn[0], lo, hi, clo, chi);
+        if (live && !(c_lo <= j && c_hi > j)) {
+            lo = glo;
+            hi = ghi;
+            clo = 0;
+            chi = n;
+            widened = true;
+        }
+    }
+    // (c) FP64 search (factor 5 per pass) while some bracket holds more than
+    //     one eigenvalue: 4 passes from the FP32 bracket (below 1e-8 span),
+    //     13 from the Gershgorin interval.  Isolated brackets go straight to
+    //     Newton's iteration.
+    const int any = __syncthreads_or((live && chi - clo != 1 ? 1 : 0) | (widened ? 2 : 0));
+    const int wide = __syncthreads_or(widened ? 1 : 0);
+    if (any && busy) {
+        const int passes = wide ? 13 : 4;
         for (int it = 0; it < passes; it++) {
-            double zq[3 * R];
-            int cq[3 * R];
-#pragma unroll
-            for (int r = 0; r < R; r++) {
-                const double w = hi[r] - lo[r];
-#pragma unroll
-                for (int q = 0; q < 3; q++) zq[3 * r + q] = lo[r] + 0.25 * (q + 1) * w;
-            }
-            sturm_counts<3 * R>(sa, sb2, n, zq, cq);
-#pragma unroll
-            for (int r = 0; r < R; r++) {
-                const int j = lane + 32 * r;
-                const double z1 = zq[3 * r], z2 = zq[3 * r + 1], z3 = zq[3 * r + 2];
-                if (cq[3 * r] > j) {
-                    hi[r] = z1;
-                    chi[r] = cq[3 * r];
-                } else if (cq[3 * r + 1] > j) {
-                    lo[r] = z1;
-                    clo[r] = cq[3 * r];
-                    hi[r] = z2;
-                    chi[r] = cq[3 * r + 1];
-                } else if (cq[3 * r + 2] > j) {
-                    lo[r] = z2;
-                    clo[r] = cq[3 * r + 1];
-                    hi[r] = z3;
-                    chi[r] = cq[3 * r + 2];
-                } else {
-                    lo[r] = z3;
-                    clo[r] = cq[3 * r + 2];
-                }
-            }
-        }
-        // (d) safeguarded Newton on p_n (each step also counts, so the bracket
-        //     keeps shrinking): a root alone in its bracket converges
-        //     quadratically; roots sharing a bracket (tight clusters) keep
-        //     the bracket midpoint and are handled as a cluster below
-        double zn[R];
-#pragma unroll
-        for (int r = 0; r < R; r++) zn[r] = 0.5 * (lo[r] + hi[r]);
-        for (int it = 0; it < 4; it++) {
-            double ratio[R];
-            int cn[R];
-            newton_counts<R>(sa, sb2, n, zn, ratio, cn);
-#pragma unroll
-            for (int r = 0; r < R; r++) {
-                const int j = lane + 32 * r;
-                if (cn[r] > j) {
-                    hi[r] = zn[r];
-                    chi[r] = cn[r];
-                } else {
-                    lo[r] = zn[r];
-                    clo[r] = cn[r];
-                }
-                const double zt = zn[r] - ratio[r];
-                const bool alone = (chi[r] - clo[r]) == 1;
-                zn[r] = (alone && zt >= lo[r] && zt <= hi[r]) ? zt : 0.5 * (lo[r] + hi[r]);  // converged: stays
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            const int j = lane + 32 * r;
-            if (j < n) {
-                sth[j] = zn[r];
-                sbw[j] = hi[r] - lo[r];
-            }
+            double zq[1] = {fma(0.2 * (q + 1), hi - lo, lo)};
+            int cq[1];
+            sturm_counts<1>(sa, sb2, n, zq, cq);
+            quad_choose(j, lane, zq[0], cq[0], lo, hi, clo, chi);
         }
     }
-    __syncwarp();
-    // 2. groups of eigenvalues (lane 0, one pass with merging): a group grows
-    //    while the next gap is below kClusterGap * span or below 16 x its
-    //    half-width, and absorbs the previous group while the gap to it is
-    //    below 17 x its half-width; one-member groups are isolated
-    //    eigenvalues, the others clusters.  A cluster closer than 16 x its
-    //    half-width to a neighbouring group sends the column to the
-    //    sequential QR.
+    if (live && q == 0) {
+        S.c0[j] = lo;
+        S.c1[j] = hi;
+        S.clo[j] = clo;
+        S.chi[j] = chi;
+    }
+    __syncthreads();
+    // (d) safeguarded Newton on p_n, one lane per eigenvalue (each step also
+    //     counts, so the bracket keeps shrinking): a root alone in its bracket
+    //     converges quadratically and stops; roots sharing a bracket (tight
+    //     clusters) halve it four times and are handled as a cluster below
+    if (warp * 32 < n) {
+        const int jr = min(tid, n - 1);
+        double l = S.c0[jr], h = S.c1[jr];
+        int cl = S.clo[jr], ch = S.chi[jr];
+        double zn[1] = {0.5 * (l + h)};
+        double w = 0.0;
+        bool done = false;
+        for (int it = 0; it < 48; it++) {
+            double ratio[1];
+            int cn[1];
+            newton_counts<1>(sa, sb2, n, zn, ratio, cn);
+            if (!done) {
+                if (cn[0] > jr) {
+                    h = zn[0];
+                    ch = cn[0];
+                } else {
+                    l = zn[0];
+                    cl = cn[0];
+                }
+                const double zt = zn[0] - ratio[0];
+                const bool alone = (ch - cl) == 1, inside = zt >= l && zt <= h;
+                w = h - l;
+                if (alone && inside) {
+                    zn[0] = zt;
+                    // the step left an error of ratio^2 / gap, gap >= kClusterGap span
+                    if (fabs(ratio[0]) <= 1e-11 * span) {
+                        w = 8.0 * DBL_EPSILON * span;
+                        done = true;
+                    }
+                } else {
+                    zn[0] = 0.5 * (l + h);
+                    if (!alone && it >= 3) done = true;
+                    if (w <= 4.0 * DBL_EPSILON * span) done = true;
+                }
+            }
+            if (__all_sync(0xffffffffu, done)) break;
+        }
+        if (tid < n) {
+            sth[jr] = zn[0];
+            sbw[jr] = w;
+        }
+    }
+    __syncthreads();
+    // 2. groups of eigenvalues: a group grows while the next gap is below
+    //    kClusterGap * span or below 16 x its half-width, and absorbs the
+    //    previous group while the gap to it is below 17 x its half-width;
+    //    one-member groups are isolated eigenvalues, the others clusters.  A
+    //    cluster closer than 16 x its half-width to a neighbouring group sends
+    //    the column to the sequential QR.  When no gap is that small (the
+    //    usual case, tested by all threads at once) every group has one member.
     const double tau = kClusterGap * span;
     double* s_cc = S.cc;
     double* s_rho = S.rho;
@@ -615,15 +632,32 @@ __device__ bool tq_spectrum(const double* __restrict__ alpha, const double* __re
     int* s_gfirst = S.gfirst;
     int* s_glast = S.glast;
     int* s_cl_of_group = S.cl_of_group;
-    if (lane == 0) {
+    bool close = false;
+    if (tid + 1 < n) {
+        const double gap = sth[tid + 1] - sth[tid];
+        close = gap < tau || gap < 8.0 * sbw[tid];
+    }
+    if (!__syncthreads_or(close)) {
+        for (int g = tid; g < n; g += NT) {
+            s_gfirst[g] = g;
+            s_glast[g] = g;
+            s_cl_of_group[g] = -1;
+        }
+        if (tid == 0) {
+            s_gfirst[n] = n;
+            S.ngroups = n;
+            S.ncl = 0;
+            S.fallback = 0;
+        }
+    } else if (tid == 0) {
         auto halfw = [&](int f, int l) {
             double h = 0.5 * (sth[l] - sth[f]);
-            for (int q = f; q <= l; q++) h = fmax(h, 0.5 * sbw[q]);
+            for (int i = f; i <= l; i++) h = fmax(h, 0.5 * sbw[i]);
             return h;
         };
         int ng = 0;
-        for (int j = 0; j < n;) {
-            int f = j, e = j;
+        for (int i = 0; i < n;) {
+            int f = i, e = i;
             for (;;) {
                 while (e + 1 < n) {
                     const double gap = sth[e + 1] - sth[e];
@@ -639,7 +673,7 @@ __device__ bool tq_spectrum(const double* __restrict__ alpha, const double* __re
             s_gfirst[ng] = f;
             s_glast[ng] = e;
             ng++;
-            j = e + 1;
+            i = e + 1;
         }
         int ncl = 0, fb = 0;
         for (int g = 0; g < ng; g++) {
@@ -662,114 +696,182 @@ __device__ bool tq_spectrum(const double* __restrict__ alpha, const double* __re
         S.ngroups = ng;
         S.ncl = ncl;
         S.fallback = fb;
-        S.n = n;
-        S.span = span;
-        S.s2 = s2;
-        S.pivmin = pivmin;
     }
-    __syncwarp();
+    __syncthreads();
     return true;
 }
 
+// Twisted-factorisation eigenvectors of the eigenvalues [rb0, rb0 + nb), nb <=
+// RB: squared norm, first and last component (the entry at the twist index is
+// 1) to S.nrm, S.z1, S.zn.  Two lanes per eigenvalue: lane 0 of the pair runs
+// the top-down pivots D_k and the components above the twist, lane 1 the
+// bottom-up pivots R_k and those below; both keep reciprocals in P ([2][MAXM]
+// [LD]), which the components need (one reciprocal per pivot, no division).
+// With KEEP the components replace the first half of P.  Every thread of the
+// CTA calls it.
+template <int MAXM, bool KEEP>
+__device__ void tq_vectors(TqShared<MAXM>& S, double* P, int rb0, int nb) {
+    constexpr int LD = TqCfg<MAXM>::LD;
+    const int tid = threadIdx.x;
+    const int r = tid >> 1, side = tid & 1, n = S.n;
+    if ((tid >> 5) * 16 < nb) {  // warp-uniform
+        const bool live = r < nb;
+        const int rr = live ? r : nb - 1;
+        const double th = S.th[rb0 + rr], pivmin = S.pivmin;
+        const double *sa = S.a, *sb = S.b, *sb2 = S.b2;
+        double* P0 = P + rr;
+        double* P1 = P + MAXM * LD + rr;
+        double* mine = side ? P1 : P0;
+        double inv = 0.0;
+        for (int i = 0; i < n; i++) {
+            const int k = side ? n - 1 - i : i;
+            const double d = guard_pivot(fma(-sb2[side ? k + 1 : k], inv, sa[k] - th), pivmin);
+            inv = 1.0 / d;
+            if (live) mine[k * LD] = inv;
+        }
+        __syncwarp();
+        // twist index: smallest |gamma_k| = |D_k + R_k - (a_k - theta)|
+        long long best = 0x7ff0000000000000LL;
+        int tw = n - 1;
+        for (int k = n - 1 - side; k >= 0; k -= 2) {
+            const double up = k > 0 ? P0[(k - 1) * LD] : 0.0, dn = k + 1 < n ? P1[(k + 1) * LD] : 0.0;
+            const long long g = absbits(fma(-sb2[k + 1], dn, fma(-sb2[k], up, sa[k] - th)));
+            if (g < best) {
+                best = g;
+                tw = k;
+            }
+        }
+        const long long ob = __shfl_xor_sync(0xffffffffu, best, 1);
+        const int ot = __shfl_xor_sync(0xffffffffu, tw, 1);
+        if (ob < best || (ob == best && ot > tw)) tw = ot;
+        __syncwarp();  // both lanes have read the reciprocals that KEEP overwrites
+        // components away from the twist
+        double z = 1.0, s = 0.0;
+        const int steps = side ? n - 1 - tw : tw;
+        for (int i = 1; i <= steps; i++) {
+            const int k = side ? tw + i : tw - i;
+            z = -(sb[side ? k - 1 : k] * z) * mine[k * LD];
+            s = fma(z, z, s);
+            if (KEEP && live) P0[k * LD] = z;
+        }
+        if (KEEP && live && side == 0) P0[tw * LD] = 1.0;
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        if (live) {
+            if (side == 0) {
+                S.nrm[rb0 + r] = 1.0 + s;
+                S.z1[rb0 + r] = z;
+            } else {
+                S.zn[rb0 + r] = z;
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// The Gauss quadrature from the spectrum and the twisted eigenvectors of all
+// eigenvalues (S.nrm, S.z1): isolated eigenvalues by their weights, clusters
+// by the contour, a warp per cluster and a lane per contour point.  Every
+// thread of the CTA calls it; thread 0 writes *psi.
 template <int MAXM>
-__global__ void __launch_bounds__(32) k_tridiag_quad(const double* __restrict__ alpha, const double* __restrict__ beta,
-                                                     const double* __restrict__ norm2, const double* __restrict__ scale,
-                                                     int count, int m_all, int ld, double* __restrict__ psi,
-                                                     const int32_t* __restrict__ cols,
-                                                     const int32_t* __restrict__ mcol) {
+__device__ void tq_quadrature(TqShared<MAXM>& S, double sc, double norm2, double* psi) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = S.n;
+    for (int g = tid; g < S.ngroups; g += blockDim.x) {
+        if (S.cl_of_group[g] >= 0) {
+            S.c0[g] = S.c1[g] = 0.0;
+            continue;
+        }
+        const int i = S.gfirst[g];
+        const double w = S.z1[i] * S.z1[i] / S.nrm[i];
+        S.c0[g] = w * f_entropy(sc * S.th[i]);
+        S.c1[g] = w;
+    }
+    for (int cl = warp; cl < S.ncl; cl += TqCfg<MAXM>::NW) {
+        double W, M1, M2;
+        resolvent_point(S.a, S.b, n, S.cc[cl], S.rho[cl], lane, W, M1, M2);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            W += __shfl_xor_sync(0xffffffffu, W, off);
+            M1 += __shfl_xor_sync(0xffffffffu, M1, off);
+            M2 += __shfl_xor_sync(0xffffffffu, M2, off);
+        }
+        if (lane == 0) {
+            W /= kContourPoints;
+            M1 /= kContourPoints;
+            M2 /= kContourPoints;
+            // sum_j w_j f(theta_j) over the cluster ~ W f(tbar) + f''(tbar) W var / 2
+            // with the weighted mean tbar and variance var; a cluster whose weight
+            // is at rounding level (eigenvectors that vanish at row 1) keeps its
+            // centre and no correction
+            const double cc = S.cc[cl], half = S.half[cl];
+            double contrib = W * f_entropy(sc * cc), errb = 0.0;
+            if (W > 0.0 && fabs(M1) <= 2.0 * half * W) {
+                const double mu = M1 / W, tbar = cc + mu;
+                const double var = fmax(M2 / W - mu * mu, 0.0);
+                contrib = W * f_entropy(sc * tbar);
+                if (tbar > 0.0) contrib -= 0.5 * (sc / tbar) * W * var;  // d2/dt2 f(sc t) = -sc / t
+            }
+            if (half > 1e-3 * fabs(cc)) {
+                // a cluster at the origin: the expansion does not hold, but its
+                // members lie in [cc - half, cc + half] and f >= 0 increases from
+                // 0, so the error is below W f(cc + half)
+                errb = fmax(W, 0.0) * f_entropy(fmin(sc * fmax(cc + half, 0.0), 0.36787944117144233));
+            }
+            S.k0[cl] = contrib;
+            S.k1[cl] = W;
+            S.k2[cl] = errb;
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        double acc = 0.0, wsum = 0.0, errb = 0.0;
+        for (int g = lane; g < S.ngroups; g += 32) {
+            acc += S.c0[g];
+            wsum += S.c1[g];
+        }
+        for (int cl = lane; cl < S.ncl; cl += 32) {
+            acc += S.k0[cl];
+            wsum += S.k1[cl];
+            errb += S.k2[cl];
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            wsum += __shfl_xor_sync(0xffffffffu, wsum, off);
+            if (S.ncl) errb += __shfl_xor_sync(0xffffffffu, errb, off);
+        }
+        if (!(errb <= 1e-10 * fabs(acc))) {
+            quad_by_qr<MAXM>(S.a, S.b, n, sc, norm2, lane, psi);
+        } else if (lane == 0) {
+            // the weights sum to one; dividing by the computed sum removes their
+            // common rounding
+            *psi = norm2 * (acc / wsum);
+        }
+    }
+}
+
+template <int MAXM>
+__global__ void __launch_bounds__(TqCfg<MAXM>::NT)
+    k_tridiag_quad(const double* __restrict__ alpha, const double* __restrict__ beta,
+                   const double* __restrict__ norm2, const double* __restrict__ scale, int count, int m_all, int ld,
+                   double* __restrict__ psi, const int32_t* __restrict__ cols, const int32_t* __restrict__ mcol) {
     __shared__ TqShared<MAXM> S;
-    extern __shared__ double piv[];  // [2][MAXM][32]: twisted pivots, transposed per lane
-    const int lane = threadIdx.x;
+    extern __shared__ double piv[];  // pivot scratch of tq_vectors
     if ((int)blockIdx.x >= count) return;
     // entry blockIdx.x: column c (of the ld-strided arrays) after m steps
     const int c = cols ? cols[blockIdx.x] : (int)blockIdx.x;
     const int m = mcol ? mcol[blockIdx.x] : m_all;
-    if (!tq_spectrum<MAXM>(alpha, beta, c, m, ld, lane, S)) {
-        if (lane == 0) psi[c] = nan("");
+    if (!tq_spectrum<MAXM>(alpha, beta, c, m, ld, S)) {
+        if (threadIdx.x == 0) psi[c] = nan("");
         return;
     }
-    const int n = S.n;
-    const double span = S.span, pivmin = S.pivmin;
-    const double* sa = S.a;
-    const double* sb = S.b;
-    const double* sth = S.th;
-    const double* s_cc = S.cc;
-    const double* s_rho = S.rho;
-    const double* s_half = S.half;
-    const int* s_gfirst = S.gfirst;
-    const int* s_cl_of_group = S.cl_of_group;
     const double sc = scale[c] / S.s2;  // f is applied to the unscaled eigenvalues
-    const int ngroups = S.ngroups, ncl = S.ncl;
     if (S.fallback) {
-        quad_by_qr<MAXM>(sa, sb, n, sc, norm2[c], lane, psi + c);
+        if (threadIdx.x < 32) quad_by_qr<MAXM>(S.a, S.b, S.n, sc, norm2[c], threadIdx.x, psi + c);
         return;
     }
-    // 3. isolated eigenvalues: twisted-factorisation weights, groups spread
-    //    over the lanes
-    double acc = 0.0, wsum = 0.0, errb = 0.0;
-    for (int g = lane; g < ngroups; g += 32) {
-        if (s_cl_of_group[g] >= 0) continue;
-        const int j = s_gfirst[g];
-        const double w = twisted_weight(sa, sb, n, sth[j], pivmin, piv + lane, piv + MAXM * 32 + lane);
-        acc += w * f_entropy(sc * sth[j]);
-        wsum += w;
-    }
-    // 4. clusters: the K contour points of all clusters spread over the lanes
-    //    (their values reuse the pivot scratch), then lane (cluster mod 32)
-    //    sums each cluster's points in order
-    __syncwarp();
-    double* pts = piv;  // [cluster][K][3]
-    for (int item = lane; item < ncl * kContourPoints; item += 32) {
-        const int cl = item / kContourPoints, q = item % kContourPoints;
-        resolvent_point(sa, sb, n, s_cc[cl], s_rho[cl], q, pts[3 * item], pts[3 * item + 1], pts[3 * item + 2]);
-    }
-    __syncwarp();
-    for (int cl = lane; cl < ncl; cl += 32) {
-        double W = 0.0, M1 = 0.0, M2 = 0.0;
-        for (int q = 0; q < kContourPoints; q++) {
-            W += pts[3 * (cl * kContourPoints + q)];
-            M1 += pts[3 * (cl * kContourPoints + q) + 1];
-            M2 += pts[3 * (cl * kContourPoints + q) + 2];
-        }
-        W /= kContourPoints;
-        M1 /= kContourPoints;
-        M2 /= kContourPoints;
-        // sum_j w_j f(theta_j) over the cluster ~ W f(tbar) + f''(tbar) W var / 2
-        // with the weighted mean tbar and variance var; a cluster whose weight
-        // is at rounding level (eigenvectors that vanish at row 1) keeps its
-        // centre and no correction
-        const double cc = s_cc[cl], half = s_half[cl];
-        double contrib = W * f_entropy(sc * cc);
-        if (W > 0.0 && fabs(M1) <= 2.0 * half * W) {
-            const double mu = M1 / W, tbar = cc + mu;
-            const double var = fmax(M2 / W - mu * mu, 0.0);
-            contrib = W * f_entropy(sc * tbar);
-            if (tbar > 0.0) contrib -= 0.5 * (sc / tbar) * W * var;  // d2/dt2 f(sc t) = -sc / t
-        }
-        if (half > 1e-3 * fabs(cc)) {
-            // a cluster at the origin: the expansion does not hold, but its
-            // members lie in [cc - half, cc + half] and f >= 0 increases from
-            // 0, so the error is below W f(cc + half)
-            errb += fmax(W, 0.0) * f_entropy(fmin(sc * fmax(cc + half, 0.0), 0.36787944117144233));
-        }
-        acc += contrib;
-        wsum += W;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        wsum += __shfl_xor_sync(0xffffffffu, wsum, off);
-        errb += __shfl_xor_sync(0xffffffffu, errb, off);
-    }
-    if (!(errb <= 1e-10 * fabs(acc))) {
-        if (lane == 0) S.fallback = 1;
-    } else if (lane == 0) {
-        // the weights sum to one; dividing by the computed sum removes their
-        // common rounding
-        psi[c] = norm2[c] * (acc / wsum);
-    }
-    __syncwarp();
-    if (S.fallback) quad_by_qr<MAXM>(sa, sb, n, sc, norm2[c], lane, psi + c);
+    for (int rb = 0; rb < S.n; rb += TqCfg<MAXM>::RB)
+        tq_vectors<MAXM, false>(S, piv, rb, min(TqCfg<MAXM>::RB, S.n - rb));
+    tq_quadrature<MAXM>(S, sc, norm2[c], psi + c);
 }
 
 // f(T) e1 by the sequential implicit QR with the full eigenvector matrix Z
@@ -809,142 +911,115 @@ __device__ void fvec_by_qr(const double* sa, const double* sb, int n, int m, dou
 // with the spectrum of k_tridiag_quad: an isolated eigenvalue adds its
 // twisted-factorisation eigenvector z scaled by z_1 f / ||z||^2; a cluster
 // adds (1/2 pi i) \oint (f(c) + f'(c)(z - c) + f''(c)(z - c)^2 / 2)
-// (z I - T)^{-1} e1 dz by the 32-point trapezoid rule (one point per lane;
-// the resolvent vector from the bottom-up continued fraction, then the
-// forward ratios x_k = x_{k-1} beta_{k-1} / g_k).  Each lane accumulates its
-// own column of a [n][32] buffer, summed in lane order at the end.
+// (z I - T)^{-1} e1 dz by the 32-point trapezoid rule (one point per lane of
+// warp 0; the resolvent vector from the bottom-up continued fraction, then the
+// forward ratios x_k = x_{k-1} beta_{k-1} / g_k).  Component k is summed by
+// four lanes over the eigenvectors of a pass (or the contour points).
 template <int MAXM>
-__global__ void __launch_bounds__(32) k_tridiag_fvec(const double* __restrict__ alpha,
-                                                     const double* __restrict__ beta,
-                                                     const double* __restrict__ scale, int count, int m, int ld,
-                                                     double* __restrict__ zvec) {
+__global__ void __launch_bounds__(TqCfg<MAXM>::NT)
+    k_tridiag_fvec(const double* __restrict__ alpha, const double* __restrict__ beta,
+                   const double* __restrict__ scale, int count, int m, int ld, double* __restrict__ zvec) {
+    constexpr int LD = TqCfg<MAXM>::LD, RB = TqCfg<MAXM>::RB;
     __shared__ TqShared<MAXM> S;
-    extern __shared__ double piv[];  // [2][MAXM][32] pivots / resolvent, [MAXM][32] partial sums
-    const int c = blockIdx.x, lane = threadIdx.x;
+    __shared__ double s_y0, s_err;
+    extern __shared__ double piv[];  // pivot scratch of tq_vectors / resolvent, Z of the QR fallback
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (c >= count) return;
-    if (!tq_spectrum<MAXM>(alpha, beta, c, m, ld, lane, S)) {
-        for (int row = lane; row < m; row += 32) zvec[(size_t)row * ld + c] = nan("");
+    if (!tq_spectrum<MAXM>(alpha, beta, c, m, ld, S)) {
+        for (int row = tid; row < m; row += blockDim.x) zvec[(size_t)row * ld + c] = nan("");
         return;
     }
     const int n = S.n;
-    const double span = S.span, pivmin = S.pivmin;
-    const double* sa = S.a;
-    const double* sb = S.b;
-    const double* sth = S.th;
     const double sc = scale[c] / S.s2;  // f is applied to the unscaled eigenvalues
     if (S.fallback) {
-        fvec_by_qr<MAXM>(sa, sb, n, m, sc, lane, piv, zvec, ld, c);
+        if (warp == 0) fvec_by_qr<MAXM>(S.a, S.b, n, m, sc, lane, piv, zvec, ld, c);
         return;
     }
-    double* Dp = piv + lane;                // this lane's pivots / real parts
-    double* Rp = piv + MAXM * 32 + lane;    // this lane's pivots / imaginary parts
-    double* ys = piv + 2 * MAXM * 32 + lane;  // this lane's partial sum of y
-    for (int k = 0; k < n; k++) ys[k * 32] = 0.0;
-    // isolated eigenvalues
-    for (int g = lane; g < S.ngroups; g += 32) {
-        if (S.cl_of_group[g] >= 0) continue;
-        const double th = sth[S.gfirst[g]];
-        double d = 0.0;
-        for (int k = 0; k < n; k++) {
-            d = guard_pivot((sa[k] - th) - (k > 0 ? sb[k - 1] * sb[k - 1] / d : 0.0), pivmin);
-            Dp[k * 32] = d;
+    // S.bw is free after the grouping: 1 marks an isolated eigenvalue
+    for (int i = tid; i < n; i += blockDim.x) S.bw[i] = 0.0;
+    if (tid == 0) s_err = 0.0;
+    __syncthreads();
+    for (int g = tid; g < S.ngroups; g += blockDim.x)
+        if (S.cl_of_group[g] < 0) S.bw[S.gfirst[g]] = 1.0;
+    __syncthreads();
+    const int yk = tid >> 2, part = tid & 3;  // component of y, lane of its quad
+    double y = 0.0;
+    for (int rb = 0; rb < n; rb += RB) {
+        const int nb = min(RB, n - rb);
+        tq_vectors<MAXM, true>(S, piv, rb, nb);
+        if (tid < nb) {
+            const int i = rb + tid;
+            S.c0[tid] = S.bw[i] != 0.0 ? S.z1[i] * f_entropy(sc * S.th[i]) / S.nrm[i] : 0.0;
         }
-        double r = 0.0, best = INFINITY;
-        int tw = n - 1;
-        for (int k = n - 1; k >= 0; k--) {
-            r = guard_pivot((sa[k] - th) - (k + 1 < n ? sb[k] * sb[k] / r : 0.0), pivmin);
-            Rp[k * 32] = r;
-            const double gam = fabs(Dp[k * 32] + r - (sa[k] - th));
-            if (gam < best) {
-                best = gam;
-                tw = k;
-            }
-        }
-        // eigenvector components overwrite the pivots they were made from
-        double nrm = 1.0, z = 1.0;
-        for (int k = tw - 1; k >= 0; k--) {
-            z = -sb[k] * z / Dp[k * 32];
-            Dp[k * 32] = z;
-            nrm = fma(z, z, nrm);
-        }
-        const double z1 = tw > 0 ? z : 1.0;
-        z = 1.0;
-        for (int k = tw + 1; k < n; k++) {
-            z = -sb[k - 1] * z / Rp[k * 32];
-            Rp[k * 32] = z;
-            nrm = fma(z, z, nrm);
-        }
-        const double coef = z1 * f_entropy(sc * th) / nrm;
-        for (int k = 0; k < n; k++) {
-            const double zk = k < tw ? Dp[k * 32] : (k == tw ? 1.0 : Rp[k * 32]);
-            ys[k * 32] += coef * zk;
-        }
+        __syncthreads();
+        if (yk < n)
+            for (int r = part; r < nb; r += 4) y += S.c0[r] * piv[yk * LD + r];
+        __syncthreads();
     }
-    // clusters: one round per cluster, contour point q on lane q
-    double errb = 0.0;
+    // clusters: one round per cluster, contour point q on lane q of warp 0
+    double* Dp = piv + lane;              // real parts of the resolvent recurrences, [k][LD]
+    double* Rp = piv + MAXM * LD + lane;  // imaginary parts
     for (int cl = 0; cl < S.ncl; cl++) {
-        const double cc = S.cc[cl], rho = S.rho[cl], half = S.half[cl];
-        double sph, cph;
-        sincospi((2.0 * lane + 1.0) / kContourPoints, &sph, &cph);
-        const double dzr = rho * cph, dzi = rho * sph;
-        const double zr = cc + dzr, zi = dzi;
-        // bottom-up continued fraction g_k, stored
-        double gr = zr - sa[n - 1], gi = zi;
-        Dp[(n - 1) * 32] = gr;
-        Rp[(n - 1) * 32] = gi;
-        for (int k = n - 2; k >= 0; k--) {
-            const double t = sb[k] * sb[k] / (gr * gr + gi * gi);
-            gr = (zr - sa[k]) - t * gr;
-            gi = zi + t * gi;
-            Dp[k * 32] = gr;
-            Rp[k * 32] = gi;
-        }
-        // Taylor weight h = dz (f0 + f1 dz + f2 dz^2 / 2) of the cluster centre
-        const double x0 = sc * cc;
-        const double f0 = f_entropy(x0);
-        const double f1 = x0 > 0.0 ? sc * (-log(x0) - 1.0) : 0.0;
-        const double f2 = cc > 0.0 ? -sc / cc : 0.0;
-        const double d2r = dzr * dzr - dzi * dzi, d2i = 2.0 * dzr * dzi;
-        const double pr = f0 + f1 * dzr + 0.5 * f2 * d2r, pi = f1 * dzi + 0.5 * f2 * d2i;
-        const double hr = (dzr * pr - dzi * pi) / kContourPoints, hi = (dzr * pi + dzi * pr) / kContourPoints;
-        // forward ratios: x_0 = 1 / g_0, x_k = x_{k-1} beta_{k-1} / g_k
-        double xr, xi;
-        {
-            const double den = gr * gr + gi * gi;
-            xr = gr / den;
-            xi = -gi / den;
-        }
-        double wq = (xr * dzr - xi * dzi) / kContourPoints;  // Re x_0 dz / K
-        ys[0] += xr * hr - xi * hi;
-        for (int k = 1; k < n; k++) {
-            const double g_r = Dp[k * 32], g_i = Rp[k * 32];
-            const double den = g_r * g_r + g_i * g_i;
-            const double ur = sb[k - 1] * g_r / den, ui = -sb[k - 1] * g_i / den;  // beta / g
-            const double nxr = xr * ur - xi * ui, nxi = xr * ui + xi * ur;
-            xr = nxr;
-            xi = nxi;
-            ys[k * 32] += xr * hr - xi * hi;
-        }
+        if (warp == 0) {
+            const double cc = S.cc[cl], rho = S.rho[cl], half = S.half[cl];
+            double sph, cph;
+            sincospi((2.0 * lane + 1.0) / kContourPoints, &sph, &cph);
+            const double dzr = rho * cph, dzi = rho * sph;
+            const double zr = cc + dzr, zi = dzi;
+            // bottom-up continued fraction g_k, stored
+            double gr = zr - S.a[n - 1], gi = zi;
+            Dp[(n - 1) * LD] = gr;
+            Rp[(n - 1) * LD] = gi;
+            for (int k = n - 2; k >= 0; k--) {
+                const double t = S.b2[k + 1] / (gr * gr + gi * gi);
+                gr = (zr - S.a[k]) - t * gr;
+                gi = zi + t * gi;
+                Dp[k * LD] = gr;
+                Rp[k * LD] = gi;
+            }
+            // Taylor weight h = dz (f0 + f1 dz + f2 dz^2 / 2) of the cluster centre
+            const double x0 = sc * cc;
+            const double f0 = f_entropy(x0);
+            const double f1 = x0 > 0.0 ? sc * (-log(x0) - 1.0) : 0.0;
+            const double f2 = cc > 0.0 ? -sc / cc : 0.0;
+            const double d2r = dzr * dzr - dzi * dzi, d2i = 2.0 * dzr * dzi;
+            const double pr = f0 + f1 * dzr + 0.5 * f2 * d2r, pi = f1 * dzi + 0.5 * f2 * d2i;
+            const double hr = (dzr * pr - dzi * pi) / kContourPoints, hi = (dzr * pi + dzi * pr) / kContourPoints;
+            // forward ratios: x_0 = 1 / g_0, x_k = x_{k-1} beta_{k-1} / g_k;
+            // this point's share of y_k replaces the real part of g_k
+            double xr, xi;
+            {
+                const double den = gr * gr + gi * gi;
+                xr = gr / den;
+                xi = -gi / den;
+            }
+            double wq = (xr * dzr - xi * dzi) / kContourPoints;  // Re x_0 dz / K
+            Dp[0] = xr * hr - xi * hi;
+            for (int k = 1; k < n; k++) {
+                const double g_r = Dp[k * LD], g_i = Rp[k * LD];
+                const double inv = S.b[k - 1] / (g_r * g_r + g_i * g_i);
+                const double ur = g_r * inv, ui = -g_i * inv;  // beta / g
+                const double nxr = xr * ur - xi * ui, nxi = xr * ui + xi * ur;
+                xr = nxr;
+                xi = nxi;
+                Dp[k * LD] = xr * hr - xi * hi;
+            }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) wq += __shfl_xor_sync(0xffffffffu, wq, off);
-        if (half > 1e-3 * fabs(cc))  // cluster at the origin: error below W f(c + half)
-            errb += fmax(wq, 0.0) * f_entropy(fmin(sc * fmax(cc + half, 0.0), 0.36787944117144233));
+            for (int off = 16; off > 0; off >>= 1) wq += __shfl_xor_sync(0xffffffffu, wq, off);
+            if (lane == 0 && half > 1e-3 * fabs(cc))  // cluster at the origin: error below W f(c + half)
+                s_err += fmax(wq, 0.0) * f_entropy(fmin(sc * fmax(cc + half, 0.0), 0.36787944117144233));
+        }
+        __syncthreads();
+        if (yk < n)
+            for (int r = part; r < 32; r += 4) y += piv[yk * LD + r];
+        __syncthreads();
     }
-    __syncwarp();
-    // y_k = sum over lanes of the partial sums, in lane order
-    double y0 = 0.0;
-    for (int k = lane; k < m; k += 32) {
-        double y = 0.0;
-        if (k < n)
-            for (int l = 0; l < 32; l++) y += piv[2 * MAXM * 32 + k * 32 + l];
-        if (k == 0) y0 = y;
-        zvec[(size_t)k * ld + c] = y;
-    }
-    y0 = __shfl_sync(0xffffffffu, y0, 0);
-    if (!(errb <= 1e-10 * fabs(y0))) {
-        __syncwarp();
-        fvec_by_qr<MAXM>(sa, sb, n, m, sc, lane, piv, zvec, ld, c);
-    }
+    y += __shfl_xor_sync(0xffffffffu, y, 1);
+    y += __shfl_xor_sync(0xffffffffu, y, 2);
+    if (part == 0 && yk < m) zvec[(size_t)yk * ld + c] = yk < n ? y : 0.0;
+    if (tid == 0) s_y0 = y;
+    __syncthreads();
+    if (warp == 0 && !(s_err <= 1e-10 * fabs(s_y0))) fvec_by_qr<MAXM>(S.a, S.b, n, m, sc, lane, piv, zvec, ld, c);
 }
 
 // A-posteriori bounds of Theorem 4.4 for the polynomial Lanczos quadrature
@@ -962,175 +1037,191 @@ __global__ void __launch_bounds__(32) k_tridiag_fvec(const double* __restrict__ 
 // shared spectrum (for a tight cluster the individual products are as
 // ill-conditioned as the formula itself).  f(x) = -x log x; the interval must
 // be positive.
-// Divided differences of f(x) = -x log x at (t, z), z = t (1 + u), given
-// log z and log t: f[t, z] = -log t - h(u) and f[t, t, z] = (1 - h(u)) / (t u)
-// with h(u) = (1 + u) log(1 + u) / u = z (log z - log t) / (t u).  For
-// |u| < 0.1 the power series 1 - h(u) = sum_{k>=1} (-1)^k u^k / (k (k + 1))
-// avoids the cancellation of the plain quotients.
-__device__ __forceinline__ void dd_entropy(double z, double lz, double t, double lt, double& dd1, double& dd2) {
-    const double u = (z - t) / t;
-    if (fabs(u) < 0.1) {
-        // (1 - h(u)) / u by Horner, 18 terms (|u|^18 / 342 < 1e-20)
-        double ser = 0.0;
+// Divided differences of f(x) = -x log x at (t, z), z = t (1 + u):
+// f[t, z] = -log t - h and f[t, t, z] = (1 - h) / (z - t) with
+// h = z (log z - log t) / (z - t) = (1 + u) log(1 + u) / u.  For |u| < 0.1 the
+// power series 1 - h = sum_{k>=1} (-1)^k u^k / (k (k + 1)) (18 terms: |u|^18 /
+// 342 < 1e-20) avoids the cancellation of the plain quotients.
+// With a Ritz value's constants this gives its term of g_m without the part
+// -2 ab gamma log t, which does not depend on z and is summed once: one
+// reciprocal and eight multiply-adds per point (four divisions and 18 in the
+// series before; a division occupies an FP64 port for 9 slots).
+struct GTerm {
+    double t, it, lt, ab2, c1;  // theta, 1 / theta, log theta, (a b)^2, 2 a b gamma
+};
+__device__ __forceinline__ double g_term(double z, double lz, const GTerm& p, double g) {
+    const double d = z - p.t;
+    const double u = d * p.it;
+    if (fabs((float)u) < 0.1f) {
+        double ser = 0.0;  // (1 - h) / u by Horner
+#pragma unroll
         for (int k = 18; k >= 1; k--) ser = fma(ser, u, ((k & 1) ? -1.0 : 1.0) / (double)(k * (k + 1)));
-        dd1 = -lt - (1.0 - ser * u);
-        dd2 = ser / t;
-    } else {
-        const double h = (z / t) * (lz - lt) / u;
-        dd1 = -lt - h;
-        dd2 = (1.0 - h) / (t * u);
+        g = fma(p.ab2 * p.it, ser, g);
+        return fma(p.c1, fma(ser, u, -1.0), g);
     }
+    const double r = 1.0 / d;
+    const double h = (lz - p.lt) * (z * r);
+    g = fma(p.ab2 * r, 1.0 - h, g);
+    return fma(-p.c1, h, g);
 }
 
 template <int MAXM>
-__global__ void __launch_bounds__(32) k_tridiag_bounds(const double* __restrict__ alpha,
-                                                       const double* __restrict__ beta,
-                                                       const double* __restrict__ norm2,
-                                                       const double* __restrict__ scale, int count, int m_all, int ld,
-                                                       double lam_min, double lam_max, int grid,
-                                                       double* __restrict__ lower, double* __restrict__ upper,
-                                                       double* __restrict__ estimate,
-                                                       const int32_t* __restrict__ cols,
-                                                       const int32_t* __restrict__ mcol,
-                                                       const double* __restrict__ lam_max_col) {
+__global__ void __launch_bounds__(TqCfg<MAXM>::NT)
+    k_tridiag_bounds(const double* __restrict__ alpha, const double* __restrict__ beta,
+                     const double* __restrict__ norm2, const double* __restrict__ scale, int count, int m_all, int ld,
+                     double lam_min, double lam_max, int grid, double* __restrict__ lower,
+                     double* __restrict__ upper, double* __restrict__ estimate, const int32_t* __restrict__ cols,
+                     const int32_t* __restrict__ mcol, const double* __restrict__ lam_max_col,
+                     double* __restrict__ psi) {
     __shared__ TqShared<MAXM> S;
-    __shared__ double s_th[MAXM], s_ab[MAXM], s_gam[MAXM], s_lt[MAXM];
-    extern __shared__ double piv[];  // [2][MAXM][32] twisted pivots
-    const int lane = threadIdx.x;
+    __shared__ GTerm G[MAXM];
+    extern __shared__ double piv[];  // pivot scratch of tq_vectors
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if ((int)blockIdx.x >= count) return;
     // entry blockIdx.x: column c (of the ld-strided arrays) after m steps,
     // with its own upper end of the spectral interval if given
     const int c = cols ? cols[blockIdx.x] : (int)blockIdx.x;
     const int m = mcol ? mcol[blockIdx.x] : m_all;
     if (lam_max_col) lam_max = lam_max_col[blockIdx.x];
-    if (!tq_spectrum<MAXM>(alpha, beta, c, m, ld, lane, S)) {
-        if (lane == 0) lower[c] = upper[c] = estimate[c] = nan("");
+    auto put = [&](double lo, double hi, double est) {
+        if (tid == 0) {
+            lower[c] = lo;
+            upper[c] = hi;
+            estimate[c] = est;
+        }
+    };
+    if (!tq_spectrum<MAXM>(alpha, beta, c, m, ld, S)) {
+        put(nan(""), nan(""), nan(""));
+        if (psi && tid == 0) psi[c] = nan("");
         return;
     }
     const int n = S.n;
+    const double sc = scale[c] / S.s2;
     const double bm = beta[(size_t)(m - 1) * ld + c] * scale[c];  // beta_m of A
-    if (n < m || bm == 0.0) {
-        // the Krylov space is invariant: the quadrature is exact
-        if (lane == 0) lower[c] = upper[c] = estimate[c] = 0.0;
+    const bool invariant = n < m || bm == 0.0;  // the Krylov space is invariant: the quadrature is exact
+    if (!invariant || (psi && !S.fallback))
+        for (int rb = 0; rb < n; rb += TqCfg<MAXM>::RB)
+            tq_vectors<MAXM, false>(S, piv, rb, min(TqCfg<MAXM>::RB, n - rb));
+    if (psi) {  // the quadrature itself, from the same spectrum
+        if (S.fallback) {
+            if (warp == 0) quad_by_qr<MAXM>(S.a, S.b, n, sc, norm2[c], lane, psi + c);
+        } else {
+            tq_quadrature<MAXM>(S, sc, norm2[c], psi + c);
+        }
+        __syncthreads();
+    }
+    if (invariant) {
+        put(0.0, 0.0, 0.0);
         return;
     }
-    const double sc = scale[c] / S.s2;
-    double* Dp = piv + lane;
-    double* Rp = piv + MAXM * 32 + lane;
-    // first and last eigenvector components
-    for (int j = lane; j < n; j += 32) {
-        const double th = S.th[j];
-        double d = 0.0;
-        for (int k = 0; k < n; k++) {
-            d = guard_pivot((S.a[k] - th) - (k > 0 ? S.b[k - 1] * S.b[k - 1] / d : 0.0), S.pivmin);
-            Dp[k * 32] = d;
-        }
-        double r = 0.0, best = INFINITY;
-        int tw = n - 1;
-        for (int k = n - 1; k >= 0; k--) {
-            r = guard_pivot((S.a[k] - th) - (k + 1 < n ? S.b[k] * S.b[k] / r : 0.0), S.pivmin);
-            Rp[k * 32] = r;
-            const double gam = fabs(Dp[k * 32] + r - (S.a[k] - th));
-            if (gam < best) {
-                best = gam;
-                tw = k;
-            }
-        }
-        double nrm = 1.0, z = 1.0;
-        for (int k = tw - 1; k >= 0; k--) {
-            z = -S.b[k] * z / Dp[k * 32];
-            nrm = fma(z, z, nrm);
-        }
-        const double z1 = tw > 0 ? z : 1.0;
-        z = 1.0;
-        for (int k = tw + 1; k < n; k++) {
-            z = -S.b[k - 1] * z / Rp[k * 32];
-            nrm = fma(z, z, nrm);
-        }
-        const double zn = tw < n - 1 ? z : 1.0;
-        s_th[j] = sc * th;
-        s_ab[j] = bm * (zn * z1) / nrm;
+    if (tid == 0) {
+        S.gmin = 0x7ff0000000000000ULL;  // +inf
+        S.gmax = 0;
     }
-    __syncwarp();
-    for (int j = lane; j < n; j += 32) {
-        const double t = s_th[j];
-        double gsum = 0.0;
-        for (int l = 0; l < n; l++)
-            if (l != j) gsum += s_ab[l] / (t - s_th[l]);
-        s_gam[j] = gsum;
-        s_lt[j] = log(t);
+    for (int j = tid; j < n; j += blockDim.x) {
+        GTerm p;
+        const double ab = bm * (S.zn[j] * S.z1[j]) / S.nrm[j];
+        p.t = sc * S.th[j];
+        p.it = 1.0 / p.t;
+        p.lt = log(p.t);
+        p.ab2 = ab * ab;
+        p.c1 = 0.0;
+        G[j] = p;
+        S.c0[j] = ab;
     }
-    __syncwarp();
+    __syncthreads();
+    {  // gamma_j = sum_{l != j} a_l b_l / (theta_j - theta_l), four lanes per j
+        const int j = tid >> 2, part = tid & 3;
+        double gs = 0.0;
+        if (j < n)
+            for (int l = part; l < n; l += 4)
+                if (l != j) gs += S.c0[l] / (G[j].t - G[l].t);
+        gs += __shfl_xor_sync(0xffffffffu, gs, 1);
+        gs += __shfl_xor_sync(0xffffffffu, gs, 2);
+        if (part == 0 && j < n) {
+            G[j].c1 = 2.0 * S.c0[j] * gs;
+            S.c1[j] = G[j].c1 * G[j].lt;
+        }
+    }
+    __syncthreads();
     if (!(lam_min > 0.0)) {
         // half the smallest positive Ritz value of this column
         double tmin = INFINITY;
-        for (int j = lane; j < n; j += 32)
-            if (s_th[j] > 0.0) tmin = fmin(tmin, s_th[j]);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) tmin = fmin(tmin, __shfl_xor_sync(0xffffffffu, tmin, off));
+        for (int j = n - 1; j >= 0 && G[j].t > 0.0; j--) tmin = G[j].t;
         lam_min = 0.5 * tmin;
     }
     if (!(lam_min > 0.0 && lam_max > lam_min)) {
-        if (lane == 0) lower[c] = upper[c] = estimate[c] = INFINITY;  // no usable interval: not converged
+        put(INFINITY, INFINITY, INFINITY);  // no usable interval: not converged
         return;
     }
+    double g0 = 0.0;  // the part of g_m that does not depend on z
+    for (int j = 0; j < n; j++) g0 -= S.c1[j];
     const int npts = 2 * grid + n;
-    const double lratio = log(lam_max / lam_min);
-    double gmin = INFINITY, gmax = 0.0;
-    for (int q = lane; q < npts; q += 32) {
-        double z;
-        if (q < grid) z = grid > 1 ? lam_min * exp(lratio * q / (grid - 1)) : lam_min;
-        else if (q < 2 * grid) z = grid > 1 ? lam_min + (lam_max - lam_min) * (q - grid) / (grid - 1) : lam_min;
-        else {
-            z = s_th[q - 2 * grid];
+    const double lmin = log(lam_min), lratio = log(lam_max / lam_min), inv = grid > 1 ? 1.0 / (grid - 1) : 0.0;
+    const double lstep = lratio * inv, zstep = (lam_max - lam_min) * inv;
+    unsigned long long gmin = 0x7ff0000000000000ULL, gmax = 0;
+    for (int q = tid; q < npts; q += blockDim.x) {
+        double z, lz;
+        if (q < grid) {
+            const double x = lstep * q;
+            z = lam_min * exp(x);
+            lz = lmin + x;
+        } else if (q < 2 * grid) {
+            z = lam_min + zstep * (q - grid);
+            lz = log(z);
+        } else {
+            z = G[q - 2 * grid].t;
             if (!(z >= lam_min && z <= lam_max)) continue;
+            lz = G[q - 2 * grid].lt;
         }
-        const double lz = log(z);
-        double g = 0.0;
-        for (int j = 0; j < n; j++) {
-            const double ab = s_ab[j];
-            double dd1, dd2;
-            dd_entropy(z, lz, s_th[j], s_lt[j], dd1, dd2);
-            g += ab * ab * dd2 + 2.0 * ab * s_gam[j] * dd1;
+        double g = g0;
+        for (int j = 0; j < n; j++) g = g_term(z, lz, G[j], g);
+        // |g| >= 0: the order of the bits; NaN takes no part
+        const unsigned long long ab = (unsigned long long)absbits(g);
+        if (ab <= 0x7ff0000000000000ULL) {
+            gmin = min(gmin, ab);
+            gmax = max(gmax, ab);
         }
-        gmin = fmin(gmin, fabs(g));
-        gmax = fmax(gmax, fabs(g));
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        gmin = fmin(gmin, __shfl_xor_sync(0xffffffffu, gmin, off));
-        gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, off));
+        gmin = min(gmin, __shfl_xor_sync(0xffffffffu, gmin, off));
+        gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, off));
     }
     if (lane == 0) {
-        const double nb = norm2[c];
-        lower[c] = nb * gmin;
-        upper[c] = nb * gmax;
-        estimate[c] = nb * sqrt(gmin * gmax);
+        atomicMin(&S.gmin, gmin);
+        atomicMax(&S.gmax, gmax);
     }
+    __syncthreads();
+    const double lo = __longlong_as_double((long long)S.gmin), hi = __longlong_as_double((long long)S.gmax);
+    const double nb = norm2[c];
+    put(nb * lo, nb * hi, nb * sqrt(lo * hi));
 }
 
 cudaError_t launch_tridiag_bounds(const double* alpha, const double* beta, const double* norm2, const double* scale,
                                   int count, int m, int ld, double lam_min, double lam_max, int grid, double* lower,
-                                  double* upper, double* estimate, cudaStream_t st) {
+                                  double* upper, double* estimate, double* psi, cudaStream_t st) {
     return launch_tridiag_bounds_list(alpha, beta, norm2, scale, count, nullptr, nullptr, nullptr, m, ld, lam_min,
-                                      lam_max, grid, lower, upper, estimate, st);
+                                      lam_max, grid, lower, upper, estimate, psi, st);
 }
 
 cudaError_t launch_tridiag_bounds_list(const double* alpha, const double* beta, const double* norm2,
                                        const double* scale, int count, const int32_t* cols, const int32_t* mcol,
                                        const double* lam_max_col, int m, int ld, double lam_min, double lam_max,
-                                       int grid, double* lower, double* upper, double* estimate, cudaStream_t st) {
+                                       int grid, double* lower, double* upper, double* estimate, double* psi,
+                                       cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     // lam_min <= 0: half the smallest positive Ritz value of each column
     if ((!lam_max_col && !(lam_max > 0.0 && lam_max > lam_min)) || grid < 1) return cudaErrorInvalidValue;
 #define VNE_BOUND_CASE(MM)                                                                                   \
     if (m <= MM) {                                                                                          \
-        const int smem = 2 * MM * 32 * (int)sizeof(double);                                                 \
+        const int smem = TqCfg<MM>::kSmem;                                                                  \
         cudaError_t e = cudaFuncSetAttribute(k_tridiag_bounds<MM>,                                          \
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);            \
         if (e != cudaSuccess) return e;                                                                     \
-        k_tridiag_bounds<MM><<<count, 32, smem, st>>>(alpha, beta, norm2, scale, count, m, ld, lam_min, lam_max, \
-                                                       grid, lower, upper, estimate, cols, mcol, lam_max_col); \
+        k_tridiag_bounds<MM><<<count, TqCfg<MM>::NT, smem, st>>>(alpha, beta, norm2, scale, count, m, ld,   \
+                                                                  lam_min, lam_max, grid, lower, upper,     \
+                                                                  estimate, cols, mcol, lam_max_col, psi);  \
         return cudaGetLastError();                                                                          \
     }
     VNE_BOUND_CASE(32)
@@ -1150,16 +1241,16 @@ cudaError_t launch_tridiag_quad_list(const double* alpha, const double* beta, co
                                      const double* scale_per_col, int count, const int32_t* cols,
                                      const int32_t* mcol, int m, int ld, double* psi, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    // one warp (CTA) per tridiagonal; dynamic shared memory holds the
-    // twisted-factorisation pivots of the 32 lanes
+    // one CTA per tridiagonal; dynamic shared memory holds the
+    // twisted-factorisation pivots of up to 64 eigenvalues
 #define VNE_QUAD_CASE(MM)                                                                                    \
     if (m <= MM) {                                                                                          \
-        const int smem = 2 * MM * 32 * (int)sizeof(double);                                                 \
+        const int smem = TqCfg<MM>::kSmem;                                                                  \
         cudaError_t e = cudaFuncSetAttribute(k_tridiag_quad<MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                              smem);                                                         \
         if (e != cudaSuccess) return e;                                                                     \
-        k_tridiag_quad<MM><<<count, 32, smem, st>>>(alpha, beta, norm2, scale_per_col, count, m, ld, psi,    \
-                                                     cols, mcol);                                           \
+        k_tridiag_quad<MM><<<count, TqCfg<MM>::NT, smem, st>>>(alpha, beta, norm2, scale_per_col, count, m,  \
+                                                                ld, psi, cols, mcol);                       \
         return cudaGetLastError();                                                                          \
     }
     VNE_QUAD_CASE(32)
@@ -1172,17 +1263,17 @@ cudaError_t launch_tridiag_quad_list(const double* alpha, const double* beta, co
 cudaError_t launch_tridiag_fvec(const double* alpha, const double* beta, const double* scale_per_col, int count,
                                 int m, int ld, double* zvec, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
-    // one warp (CTA) per tridiagonal; dynamic shared memory: pivots /
-    // resolvent and the lanes' partial sums (3 x MM x 32 doubles), or Z for
-    // the QR fallback (MM x MM)
+    // one CTA per tridiagonal; dynamic shared memory: pivots / resolvent, or
+    // Z for the QR fallback (MM x MM, which fits)
 #define VNE_FVEC_CASE(MM)                                                                                    \
     if (m <= MM) {                                                                                          \
-        const int words = 3 * MM * 32 > MM * MM ? 3 * MM * 32 : MM * MM;                                    \
-        const int smem = words * (int)sizeof(double);                                                       \
+        const int smem = TqCfg<MM>::kSmem;                                                                  \
+        static_assert(TqCfg<MM>::kSmem >= MM * MM * (int)sizeof(double), "Z of the QR fallback");           \
         cudaError_t e = cudaFuncSetAttribute(k_tridiag_fvec<MM>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                              smem);                                                         \
         if (e != cudaSuccess) return e;                                                                     \
-        k_tridiag_fvec<MM><<<count, 32, smem, st>>>(alpha, beta, scale_per_col, count, m, ld, zvec);         \
+        k_tridiag_fvec<MM><<<count, TqCfg<MM>::NT, smem, st>>>(alpha, beta, scale_per_col, count, m, ld,    \
+                                                                zvec);                                      \
         return cudaGetLastError();                                                                          \
     }
     VNE_FVEC_CASE(32)

@@ -180,7 +180,7 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
         VNE_TRY_CUDA(ctx, launch_cg_tridiag(ah, bh, Kp, kk, s0, tau_a, tdiag, toff, st));
         for (int k = 1; k <= kk; k++)
             VNE_TRY_CUDA(ctx, launch_tridiag_bounds(tdiag, toff, norm2, ones, Kp, k, Kp, lam_min, lam_max, 1000, blo,
-                                                    blo + Kp, est + (size_t)(k - 1) * Kp, st));
+                                                    blo + Kp, est + (size_t)(k - 1) * Kp, nullptr, st));
         ctx->launches += 1 + kk;
         std::vector<double> he = download(ctx, est, (size_t)std::max(kk, 1) * Kp);
         // per column: the first k with err_k / err_{k-ell-1} >= c^ell (an

@@ -493,8 +493,8 @@ int tick_impl(vne_server* S) {
         std::vector<double> blam;
     };
     auto make_lists = [&](const std::vector<int>& quad_all, const std::vector<int>& est_q, int c_begin, int c_end) {
-        // quadratures of all columns of quad_all, quadratures and estimates
-        // of columns [c_begin, c_end) of est_q
+        // quadratures of all columns of quad_all (q..); quadratures and
+        // estimates, from one kernel, of columns [c_begin, c_end) of est_q (b..)
         Lists L;
         for (int ri : quad_all) {
             const vne_server::Req& rq = S->reqs[ri];
@@ -506,8 +506,6 @@ int tick_impl(vne_server* S) {
         for (int ri : est_q) {
             const vne_server::Req& rq = S->reqs[ri];
             for (int c = c_begin; c < c_end; c++) {
-                L.qcols.push_back(rq.slot * K + c);
-                L.qm.push_back(rq.j);
                 L.bcols.push_back(rq.slot * K + c);
                 L.bm.push_back(rq.j);
                 L.blam.push_back(rq.lam_max);
@@ -613,16 +611,19 @@ int tick_impl(vne_server* S) {
     std::vector<double> hp, he;
     auto evaluate = [&](const Lists& L, const int32_t* qc, const int32_t* qm, const int32_t* bc, const int32_t* bm,
                         const double* bl) {
-        if (L.qcols.empty()) return;
+        if (L.qcols.empty() && L.bcols.empty()) return;
         // the kernels' step bucket from the largest step count listed
-        const int mx = *std::max_element(L.qm.begin(), L.qm.end());
-        VNE_TRY_CUDA(ctx, launch_tridiag_quad_list(S->alpha, S->beta, S->norm2, S->scale, (int)L.qcols.size(), qc,
-                                                   qm, mx, SK, S->psi, st));
-        ctx->launches += 1;
+        if (!L.qcols.empty()) {
+            const int mx = *std::max_element(L.qm.begin(), L.qm.end());
+            VNE_TRY_CUDA(ctx, launch_tridiag_quad_list(S->alpha, S->beta, S->norm2, S->scale, (int)L.qcols.size(),
+                                                       qc, qm, mx, SK, S->psi, st));
+            ctx->launches += 1;
+        }
         if (!L.bcols.empty()) {
+            const int mx = *std::max_element(L.bm.begin(), L.bm.end());
             VNE_TRY_CUDA(ctx, launch_tridiag_bounds_list(S->alpha, S->beta, S->norm2, S->scale, (int)L.bcols.size(),
                                                          bc, bm, bl, mx, SK, 0.0, 1.0, S->grid, S->est,
-                                                         S->est + SK, S->est + 2 * SK, st));
+                                                         S->est + SK, S->est + 2 * SK, S->psi, st));
             ctx->launches += 1;
             he = download(ctx, S->est + 2 * SK, SK);
         }
@@ -646,8 +647,8 @@ int tick_impl(vne_server* S) {
     // of the first evaluation for every other column)
     if (!candidates.empty() && kFirst < K) {
         Lists LB = make_lists({}, candidates, kFirst, K);
-        evaluate(LB, upload(ctx, "srv.qcols", LB.qcols), upload(ctx, "srv.qm", LB.qm),
-                 upload(ctx, "srv.bcols", LB.bcols), upload(ctx, "srv.bm", LB.bm), upload(ctx, "srv.blam", LB.blam));
+        evaluate(LB, nullptr, nullptr, upload(ctx, "srv.bcols", LB.bcols), upload(ctx, "srv.bm", LB.bm),
+                 upload(ctx, "srv.blam", LB.blam));
     }
     for (int ri : candidates)
         if (passes(S->reqs[ri], kFirst, K)) block_done[ri] = 1;
