@@ -687,17 +687,32 @@ std::vector<double> quadforms(vne_matrix* M, const vne_options* o, StartSource s
 }
 
 
+OpConsts op_consts(vne_ctx* ctx, const Problem& P, int Kp, double shift, const std::string& tag) {
+    const double scale = P.segs[0].scale;
+    std::vector<double> h((size_t)3 * Kp);
+    for (int c = 0; c < Kp; c++) {
+        h[c] = scale;
+        h[Kp + c] = -shift;
+        h[2 * Kp + c] = 1.0;
+    }
+    OpConsts k;
+    k.shift = shift;
+    k.sig = upload(ctx, tag, h);
+    k.cp = k.sig + Kp;
+    k.one = k.sig + 2 * Kp;
+    return k;
+}
+
 // Apply the operator to a panel-major block with the Lanczos step kernel:
 // out = A in + shift * in (A = scale M), and dq[c] = scale * (in . out).
 template <typename T>
-void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* out, double shift, double* dq,
-                    int variant, const std::string& tag) {
+void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* out, const OpConsts& k, double* dq,
+                    int variant) {
     cudaStream_t st = ctx->stream;
     const int panels = Kp / ks;
     const int ctas = P.ctas_per_panel(), tiles = P.tiles_per_panel();
     const int nh = (int)P.hubs.size();
-    const double scale = P.segs[0].scale;
-    std::vector<double> hs(Kp, scale), hc(Kp, -shift), h1(Kp, 1.0);
+    const double shift = k.shift;
     StepParams<T> p{};
     p.rowptr = P.rowptr;
     p.col = P.col;
@@ -725,9 +740,9 @@ void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* ou
     p.w_prev = in;
     p.u = out;
     p.w_next = out;
-    p.sig_cur = upload(ctx, tag + ".sig", hs);
-    p.beta_prev = upload(ctx, tag + ".cp", hc);
-    p.sig_prev = upload(ctx, tag + ".one", h1);
+    p.sig_cur = k.sig;
+    p.beta_prev = k.cp;
+    p.sig_prev = k.one;
     p.alpha = dq;
     p.part = ws_get_t<double>(ctx, "op.part", (size_t)panels * std::max(ctas, tiles) * ks);
     p.counter = ws_get_t<uint32_t>(ctx, "op.counter", (size_t)panels);
@@ -753,8 +768,7 @@ void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* ou
                                const std::string&, BlockOut&, int, bool, bool, bool, const Adaptive*);          \
     template std::vector<double> quadforms<T>(vne_matrix*, const vne_options*, StartSource, int, int,             \
                                               const double*);                                                    \
-    template void apply_operator<T>(vne_ctx*, Problem&, int, int, const T*, T*, double, double*, int,             \
-                                    const std::string&);
+    template void apply_operator<T>(vne_ctx*, Problem&, int, int, const T*, T*, const OpConsts&, double*, int);
 VNE_ENGINE_INSTANTIATE(float)
 VNE_ENGINE_INSTANTIATE(double)
 

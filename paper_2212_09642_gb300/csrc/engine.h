@@ -341,11 +341,19 @@ template <typename T>
 std::vector<double> quadforms(vne_matrix* M, const vne_options* o, StartSource src, int ncols, int m,
                               const double* abs_tol = nullptr);
 
+// The step kernel's per-column scalars for out = A in + shift * in, on the
+// device (workspace `tag`): uploaded once per solve, since a copy from
+// pageable memory waits for the stream.
+struct OpConsts {
+    double shift = 0.0;
+    const double *sig = nullptr, *cp = nullptr, *one = nullptr;
+};
+OpConsts op_consts(vne_ctx* ctx, const Problem& P, int Kp, double shift, const std::string& tag);
 // out = A in + shift * in (A = scale M) and dq[c] = scale * (in . out), with
 // the Lanczos step kernel.
 template <typename T>
-void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* out, double shift, double* dq,
-                    int variant, const std::string& tag);
+void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* out, const OpConsts& k, double* dq,
+                    int variant);
 
 // Rational Krylov quadratic forms (rational_driver.cu).
 template <typename T>

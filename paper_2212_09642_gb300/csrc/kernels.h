@@ -211,25 +211,45 @@ template <typename T>
 cudaError_t launch_cgs_scale(T* v, const double* orig2, const double* rem2, double drop, int n, int K, int ks,
                              int tiles_per_panel, const RowTile* tiles, cudaStream_t st);
 struct CgState {
-    int32_t K, nshift;
+    int32_t K, nshift, window;  // window: residuals kept between two flushes
     double scale, shift0, tol;
     const double* shift;  // [nshift] (device)
     const double* dq;     // step-kernel output: scale * (p . q) per column
-    double *rho, *rho_new, *a, *b, *a_prev, *b_prev, *cnorm;
-    double *zeta, *zeta_prev, *zeta_next, *as, *bs, *resid;  // [nshift][K]
-    int32_t *active, *iters;                                  // [nshift][K]
-    int32_t* any_active;
+    double *rho, *b, *a_prev, *b_prev, *cnorm;           // [K]
+    double *zeta, *zeta_prev, *zeta_next, *resid;        // [nshift][K]
+    int32_t *active, *iters;                              // [nshift][K]
+    int32_t* any_active;                                  // [panels]
+    double *hz, *ha, *hb;  // [window][nshift][K]: zeta_k, a_s, b_s of the window's iterations (0: shift inactive)
+    double* bstart;        // [nshift][K]: b_s of the iteration before the window
+    double *ah, *bh;       // nullable [rows][K]: a and b of the first `hist_rows` iterations
+    int32_t hist_rows;
 };
 
 template <typename T>
 struct CgVectors {
     int32_t n, tiles_per_panel;
     const RowTile* tiles;
-    T *r, *q, *p;
-    T* x[8];
-    T* ps[8];
+    const T* r;  // residual r_k
+    T* r_next;   // r_{k+1}: the next slot of the residual window
+    T *q, *p;
     double* part;
     uint32_t* counter;
+};
+
+// One flush of a residual window (k_cg_coefs, k_cg_flush).
+template <typename T>
+struct CgFlush {
+    int32_t n, K, nshift, panels;
+    int32_t count;        // residuals in the window (<= CgState::window)
+    int32_t first, last;  // first flush: x and p_s start from zero; last: p_s is not needed any more
+    const T* r;           // residual slots, [slots][K / ks][n][ks]
+    size_t slot_stride;
+    int32_t slot0, slots;  // slot of the window's first residual; slots in the ring
+    T* x[8];
+    T* ps[8];
+    T* coef;        // [window][nshift][2][K]: of r_i in x_s and in p_s
+    T* coef_p;      // [nshift][2][K]: of the incoming p_s
+    int32_t* live;  // [panels]: bit s set if shift s changed in the window
 };
 
 // Both Gram matrices of a basis W and its image A W in one pass over the
@@ -247,9 +267,11 @@ struct MultiGram {
 template <typename T> cudaError_t launch_multi_gram(MultiGram<T> g, double* out, cudaStream_t);
 
 
-cudaError_t launch_cg_scalars_a(const CgState&, cudaStream_t);
-cudaError_t launch_cg_scalars_b(const CgState&, cudaStream_t);
-template <typename T> cudaError_t launch_cg_update(const CgVectors<T>&, const CgState&, int ks, int panels, cudaStream_t);
+template <typename T>
+cudaError_t launch_cg_update(const CgVectors<T>&, const CgState&, int ks, int panels, int window_index, int iteration,
+                             cudaStream_t);
+template <typename T>
+cudaError_t launch_cg_flush(const CgFlush<T>&, const CgState&, int ks, cudaStream_t);
 template <typename T> cudaError_t launch_cg_direction(const CgVectors<T>&, const CgState&, int ks, int panels, cudaStream_t);
 template <typename T>
 struct BlockTransform {

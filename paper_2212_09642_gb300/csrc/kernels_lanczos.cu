@@ -22,57 +22,9 @@
 // (panel, segment), in a fixed order, so results are bit-reproducible.
 #include "common.cuh"
 #include "kernels.h"
+#include "reduce.cuh"
 
 namespace vne {
-
-// ---------------------------------------------------------------------------
-// fixed-order cross-CTA reduction
-//
-// Every CTA writes NQ*KS partial values at part[(panel*nparts + idx)*W + c]
-// (W = NQ*KS) and calls this; the CTA that arrives last for the counter sums
-// the `count` partials starting at `begin` in index order and returns true
-// with the totals in s_out[0..W).  The counter is reset for the next launch.
-template <int W>
-__device__ bool last_cta_reduce(const double* part, uint32_t* counter, int panel, int nparts,
-                                int begin, int count, double* s_out) {
-    __shared__ int s_last;
-    __shared__ double red[VNE_THREADS];
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned old = atomicAdd(counter, 1u);
-        s_last = (old == (unsigned)(count - 1));
-    }
-    __syncthreads();
-    if (!s_last) return false;
-    __threadfence();
-    constexpr int NS = VNE_THREADS / W;
-    const int c = threadIdx.x % W, s = threadIdx.x / W;
-    // four independent accumulators, so that four loads are in flight at
-    // once (the order of the additions is still fixed)
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    if (s < NS) {
-        const double* src = part + ((size_t)panel * nparts + begin) * W + c;
-        int i = s;
-        for (; i + 3 * NS < count; i += 4 * NS) {
-#pragma unroll
-            for (int u = 0; u < 4; u++) acc[u] += ld_cg(src + (size_t)(i + u * NS) * W);
-        }
-#pragma unroll
-        for (int u = 0; u < 3; u++)
-            if (i + u * NS < count) acc[u] += ld_cg(src + (size_t)(i + u * NS) * W);
-    }
-    red[threadIdx.x] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-    __syncthreads();
-    if (threadIdx.x < W) {
-        double t = 0.0;
-        for (int q = 0; q < NS; q++) t += red[q * W + threadIdx.x];
-        s_out[threadIdx.x] = t;
-    }
-    if (threadIdx.x == 0) *counter = 0u;
-    __syncthreads();
-    return true;
-}
 
 // ---------------------------------------------------------------------------
 // counter-based Rademacher entries (SplitMix64 mixer; see the header of
@@ -315,7 +267,7 @@ __global__ void __launch_bounds__(VNE_THREADS, 4) k_start_mean(StartParams<T> p)
     }
     cta_column_partials<KS>(sum, rsub, c0, p.part + ((size_t)panel * p.tiles_per_panel + tile) * KS);
     __shared__ double tot[KS];
-    if (last_cta_reduce<KS>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
+    if (last_cta_reduce<KS, sizeof(T) == 8>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
                             sg.tile_begin, sg.tile_count, tot)) {
         if (threadIdx.x < KS)
             p.mean[(size_t)t.seg * p.K + panel * KS + threadIdx.x] = tot[threadIdx.x] / (double)sg.rows;
@@ -427,7 +379,7 @@ __global__ void __launch_bounds__(VNE_THREADS, 3) k_start_center(StartParams<T> 
     }
     cta_column_partials<KS>(sum, rsub, c0, p.part + ((size_t)panel * p.tiles_per_panel + tile) * KS);
     __shared__ double tot[KS];
-    if (last_cta_reduce<KS>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
+    if (last_cta_reduce<KS, sizeof(T) == 8>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
                             sg.tile_begin, sg.tile_count, tot)) {
         if (threadIdx.x < KS) {
             size_t o = (size_t)t.seg * p.K + panel * KS + threadIdx.x;
@@ -831,7 +783,7 @@ __global__ void __launch_bounds__(VNE_THREADS, MINB) k_step(StepParams<T> p) {
     }
     __shared__ double tot[KS];
     const SegInfo sg = p.seg[seg];
-    if (last_cta_reduce<KS>(p.part, p.counter + (size_t)panel * p.nseg + seg, panel, p.ctas_per_panel,
+    if (last_cta_reduce<KS, sizeof(T) == 8>(p.part, p.counter + (size_t)panel * p.nseg + seg, panel, p.ctas_per_panel,
                             sg.cta_begin, sg.cta_count, tot)) {
         // add the long rows' shares in a fixed order (strided over the CTA)
         __shared__ double hred[VNE_THREADS];
@@ -908,7 +860,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_update(StepParams<T> p) {
     }
     __shared__ double tot[KS];
     const SegInfo sg = p.seg[t.seg];
-    if (last_cta_reduce<KS>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
+    if (last_cta_reduce<KS, sizeof(T) == 8>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
                             sg.tile_begin, sg.tile_count, tot)) {
         if (threadIdx.x < KS) {
             size_t o = (size_t)t.seg * p.K + panel * KS + threadIdx.x;

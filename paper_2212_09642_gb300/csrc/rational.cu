@@ -14,11 +14,24 @@
 // Per CG iteration, for a block of K columns (panel-major, as in the
 // Lanczos engine):
 //   step kernel (shared with Lanczos)  q = (A + s_0 I) p,  d = p . q
-//   k_cg_scalars_a   a = rho / d, zeta_{k+1}, a_s     (per column, FP64)
-//   k_cg_update      p_s = zeta_k r + b_s p_s, x_s += a_s p_s, r -= a q,
-//                    rho' = ||r||^2
-//   k_cg_scalars_b   b = rho'/rho, b_s, convergence, shift history
+//   k_cg_update      a = rho / d, r_{k+1} = r_k - a q into the next slot of a
+//                    window of residuals, rho' = ||r_{k+1}||^2; the CTA that
+//                    finishes a panel advances the panel's scalars: b =
+//                    rho'/rho, zeta_s, a_s, b_s, convergence, and records
+//                    zeta_s, a_s, b_s of the iteration
 //   k_cg_direction   p = r + b p
+// The shifted iterates are not touched per iteration.  With p_{s,k} =
+// zeta_k r_k + b_{s,k-1} p_{s,k-1} and x_s += a_{s,k} p_{s,k}, a whole window
+// of iterations adds to x_s and leaves in p_s fixed combinations of the
+// window's residuals and of the p_s that entered it; their coefficients
+// follow from the recorded scalars by a backward recurrence (k_cg_coefs), and
+// one pass (k_cg_flush) reads every residual of the window once for all
+// shifts.  An iteration then moves 6 vectors and a share of (window + 4 per
+// live shift) / window instead of 6 + 4 per live shift.  Measured at n = 10^6,
+// 22 columns, 8 shifts, FP32, per iteration: update 88 us and flush 46 us
+// against 283 us for the update that touched every live x_s and p_s and 19 us
+// for its scalar kernels (estimate 397 -> 278 ms); FP64, n = 30,000, 12
+// columns: 23 + 10 us against 51 + 15 us (88 -> 59 ms).
 // Afterwards the basis W and A W are formed (A^j c by the step kernel,
 // A x_s by the step kernel), their Gram matrices W^T W and W^T A W are
 // accumulated per column in one pass over the vectors (k_multi_gram), and a per-column FP64 kernel orthonormalises W in
@@ -34,6 +47,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "reduce.cuh"
 
 namespace vne {
 
@@ -42,9 +56,9 @@ constexpr int kMaxBasis = 24;  // 1 + up to 15 polynomial directions + 8 poles
 
 __device__ __forceinline__ double f_ent(double x) { return x > 0.0 ? -x * log(x) : 0.0; }
 
-// x_s = 0, r = p = p_s = c are set by copies; here the scalar state:
-// rho = ||c||^2, zeta = zeta_prev = 1, a_prev = 1, b_prev = 0, all shifts
-// active for non-zero columns.
+// r = p = c are set by copies; here the scalar state: rho = ||c||^2, zeta =
+// zeta_prev = 1, a_prev = 1, b_prev = 0, all shifts active for non-zero
+// columns.
 __global__ void k_cg_init(CgState st, const double* norm2) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= st.K) return;
@@ -53,15 +67,13 @@ __global__ void k_cg_init(CgState st, const double* norm2) {
     st.cnorm[c] = sqrt(n2);
     st.a_prev[c] = 1.0;
     st.b_prev[c] = 0.0;
-    st.a[c] = 0.0;
     st.b[c] = 0.0;
     for (int s = 0; s < st.nshift; s++) {
         const size_t o = (size_t)s * st.K + c;
         st.zeta[o] = 1.0;
         st.zeta_prev[o] = 1.0;
         st.zeta_next[o] = 1.0;
-        st.as[o] = 0.0;
-        st.bs[o] = 0.0;
+        st.bstart[o] = 0.0;
         st.active[o] = n2 > 0.0 ? 1 : 0;
         st.iters[o] = 0;
         st.resid[o] = n2 > 0.0 ? 1.0 : 0.0;
@@ -73,100 +85,37 @@ cudaError_t launch_cg_init(CgState st, const double* norm2, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// per column: a = rho / d (d from the step kernel as scale * (p . q)), then
-// the shifted coefficients
-__global__ void k_cg_scalars_a(CgState st) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= st.K) return;
-    const double d = st.dq[c] / st.scale;
-    const double rho = st.rho[c];
-    double a = (d > 0.0 && rho > 0.0) ? rho / d : 0.0;
-    st.a[c] = a;
-    for (int s = 0; s < st.nshift; s++) {
-        const size_t o = (size_t)s * st.K + c;
-        if (!st.active[o] || a == 0.0) {
-            st.as[o] = 0.0;
-            continue;
-        }
-        const double zk = st.zeta[o], zkm1 = st.zeta_prev[o];
-        const double ap = st.a_prev[c], bp = st.b_prev[c];
-        const double delta = st.shift[s] - st.shift0;
-        const double den = ap * zkm1 * (1.0 + delta * a) + a * bp * (zkm1 - zk);
-        const double zn = (den != 0.0) ? zk * zkm1 * ap / den : 0.0;
-        st.zeta_next[o] = zn;
-        st.as[o] = (zk != 0.0) ? a * zn / zk : 0.0;
-    }
-}
-
-// per column: b = rho' / rho and the shifted b_s, convergence, history shift
-__global__ void k_cg_scalars_b(CgState st) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= st.K) return;
-    const double rho = st.rho[c], rhon = st.rho_new[c];
-    const double b = (rho > 0.0) ? rhon / rho : 0.0;
-    st.b[c] = b;
-    const double rnorm = sqrt(rhon);
-    int any = 0;
-    for (int s = 0; s < st.nshift; s++) {
-        const size_t o = (size_t)s * st.K + c;
-        if (!st.active[o]) continue;
-        const double zk = st.zeta[o], zn = st.zeta_next[o];
-        const double ratio = (zk != 0.0) ? zn / zk : 0.0;
-        st.bs[o] = b * ratio * ratio;
-        st.zeta_prev[o] = zk;
-        st.zeta[o] = zn;
-        st.iters[o] += 1;
-        const double res = fabs(zn) * rnorm;
-        st.resid[o] = res / st.cnorm[c];
-        if (!(res > st.tol * st.cnorm[c])) st.active[o] = 0;  // converged (or breakdown)
-        else any = 1;
-    }
-    st.a_prev[c] = st.a[c];
-    st.b_prev[c] = b;
-    st.rho[c] = rhon;
-    if (any) atomicOr(st.any_active, 1);
-}
-
-// r -= a q;  rho' = ||r||^2 (FP64 across the CTA, fixed-order last-CTA sum);
-// for active shifts first the shifted direction of this iteration,
-// p_s = zeta_k r + b_s p_s (r before its update: the direction kernel of the
-// previous iteration left it to this pass, which reads r anyway), then
-// x_s += a_s p_s.  Each lane owns CPL consecutive columns of a row (16-byte
-// vector accesses); a shift's x_s and p_s are touched only by lanes that
-// have an active column for it.
+// r_{k+1} = r_k - a q with a = rho / d (d from the step kernel as scale *
+// (p . q)), rho' = ||r_{k+1}||^2 (runs of 16 rows in the data precision, FP64
+// across runs and CTAs).  Each lane owns CPL consecutive columns of a row
+// (16-byte vector accesses), four rows in flight.  A pure stream of three
+// vectors.  The last CTA of a panel advances the panel's scalars, one thread
+// per (shift, column): two single-warp kernels did that before, 19 us per
+// iteration of dependent FP64 arithmetic that this tail spreads over a CTA.
 template <typename T, int KS>
-__global__ void __launch_bounds__(VNE_THREADS, 2) k_cg_update(CgVectors<T> v, CgState st) {
+__global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgState st, int wi, int it) {
     constexpr int CPL = LaneVec<T>::CPL;
     constexpr int LPR = KS / CPL;            // lanes per row
     constexpr int RPI = VNE_THREADS / LPR;   // rows per iteration
+    constexpr int U = 4;
     const int panel = blockIdx.x / v.tiles_per_panel, tile = blockIdx.x % v.tiles_per_panel;
     const RowTile t = v.tiles[tile];
     const int sub = threadIdx.x % LPR, rs = threadIdx.x / LPR;
     const int cofs = sub * CPL;
     const size_t pofs = (size_t)panel * v.n * KS;
-    // per-column coefficients in shared memory; this lane's active columns
-    // as a bit mask (bit s * CPL + q)
-    __shared__ __align__(16) T s_as[kMaxShifts][KS], s_z[kMaxShifts][KS], s_b[kMaxShifts][KS];
-    for (int i = threadIdx.x; i < kMaxShifts * KS; i += VNE_THREADS) {
-        const int sh = i / KS, cc = i % KS;
-        const size_t o = (size_t)sh * st.K + panel * KS + cc;
-        const bool on = sh < st.nshift && st.active[o];
-        s_as[sh][cc] = on ? (T)st.as[o] : (T)0;
-        s_z[sh][cc] = on ? (T)st.zeta[o] : (T)0;  // zeta_k
-        s_b[sh][cc] = on ? (T)st.bs[o] : (T)0;    // b_s of the previous iteration
+    __shared__ double s_a[KS];
+    if (threadIdx.x < KS) {
+        const int c = panel * KS + threadIdx.x;
+        const double d = st.dq[c] / st.scale, rho = st.rho[c];
+        s_a[threadIdx.x] = (d > 0.0 && rho > 0.0) ? rho / d : 0.0;
     }
-    uint32_t amask = 0;
-#pragma unroll
-    for (int sh = 0; sh < kMaxShifts; sh++)
-#pragma unroll
-        for (int q = 0; q < CPL; q++)
-            if (sh < st.nshift && st.active[(size_t)sh * st.K + panel * KS + cofs + q]) amask |= 1u << (sh * CPL + q);
     __syncthreads();
     T a[CPL];
 #pragma unroll
-    for (int q = 0; q < CPL; q++) a[q] = (T)st.a[panel * KS + cofs + q];
-    T* R = v.r + pofs;
-    const T* Q = v.q + pofs;
+    for (int q = 0; q < CPL; q++) a[q] = (T)s_a[cofs + q];
+    const T* __restrict__ R = v.r + pofs;
+    T* __restrict__ Rn = v.r_next + pofs;
+    const T* __restrict__ Q = v.q + pofs;
     double acc[CPL];
     T accf[CPL];
 #pragma unroll
@@ -175,29 +124,29 @@ __global__ void __launch_bounds__(VNE_THREADS, 2) k_cg_update(CgVectors<T> v, Cg
         accf[q] = (T)0;
     }
     int cnt = 0;
-    for (int r = t.row_begin + rs; r < t.row_end; r += RPI) {
-        const size_t o = (size_t)r * KS + cofs;
-        // every load of the row first (the pointers may alias as far as the
-        // compiler knows, so a store between them would serialise them)
-        T rv[CPL], qv[CPL];
-        load_lane(R + o, rv);
-        load_lane_stream(Q + o, qv);
-        T xv[kMaxShifts][CPL], pv[kMaxShifts][CPL];
+    for (int r0 = t.row_begin + rs; r0 < t.row_end; r0 += U * RPI) {
+        T rv[U][CPL], qv[U][CPL];
 #pragma unroll
-        for (int sh = 0; sh < kMaxShifts; sh++)
-            if ((amask >> (sh * CPL)) & ((1u << CPL) - 1u)) {
-                load_lane(v.x[sh] + pofs + o, xv[sh]);
-                load_lane_stream(v.ps[sh] + pofs + o, pv[sh]);
+        for (int u = 0; u < U; u++) {
+            const int r = r0 + u * RPI;
+            if (r < t.row_end) {
+                load_lane(R + (size_t)r * KS + cofs, rv[u]);
+                load_lane_stream(Q + (size_t)r * KS + cofs, qv[u]);
             }
-        T r0[CPL];  // r_k, for the shifted directions
-#pragma unroll
-        for (int q = 0; q < CPL; q++) {
-            r0[q] = rv[q];
-            rv[q] -= a[q] * qv[q];
-            accf[q] += rv[q] * rv[q];
         }
-        store_lane(R + o, rv);
-        if (++cnt == 16) {
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int r = r0 + u * RPI;
+            if (r < t.row_end) {
+#pragma unroll
+                for (int q = 0; q < CPL; q++) {
+                    rv[u][q] -= a[q] * qv[u][q];
+                    accf[q] += rv[u][q] * rv[u][q];
+                }
+                store_lane(Rn + (size_t)r * KS + cofs, rv[u]);
+            }
+        }
+        if ((cnt += U) == 16) {
 #pragma unroll
             for (int q = 0; q < CPL; q++) {
                 acc[q] += (double)accf[q];
@@ -205,57 +154,93 @@ __global__ void __launch_bounds__(VNE_THREADS, 2) k_cg_update(CgVectors<T> v, Cg
             }
             cnt = 0;
         }
-#pragma unroll
-        for (int sh = 0; sh < kMaxShifts; sh++) {
-            const uint32_t m = (amask >> (sh * CPL)) & ((1u << CPL) - 1u);
-            if (!m) continue;
-            T cv[CPL], zv[CPL], bv[CPL];
-            load_lane(&s_as[sh][cofs], cv);
-            load_lane(&s_z[sh][cofs], zv);
-            load_lane(&s_b[sh][cofs], bv);
-#pragma unroll
-            for (int q = 0; q < CPL; q++)
-                if (m & (1u << q)) {
-                    pv[sh][q] = zv[q] * r0[q] + bv[q] * pv[sh][q];
-                    xv[sh][q] += cv[q] * pv[sh][q];
-                }
-            store_lane(v.ps[sh] + pofs + o, pv[sh]);
-            store_lane(v.x[sh] + pofs + o, xv[sh]);
-        }
     }
-    __shared__ double red[RPI][KS];
 #pragma unroll
-    for (int q = 0; q < CPL; q++) red[rs][cofs + q] = acc[q] + (double)accf[q];
-    __syncthreads();
-    if (threadIdx.x < KS) {
-        double sum = 0.0;
-        for (int q = 0; q < RPI; q++) sum += red[q][threadIdx.x];
-        v.part[((size_t)panel * v.tiles_per_panel + tile) * KS + threadIdx.x] = sum;
-    }
-    // last CTA of the panel sums the partials in tile order
-    __shared__ int s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = (atomicAdd(v.counter + panel, 1u) == (unsigned)(v.tiles_per_panel - 1));
-    __syncthreads();
-    if (s_last) {
+    for (int q = 0; q < CPL; q++) acc[q] += (double)accf[q];
+    constexpr bool kSerial = sizeof(T) == 8;
+    __shared__ double red[kSerial ? RPI : VNE_WARPS][KS];
+    double tot;
+    if (kSerial) cta_colsum_serial<KS, CPL>(acc, red, tot);
+    else cta_colsum<KS, CPL>(acc, red, tot);
+    if (threadIdx.x < KS) v.part[((size_t)panel * v.tiles_per_panel + tile) * KS + threadIdx.x] = tot;
+    __shared__ double s_rho[KS];
+    if (kSerial) {
+        __shared__ int s_last;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) s_last = (atomicAdd(v.counter + panel, 1u) == (unsigned)(v.tiles_per_panel - 1));
+        __syncthreads();
+        if (!s_last) return;
         __threadfence();
         if (threadIdx.x < KS) {
             double sum = 0.0;
             for (int i = 0; i < v.tiles_per_panel; i++)
                 sum += __ldcg(&v.part[((size_t)panel * v.tiles_per_panel + i) * KS + threadIdx.x]);
-            st.rho_new[panel * KS + threadIdx.x] = sum;
+            s_rho[threadIdx.x] = sum;
         }
         if (threadIdx.x == 0) v.counter[panel] = 0u;
+        __syncthreads();
+    } else if (!last_cta_reduce<KS>(v.part, v.counter + panel, panel, v.tiles_per_panel, 0, v.tiles_per_panel, s_rho)) {
+        return;
     }
+    int any = 0;
+    for (int idx = threadIdx.x; idx < st.nshift * KS; idx += VNE_THREADS) {
+        const int s = idx / KS, cc = idx % KS, c = panel * KS + cc;
+        const size_t o = (size_t)s * st.K + c, h = ((size_t)wi * st.nshift + s) * st.K + c;
+        if (!st.active[o]) {
+            st.hz[h] = st.ha[h] = st.hb[h] = 0.0;
+            continue;
+        }
+        // shifted step length from the collinear residuals
+        const double aa = s_a[cc], rho = st.rho[c], rhon = s_rho[cc];
+        const double zk = st.zeta[o];
+        double zn = st.zeta_next[o], as = 0.0;
+        if (aa != 0.0) {
+            const double zkm1 = st.zeta_prev[o];
+            const double ap = st.a_prev[c], bp = st.b_prev[c];
+            const double delta = st.shift[s] - st.shift0;
+            const double den = ap * zkm1 * (1.0 + delta * aa) + aa * bp * (zkm1 - zk);
+            zn = (den != 0.0) ? zk * zkm1 * ap / den : 0.0;
+            as = (zk != 0.0) ? aa * zn / zk : 0.0;
+            st.zeta_next[o] = zn;
+        }
+        const double b = (rho > 0.0) ? rhon / rho : 0.0;
+        const double ratio = (zk != 0.0) ? zn / zk : 0.0;
+        st.hz[h] = zk;
+        st.ha[h] = as;
+        st.hb[h] = b * ratio * ratio;
+        st.zeta_prev[o] = zk;
+        st.zeta[o] = zn;
+        st.iters[o] += 1;
+        const double res = fabs(zn) * sqrt(rhon);
+        st.resid[o] = res / st.cnorm[c];
+        if (!(res > st.tol * st.cnorm[c])) st.active[o] = 0;  // converged (or breakdown)
+        else any = 1;
+    }
+    any = __syncthreads_or(any);
+    if (threadIdx.x < KS) {
+        const int c = panel * KS + threadIdx.x;
+        const double rho = st.rho[c], rhon = s_rho[threadIdx.x], aa = s_a[threadIdx.x];
+        const double b = (rho > 0.0) ? rhon / rho : 0.0;
+        st.a_prev[c] = aa;
+        st.b_prev[c] = b;
+        st.b[c] = b;
+        st.rho[c] = rhon;
+        if (st.ah && it < st.hist_rows) {
+            st.ah[(size_t)it * st.K + c] = aa;
+            st.bh[(size_t)it * st.K + c] = b;
+        }
+    }
+    if (threadIdx.x == 0) st.any_active[panel] = any;
 }
 
-// p = r + b p (the shifted directions are formed by the next k_cg_update)
+// p = r + b p
 template <typename T, int KS>
 __global__ void __launch_bounds__(VNE_THREADS) k_cg_direction(CgVectors<T> v, CgState st) {
     constexpr int CPL = LaneVec<T>::CPL;
     constexpr int LPR = KS / CPL;
     constexpr int RPI = VNE_THREADS / LPR;
+    constexpr int U = 4;
     const int panel = blockIdx.x / v.tiles_per_panel, tile = blockIdx.x % v.tiles_per_panel;
     const RowTile t = v.tiles[tile];
     const int sub = threadIdx.x % LPR, rs = threadIdx.x / LPR;
@@ -264,16 +249,173 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_direction(CgVectors<T> v, Cg
     T b[CPL];
 #pragma unroll
     for (int q = 0; q < CPL; q++) b[q] = (T)st.b[panel * KS + cofs + q];
-    const T* R = v.r + pofs;
-    T* Pp = v.p + pofs;
-    for (int r = t.row_begin + rs; r < t.row_end; r += RPI) {
-        const size_t o = (size_t)r * KS + cofs;
-        T rv[CPL], pv[CPL];
-        load_lane_stream(R + o, rv);
-        load_lane(Pp + o, pv);
+    const T* __restrict__ R = v.r_next + pofs;
+    T* __restrict__ Pp = v.p + pofs;
+    for (int r0 = t.row_begin + rs; r0 < t.row_end; r0 += U * RPI) {
+        T rv[U][CPL], pv[U][CPL];
 #pragma unroll
-        for (int q = 0; q < CPL; q++) pv[q] = rv[q] + b[q] * pv[q];
-        store_lane(Pp + o, pv);
+        for (int u = 0; u < U; u++) {
+            const int r = r0 + u * RPI;
+            if (r < t.row_end) {
+                load_lane(R + (size_t)r * KS + cofs, rv[u]);
+                load_lane(Pp + (size_t)r * KS + cofs, pv[u]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int r = r0 + u * RPI;
+            if (r < t.row_end) {
+#pragma unroll
+                for (int q = 0; q < CPL; q++) pv[u][q] = rv[u][q] + b[q] * pv[u][q];
+                store_lane(Pp + (size_t)r * KS + cofs, pv[u]);
+            }
+        }
+    }
+}
+
+// Coefficients of a window of `count` iterations, one thread per (shift,
+// column), one CTA per panel.  With A_i = a_{s,i} + b_{s,i} A_{i+1} (A = 0
+// after the last) and B_i = b_{s,i} B_{i+1} (B = 1 at the last):
+//   x_s  += sum_i (zeta_i A_i) r_i + (b_start A_first) p_s
+//   p_s   = sum_i (zeta_i B_i) r_i + (b_start B_first) p_s
+// All factors are non-negative, and the residuals are orthogonal, so no term
+// of x_s exceeds x_s itself.  An inactive iteration has zeta = a = b = 0.
+template <typename T>
+__global__ void __launch_bounds__(VNE_THREADS) k_cg_coefs(CgFlush<T> f, CgState st, int ks) {
+    __shared__ int s_live;
+    if (threadIdx.x == 0) s_live = f.first ? (1 << st.nshift) - 1 : 0;
+    __syncthreads();
+    const int panel = blockIdx.x;
+    for (int idx = threadIdx.x; idx < st.nshift * ks; idx += VNE_THREADS) {
+        const int s = idx / ks, c = panel * ks + idx % ks;
+        const size_t o = (size_t)s * st.K + c;
+        double A = 0.0, B = 1.0;
+        bool live = false;
+        for (int i = f.count - 1; i >= 0; i--) {
+            const size_t h = ((size_t)i * st.nshift + s) * st.K + c;
+            const double z = st.hz[h], a = st.ha[h], b = st.hb[h];
+            live = live || z != 0.0 || a != 0.0;
+            A = fma(b, A, a);
+            if (i != f.count - 1) B *= b;
+            T* out = f.coef + ((size_t)i * st.nshift + s) * 2 * st.K + c;
+            out[0] = (T)(z * A);
+            out[st.K] = (T)(z * B);
+        }
+        const double bs = st.bstart[o];
+        T* out = f.coef_p + (size_t)s * 2 * st.K + c;
+        out[0] = (T)(bs * A);
+        out[st.K] = (T)(bs * B);
+        st.bstart[o] = st.hb[((size_t)(f.count - 1) * st.nshift + s) * st.K + c];
+        if (live) atomicOr(&s_live, 1 << s);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) f.live[panel] = s_live;
+}
+
+// x_s and p_s of the live shifts from a window of residuals: four shifts at a
+// time in registers, two rows per lane (a coefficient read from shared memory
+// serves both), every residual of the window read once per four live shifts.
+// Bound by HBM: (count + 4 per live shift) vectors.
+constexpr int kFlushShifts = 4;
+constexpr int kFlushRows = 1024;  // rows per CTA
+
+template <typename T, int KS>
+__global__ void __launch_bounds__(VNE_THREADS) k_cg_flush(CgFlush<T> f) {
+    constexpr int CPL = LaneVec<T>::CPL;
+    constexpr int LPR = KS / CPL;
+    constexpr int RPI = VNE_THREADS / LPR;
+    constexpr int G = kFlushShifts;
+    extern __shared__ __align__(16) unsigned char fl_smem[];
+    T* cf = reinterpret_cast<T*>(fl_smem);       // [count][G][2][KS]
+    __shared__ __align__(16) T cp[G][2][KS];
+    const int chunks = (f.n + kFlushRows - 1) / kFlushRows;
+    const int panel = blockIdx.x / chunks, chunk = blockIdx.x % chunks;
+    const int r_begin = chunk * kFlushRows, r_end = min(f.n, r_begin + kFlushRows);
+    const int sub = threadIdx.x % LPR, rs = threadIdx.x / LPR, cofs = sub * CPL;
+    const size_t pofs = (size_t)panel * f.n * KS;
+    unsigned live = (unsigned)f.live[panel];
+    while (live) {
+        int sh[G], ns = 0;
+#pragma unroll
+        for (int g = 0; g < G; g++) {
+            sh[g] = -1;
+            if (live) {
+                sh[g] = __ffs(live) - 1;
+                live &= live - 1;
+                ns++;
+            }
+        }
+        __syncthreads();  // the previous group's coefficients are no longer read
+        for (int idx = threadIdx.x; idx < f.count * G * 2 * KS; idx += VNE_THREADS) {
+            const int cc = idx % KS, w = (idx / KS) & 1, g = (idx / (2 * KS)) % G, i = idx / (2 * KS * G);
+            const int s = sh[g];
+            cf[idx] = s >= 0 ? f.coef[(((size_t)i * f.nshift + s) * 2 + w) * f.K + panel * KS + cc] : (T)0;
+        }
+        for (int idx = threadIdx.x; idx < G * 2 * KS; idx += VNE_THREADS) {
+            const int cc = idx % KS, w = (idx / KS) & 1, g = idx / (2 * KS);
+            cp[g][w][cc] = sh[g] >= 0 ? f.coef_p[((size_t)sh[g] * 2 + w) * f.K + panel * KS + cc] : (T)0;
+        }
+        __syncthreads();
+        for (int r0 = r_begin + rs; r0 < r_end; r0 += 2 * RPI) {
+            const bool two = r0 + RPI < r_end;
+            const size_t o0 = pofs + (size_t)r0 * KS + cofs, o1 = two ? o0 + (size_t)RPI * KS : o0;
+            T x[G][2][CPL], p[G][2][CPL];
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                if (g < ns && !f.first) {
+                    load_lane_stream(f.x[sh[g]] + o0, x[g][0]);
+                    load_lane_stream(f.x[sh[g]] + o1, x[g][1]);
+                    load_lane_stream(f.ps[sh[g]] + o0, p[g][0]);
+                    load_lane_stream(f.ps[sh[g]] + o1, p[g][1]);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 2; u++)
+#pragma unroll
+                        for (int q = 0; q < CPL; q++) x[g][u][q] = p[g][u][q] = (T)0;
+                }
+#pragma unroll
+                for (int u = 0; u < 2; u++)
+#pragma unroll
+                    for (int q = 0; q < CPL; q++) {
+                        x[g][u][q] += cp[g][0][cofs + q] * p[g][u][q];
+                        p[g][u][q] *= cp[g][1][cofs + q];
+                    }
+            }
+            int slot = f.slot0;
+#pragma unroll 2
+            for (int i = 0; i < f.count; i++) {
+                T a[2][CPL];
+                load_lane_stream(f.r + (size_t)slot * f.slot_stride + o0, a[0]);
+                load_lane_stream(f.r + (size_t)slot * f.slot_stride + o1, a[1]);
+                if (++slot == f.slots) slot = 0;
+                const T* ci = cf + (size_t)i * G * 2 * KS + cofs;
+#pragma unroll
+                for (int g = 0; g < G; g++) {
+                    if (g < ns) {
+                        T cx[CPL], cq[CPL];
+                        load_lane(ci + (g * 2) * KS, cx);
+                        load_lane(ci + (g * 2 + 1) * KS, cq);
+#pragma unroll
+                        for (int u = 0; u < 2; u++)
+#pragma unroll
+                            for (int q = 0; q < CPL; q++) {
+                                x[g][u][q] += cx[q] * a[u][q];
+                                p[g][u][q] += cq[q] * a[u][q];
+                            }
+                    }
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < G; g++)
+                if (g < ns) {
+                    store_lane_stream(f.x[sh[g]] + o0, x[g][0]);
+                    if (two) store_lane_stream(f.x[sh[g]] + o1, x[g][1]);
+                    if (!f.last) {
+                        store_lane_stream(f.ps[sh[g]] + o0, p[g][0]);
+                        if (two) store_lane_stream(f.ps[sh[g]] + o1, p[g][1]);
+                    }
+                }
+        }
     }
 }
 
@@ -592,15 +734,6 @@ __global__ void k_gram_mirror(const double* uniq, int nb, int K, double* full) {
 
 // ---------------------------------------------------------------------------
 
-cudaError_t launch_cg_scalars_a(const CgState& st, cudaStream_t s) {
-    k_cg_scalars_a<<<(st.K + 63) / 64, 64, 0, s>>>(st);
-    return cudaGetLastError();
-}
-cudaError_t launch_cg_scalars_b(const CgState& st, cudaStream_t s) {
-    k_cg_scalars_b<<<(st.K + 63) / 64, 64, 0, s>>>(st);
-    return cudaGetLastError();
-}
-
 #define VNE_KS_SWITCH(T, ks, CALL)                                        \
     do {                                                                  \
         if ((ks) == 4) { constexpr int KS = 4; CALL; }                    \
@@ -611,9 +744,30 @@ cudaError_t launch_cg_scalars_b(const CgState& st, cudaStream_t s) {
     } while (0)
 
 template <typename T>
-cudaError_t launch_cg_update(const CgVectors<T>& v, const CgState& st, int ks, int panels, cudaStream_t s) {
-    VNE_KS_SWITCH(T, ks, (k_cg_update<T, KS><<<panels * v.tiles_per_panel, VNE_THREADS, 0, s>>>(v, st)));
+cudaError_t launch_cg_update(const CgVectors<T>& v, const CgState& st, int ks, int panels, int window_index,
+                             int iteration, cudaStream_t s) {
+    VNE_KS_SWITCH(T, ks, (k_cg_update<T, KS><<<panels * v.tiles_per_panel, VNE_THREADS, 0, s>>>(v, st, window_index,
+                                                                                                iteration)));
     return cudaGetLastError();
+}
+template <typename T, int KS>
+cudaError_t cg_flush_ks(const CgFlush<T>& f, cudaStream_t s) {
+    const size_t smem = (size_t)f.count * kFlushShifts * 2 * KS * sizeof(T);
+    if (smem + 4096 > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_cg_flush<T, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_cg_flush<T, KS><<<f.panels * ((f.n + kFlushRows - 1) / kFlushRows), VNE_THREADS, smem, s>>>(f);
+    return cudaSuccess;
+}
+template <typename T>
+cudaError_t launch_cg_flush(const CgFlush<T>& f, const CgState& st, int ks, cudaStream_t s) {
+    if (f.count <= 0) return cudaSuccess;
+    k_cg_coefs<T><<<f.panels, VNE_THREADS, 0, s>>>(f, st, ks);
+    cudaError_t e = cudaSuccess;
+    VNE_KS_SWITCH(T, ks, (e = cg_flush_ks<T, KS>(f, s)));
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 template <typename T>
 cudaError_t launch_cg_direction(const CgVectors<T>& v, const CgState& st, int ks, int panels, cudaStream_t s) {
@@ -694,8 +848,11 @@ cudaError_t launch_block_transform(const BlockTransform<T>& bt, int ks, int pane
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template cudaError_t launch_cg_update<float>(const CgVectors<float>&, const CgState&, int, int, cudaStream_t);
-template cudaError_t launch_cg_update<double>(const CgVectors<double>&, const CgState&, int, int, cudaStream_t);
+template cudaError_t launch_cg_update<float>(const CgVectors<float>&, const CgState&, int, int, int, int, cudaStream_t);
+template cudaError_t launch_cg_update<double>(const CgVectors<double>&, const CgState&, int, int, int, int,
+                                              cudaStream_t);
+template cudaError_t launch_cg_flush<float>(const CgFlush<float>&, const CgState&, int, cudaStream_t);
+template cudaError_t launch_cg_flush<double>(const CgFlush<double>&, const CgState&, int, cudaStream_t);
 template cudaError_t launch_cg_direction<float>(const CgVectors<float>&, const CgState&, int, int, cudaStream_t);
 template cudaError_t launch_cg_direction<double>(const CgVectors<double>&, const CgState&, int, int, cudaStream_t);
 template cudaError_t launch_block_transform<float>(const BlockTransform<float>&, int, int, cudaStream_t);

@@ -57,31 +57,41 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
         sp.counter = ws_get_t<uint32_t>(ctx, "counter", (size_t)panels, true);
         VNE_TRY_CUDA(ctx, launch_start<T>(sp, ks, panels, st));
     }
-    // CG vectors
+    // CG vectors.  Residuals go to a ring of window + 1 slots; every `window`
+    // iterations one pass adds their combinations to the shifted iterates
+    // (rational.cu).  32 residuals make that pass's share of an iteration
+    // about one vector per 8 live shifts; fewer when 33 slots would take more
+    // than kRingBytes.  The ring lies in the buffer of the orthonormalised
+    // basis (nb vectors), which is written after the iteration.
+    constexpr size_t kRingBytes = (size_t)16 << 30;
+    const int nb_min = (mixed ? 1 : n_inf + 1) + nshift;
+    const int window = std::max({2, nb_min - 1,
+                                 (int)std::min<size_t>(32, kRingBytes / (blk * sizeof(T)))});
+    const int slots = window + 1;
+    const char* basis_tag = sizeof(T) == 8 ? "rat.V" : "rat.tw";
+    T* ring = ws_get_t<T>(ctx, basis_tag, blk * std::max(slots, nb_min));
     CgVectors<T> v{};
     v.n = n;
     v.tiles_per_panel = tiles;
     v.tiles = P.d_tiles;
-    v.r = ws_get_t<T>(ctx, "rat.r", blk);
     v.q = ws_get_t<T>(ctx, "rat.q", blk);
     v.p = ws_get_t<T>(ctx, "rat.p", blk);
     T* xs = ws_get_t<T>(ctx, "rat.x", blk * nshift);
     T* pss = ws_get_t<T>(ctx, "rat.ps", blk * nshift);
+    T *vx[8], *vps[8];
     for (int i = 0; i < nshift; i++) {
-        v.x[i] = xs + (size_t)i * blk;
-        v.ps[i] = pss + (size_t)i * blk;
+        vx[i] = xs + (size_t)i * blk;
+        vps[i] = pss + (size_t)i * blk;
     }
     v.part = ws_get_t<double>(ctx, "rat.part", (size_t)panels * tiles * ks);
     v.counter = ws_get_t<uint32_t>(ctx, "rat.counter", (size_t)panels, true);
-    VNE_TRY_CUDA(ctx, cudaMemcpyAsync(v.r, C, blk * sizeof(T), cudaMemcpyDeviceToDevice, st));
+    VNE_TRY_CUDA(ctx, cudaMemcpyAsync(ring, C, blk * sizeof(T), cudaMemcpyDeviceToDevice, st));
     VNE_TRY_CUDA(ctx, cudaMemcpyAsync(v.p, C, blk * sizeof(T), cudaMemcpyDeviceToDevice, st));
-    VNE_TRY_CUDA(ctx, cudaMemsetAsync(xs, 0, blk * nshift * sizeof(T), st));
-    for (int i = 0; i < nshift; i++)
-        VNE_TRY_CUDA(ctx, cudaMemcpyAsync(v.ps[i], C, blk * sizeof(T), cudaMemcpyDeviceToDevice, st));
     // scalar state
     CgState cs{};
     cs.K = Kp;
     cs.nshift = nshift;
+    cs.window = window;
     cs.scale = scale;
     cs.shift0 = s0;
     cs.tol = tol;
@@ -89,81 +99,139 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     cs.shift = upload(ctx, "rat.shifts", hsh);
     double* dq = ws_get_t<double>(ctx, "rat.dq", Kp);
     cs.dq = dq;
-    double* sc = ws_get_t<double>(ctx, "rat.scalars", (size_t)Kp * (7 + 6 * nshift));
+    const size_t SKp = (size_t)nshift * Kp;
+    double* sc = ws_get_t<double>(ctx, "rat.scalars", 5 * (size_t)Kp + (5 + 3 * (size_t)window) * SKp);
     cs.rho = sc;
-    cs.rho_new = sc + Kp;
-    cs.a = sc + 2 * Kp;
-    cs.b = sc + 3 * Kp;
-    cs.a_prev = sc + 4 * Kp;
-    cs.b_prev = sc + 5 * Kp;
-    cs.cnorm = sc + 6 * Kp;
-    double* sh = sc + 7 * Kp;
+    cs.b = sc + Kp;
+    cs.a_prev = sc + 2 * Kp;
+    cs.b_prev = sc + 3 * Kp;
+    cs.cnorm = sc + 4 * Kp;
+    double* sh = sc + 5 * Kp;
     cs.zeta = sh;
-    cs.zeta_prev = sh + (size_t)nshift * Kp;
-    cs.zeta_next = sh + 2 * (size_t)nshift * Kp;
-    cs.as = sh + 3 * (size_t)nshift * Kp;
-    cs.bs = sh + 4 * (size_t)nshift * Kp;
-    cs.resid = sh + 5 * (size_t)nshift * Kp;
-    int32_t* ibuf = ws_get_t<int32_t>(ctx, "rat.ints", (size_t)2 * nshift * Kp + 1);
+    cs.zeta_prev = sh + SKp;
+    cs.zeta_next = sh + 2 * SKp;
+    cs.resid = sh + 3 * SKp;
+    cs.bstart = sh + 4 * SKp;
+    cs.hz = sh + 5 * SKp;
+    cs.ha = cs.hz + window * SKp;
+    cs.hb = cs.ha + window * SKp;
+    int32_t* ibuf = ws_get_t<int32_t>(ctx, "rat.ints", 2 * SKp + 2 * panels);
     cs.active = ibuf;
-    cs.iters = ibuf + (size_t)nshift * Kp;
-    cs.any_active = ibuf + 2 * (size_t)nshift * Kp;
-    VNE_TRY_CUDA(ctx, launch_cg_init(cs, norm2, st));
-    ctx->launches += 1;
+    cs.iters = ibuf + SKp;
+    cs.any_active = ibuf + 2 * SKp;
     double* ah = mixed ? ws_get_t<double>(ctx, "rat.ahist", (size_t)kMixMax * Kp) : nullptr;
     double* bh = mixed ? ws_get_t<double>(ctx, "rat.bhist", (size_t)kMixMax * Kp) : nullptr;
+    cs.ah = ah;
+    cs.bh = bh;
+    cs.hist_rows = mixed ? kMixMax : 0;
+    VNE_TRY_CUDA(ctx, launch_cg_init(cs, norm2, st));
+    ctx->launches += 1;
+    CgFlush<T> fl{};
+    fl.n = n;
+    fl.K = Kp;
+    fl.nshift = nshift;
+    fl.panels = panels;
+    fl.r = ring;
+    fl.slot_stride = blk;
+    fl.slots = slots;
+    for (int i = 0; i < nshift; i++) {
+        fl.x[i] = vx[i];
+        fl.ps[i] = vps[i];
+    }
+    fl.coef = ws_get_t<T>(ctx, "rat.coef", 2 * (size_t)window * SKp);
+    fl.coef_p = ws_get_t<T>(ctx, "rat.coefp", 2 * SKp);
+    fl.live = cs.any_active + panels;
+    const OpConsts op_s0 = op_consts(ctx, P, Kp, s0, "rat.op"), op_a = op_consts(ctx, P, Kp, 0.0, "rat.op0");
     T* rh = mixed ? ws_get_t<T>(ctx, "rat.rhist", blk * (kMixMax - 1)) : nullptr;  // r_1 .. r_{kMixMax-1}
-    int it = 0;
-    for (; it < max_iter; it++) {
-        apply_operator<T>(ctx, P, ks, Kp, v.p, v.q, s0, dq, variant, "rat.op");
-        VNE_TRY_CUDA(ctx, launch_cg_scalars_a(cs, st));
-        if (mixed && it < kMixMax)
-            VNE_TRY_CUDA(ctx, cudaMemcpyAsync(ah + (size_t)it * Kp, cs.a, Kp * sizeof(double),
-                                              cudaMemcpyDeviceToDevice, st));
+    // the panels' activity flags arrive in pinned memory four iterations after
+    // the copy is issued, so that the stream does not run dry while the host
+    // looks at them
+    int32_t* any_host = (int32_t*)pinned_bytes(ctx, "rat.any", panels * sizeof(int32_t));
+    VNE_REQUIRE(ctx, any_host, VNE_ENOMEM, "pinned allocation failed");
+    struct Event {
+        cudaEvent_t e = nullptr;
+        ~Event() {
+            if (e) cudaEventDestroy(e);
+        }
+    } any_ev;
+    VNE_TRY_CUDA(ctx, cudaEventCreateWithFlags(&any_ev.e, cudaEventDisableTiming));
+    auto ask = [&]() {
+        VNE_TRY_CUDA(ctx, cudaMemcpyAsync(any_host, cs.any_active, panels * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                                          st));
+        VNE_TRY_CUDA(ctx, cudaEventRecord(any_ev.e, st));
+    };
+    auto finished = [&]() {
+        VNE_TRY_CUDA(ctx, cudaEventSynchronize(any_ev.e));
+        for (int i = 0; i < panels; i++)
+            if (any_host[i]) return false;
+        return true;
+    };
+    const double vec = (double)n * K * sizeof(T);
+    int it = 0, flushed = 0;
+    auto flush = [&](bool last) {
+        fl.count = it - flushed;
+        fl.first = flushed == 0;
+        fl.last = last;
+        fl.slot0 = flushed % slots;
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        if (ctx->profile) {
+            e0 = ctx_event(ctx);
+            VNE_TRY_CUDA(ctx, cudaEventRecord(e0, st));
+        }
+        VNE_TRY_CUDA(ctx, launch_cg_flush<T>(fl, cs, ks, st));
+        ctx->launches += 2;
+        if (ctx->profile) {
+            e1 = ctx_event(ctx);
+            VNE_TRY_CUDA(ctx, cudaEventRecord(e1, st));
+            // the window's residuals; the shifts' x_s and p_s are added after
+            // the loop from the iterations each shift stayed active
+            ctx->pending.push_back({2, e0, e1, vec * fl.count});
+        }
+        flushed = it;
+    };
+    for (;;) {
+        v.r = ring + (size_t)(it % slots) * blk;
+        v.r_next = ring + (size_t)((it + 1) % slots) * blk;
+        apply_operator<T>(ctx, P, ks, Kp, v.p, v.q, op_s0, dq, variant);
         cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr, e3 = nullptr;
         if (ctx->profile) {
             e0 = ctx_event(ctx);
             VNE_TRY_CUDA(ctx, cudaEventRecord(e0, st));
         }
-        VNE_TRY_CUDA(ctx, launch_cg_update<T>(v, cs, ks, panels, st));
+        VNE_TRY_CUDA(ctx, launch_cg_update<T>(v, cs, ks, panels, it - flushed, it, st));
         if (ctx->profile) {
             e1 = ctx_event(ctx);
             VNE_TRY_CUDA(ctx, cudaEventRecord(e1, st));
         }
         if (mixed && it + 1 < kMixMax)
-            VNE_TRY_CUDA(ctx, cudaMemcpyAsync(rh + (size_t)it * blk, v.r, blk * sizeof(T), cudaMemcpyDeviceToDevice,
-                                              st));
-        VNE_TRY_CUDA(ctx, cudaMemsetAsync(cs.any_active, 0, sizeof(int32_t), st));
-        VNE_TRY_CUDA(ctx, launch_cg_scalars_b(cs, st));
-        if (mixed && it < kMixMax)
-            VNE_TRY_CUDA(ctx, cudaMemcpyAsync(bh + (size_t)it * Kp, cs.b, Kp * sizeof(double),
+            VNE_TRY_CUDA(ctx, cudaMemcpyAsync(rh + (size_t)it * blk, v.r_next, blk * sizeof(T),
                                               cudaMemcpyDeviceToDevice, st));
         if (ctx->profile) {
             e2 = ctx_event(ctx);
             VNE_TRY_CUDA(ctx, cudaEventRecord(e2, st));
         }
         VNE_TRY_CUDA(ctx, launch_cg_direction<T>(v, cs, ks, panels, st));
-        ctx->launches += 4;
+        ctx->launches += 2;
         if (ctx->profile) {
             e3 = ctx_event(ctx);
             VNE_TRY_CUDA(ctx, cudaEventRecord(e3, st));
-            // algorithmic bytes of the seed part: update reads r, q, writes r;
-            // direction reads r, p, writes p.  The per-shift part (update:
-            // p_s and x_s read and written) is added after the loop from the
-            // iterations each shift stayed active.
-            const double vec = (double)n * K * sizeof(T);
+            // algorithmic bytes: update reads r, q, writes r; direction reads
+            // r, p, writes p
             ctx->pending.push_back({2, e0, e1, vec * 3.0});
             ctx->pending.push_back({3, e2, e3, vec * 3.0});
         }
-        if ((it & 7) == 7 || it + 1 == max_iter) {
-            int32_t any = 0;
-            VNE_TRY_CUDA(ctx, cudaMemcpyAsync(&any, cs.any_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-            VNE_TRY_CUDA(ctx, cudaStreamSynchronize(st));
-            if (!any) {
-                it++;
-                break;
-            }
+        it++;
+        bool done = it >= max_iter;
+        // the switching rule counts the iterations of a short solve, so it
+        // looks at the flags of the iteration itself
+        const bool lagged = !(mixed && it <= kMixMax);
+        if (!done && lagged && (it & 7) == 4) ask();
+        if (!done && (it & 7) == 0) {
+            if (!lagged) ask();
+            done = finished();
         }
+        if (done || it - flushed == window) flush(done);
+        if (done) break;
     }
     // polynomial part: K_{n_inf+1}(A, c) by powers of A, or, with the
     // switching rule, K_k(A, c) by the seed residuals
@@ -213,24 +281,24 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     if (mixed) {
         for (int j = 1; j < kpoly; j++) W[j] = rh + (size_t)(j - 1) * blk;
         for (int j = 0; j < kpoly && need_aw; j++) {
-            apply_operator<T>(ctx, P, ks, Kp, W[j], apow + (size_t)j * blk, 0.0, dq, variant, "rat.op0");
+            apply_operator<T>(ctx, P, ks, Kp, W[j], apow + (size_t)j * blk, op_a, dq, variant);
             AW[j] = apow + (size_t)j * blk;
         }
     } else {
         const T* prev = C;
         for (int j = 0; j < kpoly; j++) {
             T* out = apow + (size_t)j * blk;
-            apply_operator<T>(ctx, P, ks, Kp, prev, out, 0.0, dq, variant, "rat.op0");
+            apply_operator<T>(ctx, P, ks, Kp, prev, out, op_a, dq, variant);
             prev = out;
         }
         for (int j = 1; j < kpoly; j++) W[j] = apow + (size_t)(j - 1) * blk;
         for (int j = 0; j < kpoly; j++) AW[j] = apow + (size_t)j * blk;
     }
     for (int i = 0; i < nshift && need_aw; i++)  // A x_s into the (now free) direction buffers
-        apply_operator<T>(ctx, P, ks, Kp, v.x[i], v.ps[i], 0.0, dq, variant, "rat.op0");
+        apply_operator<T>(ctx, P, ks, Kp, vx[i], vps[i], op_a, dq, variant);
     for (int i = 0; i < nshift; i++) {
-        W[kpoly + i] = v.x[i];
-        AW[kpoly + i] = v.ps[i];
+        W[kpoly + i] = vx[i];
+        AW[kpoly + i] = vps[i];
     }
     // Gram matrices of (W, A W), Cholesky-QR2: pass 1 basis change X1, then
     // the Gram matrices of (W X1, A W X1) for the final orthonormalisation.
@@ -320,7 +388,7 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
         }
         std::vector<const T*> Vv(nb), AVv(nb);
         for (int a = 0; a < nb; a++) {
-            apply_operator<T>(ctx, P, ks, Kp, V + (size_t)a * blk, AV + (size_t)a * blk, 0.0, dq, variant, "rat.op0");
+            apply_operator<T>(ctx, P, ks, Kp, V + (size_t)a * blk, AV + (size_t)a * blk, op_a, dq, variant);
             Vv[a] = V + (size_t)a * blk;
             AVv[a] = AV + (size_t)a * blk;
         }
@@ -367,11 +435,16 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     VNE_TRY_CUDA(ctx, cudaMemcpyAsync(hres.data(), cs.resid, hres.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
     VNE_TRY_CUDA(ctx, cudaStreamSynchronize(st));
     if (ctx->profile) {
-        double shift_iters = 0.0;
+        // x_s and p_s read and written in every flush of a window in which
+        // the shift was active (only written in the first)
+        double touched = 0.0;
         for (int i = 0; i < nshift; i++)
-            for (int c = 0; c < K; c++) shift_iters += hit[(size_t)i * Kp + c];
+            for (int c = 0; c < K; c++) {
+                const int w = (hit[(size_t)i * Kp + c] + window - 1) / window;
+                touched += w > 0 ? 4.0 * w - 2.0 : 0.0;
+            }
         const double per = (double)n * sizeof(T);
-        ctx->pending.push_back({2, nullptr, nullptr, shift_iters * per * 4.0});
+        ctx->pending.push_back({2, nullptr, nullptr, touched * per});
         ctx_flush_profile(ctx);
     }
     iters.assign((size_t)nshift * K, 0);
@@ -384,7 +457,6 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     int rmin = nb;
     for (int c = 0; c < K; c++) rmin = std::min(rmin, hr[c]);
     if (rank_min) *rank_min = rmin;
-    (void)it;
 }
 
 }  // namespace
