@@ -197,10 +197,13 @@ void plan_segment(const int64_t* rowptr, int32_t row_begin, int32_t rows, int32_
     sg.cta_count = (int32_t)((P.items.size() - first_item) / ((size_t)VNE_WARPS * P.ipw));
     for (int32_t c = 0; c < sg.cta_count; c++) P.cta_seg.push_back(seg);
     sg.tile_begin = (int32_t)P.tiles.size();
-    // row tiles of the streaming kernels: 4096 rows, fewer for small
-    // segments (at least 16 tiles down to 256 rows) so that their update and
-    // reorthogonalisation passes still spread over several SMs
-    const int32_t trows = std::max<int32_t>(256, std::min<int32_t>(kTileRows, ((rows / 16) + 31) & ~31));
+    // row tiles of the streaming kernels: at most 1024 rows (FP64: 4096, which
+    // the passes split further, see Problem::sub), fewer for small segments
+    // (at least 16 tiles down to 256 rows) so that the passes spread over the
+    // SMs.  At 4096 rows a block of 64 FP32 columns and 150,000 rows made 148
+    // CTAs: 46 us per update, @UPD@ with 1024
+    const int32_t cap = P.fp64 ? kTileRows : 1024;
+    const int32_t trows = std::max<int32_t>(256, std::min<int32_t>(cap, ((rows / 16) + 31) & ~31));
     for (int32_t r = row_begin; r < row_begin + rows; r += trows)
         P.tiles.push_back(RowTile{r, std::min(row_begin + rows, r + trows), seg, 0});
     sg.tile_count = (int32_t)P.tiles.size() - sg.tile_begin;
@@ -300,7 +303,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
     double* mean = ws_get_t<double>(ctx, "mean", SK);
     double* psi = ws_get_t<double>(ctx, tag + ".psi", SK);
     const int ctas = P.ctas_per_panel(), tiles = P.tiles_per_panel();
-    double* part = ws_get_t<double>(ctx, "part", (size_t)panels * std::max(ctas, tiles) * ks);
+    double* part = ws_get_t<double>(ctx, "part", (size_t)panels * std::max(ctas, tiles * P.sub()) * ks);
     uint32_t* counter = ws_get_t<uint32_t>(ctx, "counter", (size_t)panels * S, true);
     const int nh = (int)P.hubs.size();
     const int64_t nnz_total = P.nnz_total;
@@ -360,6 +363,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
     p.ipw = P.ipw;
     p.tiles = P.d_tiles;
     p.tiles_per_panel = tiles;
+    p.sub = P.sub();
     p.u = u;
     p.part = part;
     p.counter = counter;
@@ -468,6 +472,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 rp.n_total = P.n_total;
                 rp.panels = panels;
                 rp.tiles_per_panel = tiles;
+                rp.sub = P.sub();
                 rp.tiles = P.d_tiles;
                 rp.part = rpart;
                 rp.coef = rcoef;
@@ -499,6 +504,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 rp.n_total = P.n_total;
                 rp.panels = panels;
                 rp.tiles_per_panel = tiles;
+                rp.sub = P.sub();
                 rp.tiles = P.d_tiles;
                 rp.part = rpart;
                 rp.coef = rcoef;

@@ -184,6 +184,11 @@ struct Problem {
         }
         for (void* p : owned) vne_engine::dev_free(p);
     }
+    // CTAs per row tile in the update and reorthogonalisation passes: FP64 tiles
+    // keep up to 4096 rows (the conjugate gradients' order of additions), so
+    // these passes split them; a constant, so that a graph's numbers are the
+    // same alone and in a batch
+    int sub() const { return fp64 ? 4 : 1; }
     int ctas_per_panel() const { return (int)(items.size() / ((size_t)VNE_WARPS * ipw)); }
     int tiles_per_panel() const { return (int)tiles.size(); }
 };

@@ -56,6 +56,7 @@ struct StepParams {
     double* hub_dot;   // [panels][nhubs][KS]: w_j . u of each long row (added in fixed order)
     const RowTile* tiles;
     int32_t tiles_per_panel;
+    int32_t sub;        // update kernel: CTAs per row tile
     int32_t stage_nnz;  // largest work item in nonzeros (staged variants)
     int32_t ipw;        // work items per warp (a CTA covers VNE_WARPS * ipw consecutive items)
     // per-segment step counters (serving): with segj set, segment s runs its
@@ -91,6 +92,7 @@ struct ReorthParams {
     size_t slot_stride;   // elements between consecutive slots
     T* w;                 // vector being orthogonalised (slot j)
     int32_t j, K, n_total, panels, tiles_per_panel;
+    int32_t sub;          // update pass: CTAs per row tile
     const RowTile* tiles;
     double* part;         // [panels][j][tiles][KS]
     const double* coef;   // [j][K]

@@ -182,18 +182,26 @@ struct RadQuad {
 
 // Per-column totals of a CTA: each thread holds four columns' partial sums;
 // sum them over the threads of the same columns in a fixed order and write
-// the CTA's partial for the segment reduction.
-template <int KS>
-__device__ __forceinline__ void cta_column_partials(const double (&sum)[4], int rsub, int c0, double* part_out) {
-    constexpr int RPP = VNE_THREADS / (KS / 4);
-    __shared__ double red[RPP][KS];
+// the CTA's partial for the segment reduction (SERIAL: FP64 blocks, whose
+// conjugate gradients keep the order of additions).
+template <int KS, bool SERIAL>
+__device__ __forceinline__ void cta_column_partials(double (&sum)[4], int rsub, int c0, double* part_out) {
+    if (SERIAL) {
+        constexpr int RPP = VNE_THREADS / (KS / 4);
+        __shared__ double red[RPP][KS];
 #pragma unroll
-    for (int j = 0; j < 4; j++) red[rsub][c0 + j] = sum[j];
-    __syncthreads();
-    if (threadIdx.x < KS) {
-        double s = 0.0;
-        for (int q = 0; q < RPP; q++) s += red[q][threadIdx.x];
-        part_out[threadIdx.x] = s;
+        for (int j = 0; j < 4; j++) red[rsub][c0 + j] = sum[j];
+        __syncthreads();
+        if (threadIdx.x < KS) {
+            double s = 0.0;
+            for (int q = 0; q < RPP; q++) s += red[q][threadIdx.x];
+            part_out[threadIdx.x] = s;
+        }
+    } else {
+        __shared__ double red[VNE_WARPS][KS];
+        double s;
+        cta_colsum<KS, 4>(sum, red, s);
+        if (threadIdx.x < KS) part_out[threadIdx.x] = s;
     }
 }
 
@@ -265,7 +273,7 @@ __global__ void __launch_bounds__(VNE_THREADS, 4) k_start_mean(StartParams<T> p)
 #pragma unroll
         for (int j = 0; j < 4; j++) sum[j] = rs[j].total();
     }
-    cta_column_partials<KS>(sum, rsub, c0, p.part + ((size_t)panel * p.tiles_per_panel + tile) * KS);
+    cta_column_partials<KS, sizeof(T) == 8>(sum, rsub, c0, p.part + ((size_t)panel * p.tiles_per_panel + tile) * KS);
     __shared__ double tot[KS];
     if (last_cta_reduce<KS, sizeof(T) == 8>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
                             sg.tile_begin, sg.tile_count, tot)) {
@@ -377,7 +385,7 @@ __global__ void __launch_bounds__(VNE_THREADS, 3) k_start_center(StartParams<T> 
 #pragma unroll
         for (int j = 0; j < 4; j++) sum[j] = rs[j].total();
     }
-    cta_column_partials<KS>(sum, rsub, c0, p.part + ((size_t)panel * p.tiles_per_panel + tile) * KS);
+    cta_column_partials<KS, sizeof(T) == 8>(sum, rsub, c0, p.part + ((size_t)panel * p.tiles_per_panel + tile) * KS);
     __shared__ double tot[KS];
     if (last_cta_reduce<KS, sizeof(T) == 8>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
                             sg.tile_begin, sg.tile_count, tot)) {
@@ -762,41 +770,48 @@ __global__ void __launch_bounds__(VNE_THREADS, MINB) k_step(StepParams<T> p) {
     }
     }  // work items of this warp
 
-    // CTA partial of w_j . u per column: FP64 across groups, warps, CTAs
+    // CTA partial of w_j . u per column: FP64 across groups, warps, CTAs (FP64
+    // blocks in the order of the conjugate gradients, see reduce.cuh)
+    constexpr bool kSerial = sizeof(T) == 8;
     __shared__ double sred[VNE_WARPS][KS];
-    double d[CPL];
+    double d[CPL], part = 0.0;
 #pragma unroll
-    for (int q = 0; q < CPL; q++) {
-        d[q] = (double)dot[q];
+    for (int q = 0; q < CPL; q++) d[q] = (double)dot[q];
+    if (kSerial) {
 #pragma unroll
-        for (int off = LPR; off < 32; off <<= 1) d[q] += __shfl_xor_sync(0xffffffffu, d[q], off);
+        for (int q = 0; q < CPL; q++)
+#pragma unroll
+            for (int off = LPR; off < 32; off <<= 1) d[q] += __shfl_xor_sync(0xffffffffu, d[q], off);
+        if (g == 0)
+#pragma unroll
+            for (int q = 0; q < CPL; q++) sred[warp][cofs + q] = d[q];
+        __syncthreads();
+        if (threadIdx.x < KS)
+#pragma unroll
+            for (int w = 0; w < VNE_WARPS; w++) part += sred[w][threadIdx.x];
+    } else {
+        cta_colsum<KS, CPL>(d, sred, part);
     }
-    if (g == 0)
-#pragma unroll
-        for (int q = 0; q < CPL; q++) sred[warp][cofs + q] = d[q];
-    __syncthreads();
-    if (threadIdx.x < KS) {
-        double s = 0.0;
-#pragma unroll
-        for (int w = 0; w < VNE_WARPS; w++) s += sred[w][threadIdx.x];
-        p.part[((size_t)panel * p.ctas_per_panel + cta) * KS + threadIdx.x] = s;
-    }
+    if (threadIdx.x < KS) p.part[((size_t)panel * p.ctas_per_panel + cta) * KS + threadIdx.x] = part;
     __shared__ double tot[KS];
     const SegInfo sg = p.seg[seg];
-    if (last_cta_reduce<KS, sizeof(T) == 8>(p.part, p.counter + (size_t)panel * p.nseg + seg, panel, p.ctas_per_panel,
-                            sg.cta_begin, sg.cta_count, tot)) {
+    if (last_cta_reduce<KS, kSerial>(p.part, p.counter + (size_t)panel * p.nseg + seg, panel, p.ctas_per_panel,
+                                     sg.cta_begin, sg.cta_count, tot)) {
         // add the long rows' shares in a fixed order (strided over the CTA)
         __shared__ double hred[VNE_THREADS];
         constexpr int NS = VNE_THREADS / KS;
-        const int c = threadIdx.x % KS, s = threadIdx.x / KS;
-        double hacc = 0.0;
-        for (int h = s; h < sg.hub_count; h += NS)
-            hacc += ld_cg(&p.hub_dot[((size_t)panel * p.nhubs + sg.hub_begin + h) * KS + c]);
-        hred[threadIdx.x] = hacc;
-        __syncthreads();
+        if (sg.hub_count > 0) {
+            const int c = threadIdx.x % KS, s = threadIdx.x / KS;
+            double hacc = 0.0;
+            for (int h = s; h < sg.hub_count; h += NS)
+                hacc += ld_cg(&p.hub_dot[((size_t)panel * p.nhubs + sg.hub_begin + h) * KS + c]);
+            hred[threadIdx.x] = hacc;
+            __syncthreads();
+        }
         if (threadIdx.x < KS) {
             double t = tot[threadIdx.x];
-            for (int q = 0; q < NS; q++) t += hred[q * KS + threadIdx.x];
+            if (sg.hub_count > 0)
+                for (int q = 0; q < NS; q++) t += hred[q * KS + threadIdx.x];
             size_t o = (size_t)seg * p.K + panel * KS + threadIdx.x;
             sv.alpha[o] = sv.sig_cur[o] * t;
         }
@@ -815,9 +830,9 @@ __global__ void __launch_bounds__(VNE_THREADS) k_update(StepParams<T> p) {
     // panels in reverse order: the step kernel walked them forwards, so the
     // first panels updated are the ones it touched last (still partly in L2),
     // and the next step starts on the panel updated last
-    const int np = gridDim.x / p.tiles_per_panel;
-    const int panel = p.panel_base + (np - 1 - (int)(blockIdx.x / p.tiles_per_panel)),
-              tile = blockIdx.x % p.tiles_per_panel;
+    const int per = p.tiles_per_panel * p.sub, np = gridDim.x / per;
+    const int panel = p.panel_base + (np - 1 - (int)(blockIdx.x / per));
+    const int tile = (int)(blockIdx.x % per) / p.sub, piece = (int)(blockIdx.x % per) % p.sub;
     if (p.renorm && p.panel_active && !p.panel_active[panel]) return;  // nothing changed in this panel
     const RowTile t = p.tiles[tile];
     StepView<T> sv;
@@ -825,43 +840,71 @@ __global__ void __launch_bounds__(VNE_THREADS) k_update(StepParams<T> p) {
     const int sub = threadIdx.x % LPR, rsub = threadIdx.x / LPR;
     const int cofs = sub * CPL;
     const size_t pofs = (size_t)panel * p.n_total * KS;
-    const size_t so = (size_t)t.seg * p.K + panel * KS + cofs;
+    const int len = ((t.row_end - t.row_begin) + p.sub - 1) / p.sub;
+    const int r_begin = t.row_begin + piece * len, r_end = min(t.row_end, r_begin + len);
+    // alpha_j sigma_j once per column (an FP64 product per lane would take an
+    // FP64 port for CPL x 64 cycles per warp)
+    __shared__ T s_a[KS];
+    if (threadIdx.x < KS) {
+        const size_t o = (size_t)t.seg * p.K + panel * KS + threadIdx.x;
+        s_a[threadIdx.x] = p.renorm ? (T)0 : (T)(sv.alpha[o] * sv.sig_cur[o]);
+    }
+    __syncthreads();
     T a[CPL], nrm[CPL];
 #pragma unroll
     for (int q = 0; q < CPL; q++) {
-        a[q] = p.renorm ? (T)0 : (T)(sv.alpha[so + q] * sv.sig_cur[so + q]);
+        a[q] = s_a[cofs + q];
         nrm[q] = (T)0;
     }
     const T* __restrict__ Uu = p.u + pofs;
     const T* __restrict__ W = sv.w_cur + pofs;
     T* __restrict__ Wn = sv.w_next + pofs;
-    for (int r = t.row_begin + rsub; r < t.row_end; r += RPI) {
-        T uu[CPL], x[CPL], wn[CPL];
+    constexpr int U = 4;  // rows in flight per lane
+    for (int r0 = r_begin + rsub; r0 < r_end; r0 += U * RPI) {
+        T wn[U][CPL];
         if (p.renorm) {
-            load_lane(Wn + (size_t)r * KS + cofs, wn);
-        } else {
-            load_lane_stream(Uu + (size_t)r * KS + cofs, uu);
-            load_lane(W + (size_t)r * KS + cofs, x);
 #pragma unroll
-            for (int q = 0; q < CPL; q++) wn[q] = uu[q] - a[q] * x[q];
-            store_lane(Wn + (size_t)r * KS + cofs, wn);
+            for (int u = 0; u < U; u++) {
+                const int r = r0 + u * RPI;
+                if (r < r_end) load_lane(Wn + (size_t)r * KS + cofs, wn[u]);
+            }
+        } else {
+            T x[U][CPL];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int r = r0 + u * RPI;
+                if (r < r_end) {
+                    load_lane_stream(Uu + (size_t)r * KS + cofs, wn[u]);
+                    load_lane(W + (size_t)r * KS + cofs, x[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int r = r0 + u * RPI;
+                if (r < r_end) {
+#pragma unroll
+                    for (int q = 0; q < CPL; q++) wn[u][q] -= a[q] * x[u][q];
+                    store_lane(Wn + (size_t)r * KS + cofs, wn[u]);
+                }
+            }
         }
 #pragma unroll
-        for (int q = 0; q < CPL; q++) nrm[q] += wn[q] * wn[q];
-    }
-    __shared__ double red[VNE_THREADS / LPR][KS];
+        for (int u = 0; u < U; u++)
+            if (r0 + u * RPI < r_end)
 #pragma unroll
-    for (int q = 0; q < CPL; q++) red[rsub][cofs + q] = (double)nrm[q];
-    __syncthreads();
-    if (threadIdx.x < KS) {
-        double s = 0.0;
-        for (int i = 0; i < RPI; i++) s += red[i][threadIdx.x];
-        p.part[((size_t)panel * p.tiles_per_panel + tile) * KS + threadIdx.x] = s;
+                for (int q = 0; q < CPL; q++) nrm[q] += wn[u][q] * wn[u][q];
     }
+    __shared__ double red[VNE_WARPS][KS];
+    double nd[CPL], part;
+#pragma unroll
+    for (int q = 0; q < CPL; q++) nd[q] = (double)nrm[q];
+    cta_colsum<KS, CPL>(nd, red, part);
+    if (threadIdx.x < KS)
+        p.part[(((size_t)panel * p.tiles_per_panel + tile) * p.sub + piece) * KS + threadIdx.x] = part;
     __shared__ double tot[KS];
     const SegInfo sg = p.seg[t.seg];
-    if (last_cta_reduce<KS, sizeof(T) == 8>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel,
-                            sg.tile_begin, sg.tile_count, tot)) {
+    if (last_cta_reduce<KS>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel * p.sub,
+                            sg.tile_begin * p.sub, sg.tile_count * p.sub, tot)) {
         if (threadIdx.x < KS) {
             size_t o = (size_t)t.seg * p.K + panel * KS + threadIdx.x;
             double b = sqrt(tot[threadIdx.x]);
@@ -1048,7 +1091,8 @@ template <typename T, int KS>
 __global__ void __launch_bounds__(VNE_THREADS) k_reorth_apply(ReorthParams<T> p) {
     constexpr int V = Chunk16<T>::V, G = KS / V, U = 4;
     static_assert(KS % V == 0 && VNE_THREADS % G == 0, "chunk layout");
-    const int panel = blockIdx.x / p.tiles_per_panel, tile = blockIdx.x % p.tiles_per_panel;
+    const int per = p.tiles_per_panel * p.sub;
+    const int panel = blockIdx.x / per, tile = (int)(blockIdx.x % per) / p.sub, piece = (int)(blockIdx.x % per) % p.sub;
     if (p.panel_active && !p.panel_active[panel]) return;
     __shared__ int16_t act[kReorthMaxJ];
     __shared__ T cf[kReorthMaxJ * KS];
@@ -1075,10 +1119,12 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_apply(ReorthParams<T> p)
     __syncthreads();
     if (na == 0) return;
     const RowTile t = p.tiles[tile];
-    const size_t base = (size_t)panel * p.n_total * KS + (size_t)t.row_begin * KS;
+    const int len = ((t.row_end - t.row_begin) + p.sub - 1) / p.sub;
+    const int r_begin = t.row_begin + piece * len, r_end = min(t.row_end, r_begin + len);
+    const size_t base = (size_t)panel * p.n_total * KS + (size_t)r_begin * KS;
     T* Wn = p.w + base;
     const T* B = p.basis + base;
-    const int nchunks = (t.row_end - t.row_begin) * G;
+    const int nchunks = max(r_end - r_begin, 0) * G;
     const int g = threadIdx.x % G;
     if constexpr (sizeof(T) == 8) {
         // full groups of U chunks, then the remaining chunks one at a time (a
@@ -1378,7 +1424,7 @@ cudaError_t launch_step(const StepParams<T>& p, int ks, int panels, bool valued,
 
 template <typename T>
 cudaError_t launch_update(const StepParams<T>& p, int ks, int panels, cudaStream_t st) {
-    dim3 grid(panels * p.tiles_per_panel);
+    dim3 grid(panels * p.tiles_per_panel * p.sub);
     VNE_DISPATCH_KS(T, ks, (k_update<T, KS><<<grid, VNE_THREADS, 0, st>>>(p)));
     return cudaGetLastError();
 }
@@ -1402,7 +1448,7 @@ cudaError_t launch_step_update_segj(const StepParams<T>& p, int ks, int panels, 
     if (!p.segj) return cudaErrorInvalidValue;
     const size_t smem = (size_t)VNE_WARPS * (p.stage_nnz + kStageRp) * sizeof(int32_t);
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
-    dim3 gs(panels * p.ctas_per_panel), gu(panels * p.tiles_per_panel);
+    dim3 gs(panels * p.ctas_per_panel), gu(panels * p.tiles_per_panel * p.sub);
     VNE_DISPATCH_KS(T, ks, (k_step<T, KS, false, 4, 8, true, true, 0, true, true><<<gs, VNE_THREADS, smem, st>>>(p)));
     VNE_DISPATCH_KS(T, ks, (k_update<T, KS, true><<<gu, VNE_THREADS, 0, st>>>(p)));
     return cudaGetLastError();
@@ -1415,7 +1461,7 @@ cudaError_t launch_reorth(const ReorthParams<T>& p, const ReorthCoefParams& c, i
     VNE_DISPATCH_KS(T, ks, (k_reorth_dots<T, KS><<<dim3(p.panels * p.tiles_per_panel * p.j), VNE_THREADS, 0, st>>>(p)));
     int total = c.panels * c.j * ks;
     VNE_DISPATCH_KS(T, ks, (k_reorth_coef<KS><<<dim3((total + 255) / 256), 256, 0, st>>>(c)));
-    VNE_DISPATCH_KS(T, ks, (k_reorth_apply<T, KS><<<dim3(p.panels * p.tiles_per_panel), VNE_THREADS, 0, st>>>(p)));
+    VNE_DISPATCH_KS(T, ks, (k_reorth_apply<T, KS><<<dim3(p.panels * p.tiles_per_panel * p.sub), VNE_THREADS, 0, st>>>(p)));
     return cudaGetLastError();
 }
 

@@ -352,6 +352,7 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
         rp.n_total = n;
         rp.panels = panels;
         rp.tiles_per_panel = tiles;
+        rp.sub = P.sub();
         rp.tiles = P.d_tiles;
         rp.part = cpart;
         rp.coef = coef;

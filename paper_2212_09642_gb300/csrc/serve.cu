@@ -595,8 +595,9 @@ int tick_impl(vne_server* S) {
     p.ipw = 1;
     p.tiles = P.d_tiles;
     p.tiles_per_panel = (int32_t)tile_high;
+    p.sub = P.sub();
     p.u = (T*)S->u;
-    p.part = ws_get_t<double>(ctx, "srv.step_part", (size_t)panels * std::max(cta_high, tile_high) * ks);
+    p.part = ws_get_t<double>(ctx, "srv.step_part", (size_t)panels * std::max(cta_high, tile_high * P.sub()) * ks);
     p.counter = ws_get_t<uint32_t>(ctx, "srv.step_counter", (size_t)panels * P.nseg);
     p.segj = (const int32_t*)dptr(i_sj);
     p.slot0 = (T*)S->slot0;
