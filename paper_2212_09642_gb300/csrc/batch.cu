@@ -29,9 +29,9 @@ extern "C" vne_status vne_batch_hutchinson(vne_matrix* const* mats, int32_t coun
     VNE_REQUIRE(ctx, !any_valued, VNE_EUNSUPPORTED, "batched mode packs pattern (graph) matrices");
     VNE_REQUIRE(ctx, ntot < INT32_MAX && nnztot < INT32_MAX, VNE_EINVAL, "packed batch too large");
     double taurel = o.breakdown_tol > 0 ? o.breakdown_tol : default_tau(fp64);
-    const int target = default_item_nnz(&o);
     std::vector<uint64_t> key;
-    key.push_back((uint64_t)target);
+    key.push_back((uint64_t)o.item_nnz);
+    key.push_back((uint64_t)o.items_per_warp);
     uint64_t tbits = 0;
     memcpy(&tbits, &taurel, sizeof(tbits));
     key.push_back(tbits);
@@ -53,6 +53,16 @@ extern "C" vne_status vne_batch_hutchinson(vne_matrix* const* mats, int32_t coun
         P->n_total = (int32_t)ntot;
         P->nnz_total = nnztot;
         P->nseg = count;
+        // every graph takes its own schedule (items by its own size), so that
+        // its numbers are those of the graph alone
+        std::vector<std::pair<int, int>> sched(count);  // item nonzeros, items per warp
+        for (int i = 0; i < count; i++) {
+            default_items(fp64, mats[i]->nnz, &sched[i].first, &sched[i].second);
+            if (o.item_nnz > 0) sched[i].first = o.item_nnz;
+            if (o.items_per_warp == 1 || o.items_per_warp == 2 || o.items_per_warp == 4)
+                sched[i].second = o.items_per_warp;
+            P->ipw = std::max(P->ipw, sched[i].second);
+        }
         int64_t r0 = 0, e0 = 0;
         for (int i = 0; i < count; i++) {
             vne_matrix* M = mats[i];
@@ -71,7 +81,8 @@ extern "C" vne_status vne_batch_hutchinson(vne_matrix* const* mats, int32_t coun
             r0 += M->n;
             e0 += M->nnz;
         }
-        for (int i = 0; i < count; i++) plan_segment(rp.data(), P->segs[i].row_begin, P->segs[i].rows, i, target, *P);
+        for (int i = 0; i < count; i++)
+            plan_segment(rp.data(), P->segs[i].row_begin, P->segs[i].rows, i, sched[i].first, sched[i].second, *P);
         std::vector<int32_t> rp32(ntot + 1);
         for (int64_t i = 0; i <= ntot; i++) rp32[i] = (int32_t)rp[i];
         int32_t* drp = dev_copy(ctx, rp32);
@@ -96,7 +107,7 @@ extern "C" vne_status vne_batch_hutchinson(vne_matrix* const* mats, int32_t coun
     }
     Problem* P = ctx->batch_prob;
     const int ks = ctx->batch_ks;
-    const int variant = fp64 ? 0 : (o.step_variant >= 0 ? o.step_variant : 4);
+    const int variant = fp64 ? 0 : (o.step_variant >= 0 ? o.step_variant : kDefaultVariant);
     StartSource s{};
     s.kind = SRC_RADEMACHER;
     s.gaussian = o.gaussian_probes != 0;

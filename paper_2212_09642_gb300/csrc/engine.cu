@@ -148,7 +148,10 @@ extern const int kTileRows = 4096;
 // Work items of one segment (rows [row_begin, row_begin + rows) of the packed
 // CSR): runs of short rows with about `target` nonzeros (at most 64 rows),
 // and rows longer than `long_thresh` split into chunks of `chunk` nonzeros.
-void plan_segment(const int64_t* rowptr, int32_t row_begin, int32_t rows, int32_t seg, int target, Problem& P) {
+// A segment takes seg_ipw <= P.ipw items per warp: the rest of its CTAs' item
+// slots stay empty, so its sums are those of the segment alone.
+void plan_segment(const int64_t* rowptr, int32_t row_begin, int32_t rows, int32_t seg, int target, int seg_ipw,
+                  Problem& P) {
     // every item holds at most `target` nonzeros: short rows are packed into
     // runs (at most 64 rows), rows longer than `target` are split into chunks
     const int64_t chunk = std::max(target, 32);
@@ -188,7 +191,16 @@ void plan_segment(const int64_t* rowptr, int32_t row_begin, int32_t rows, int32_
         blk_nnz += deg;
     }
     flush();
-    while ((P.items.size() - first_item) % ((size_t)VNE_WARPS * P.ipw)) P.items.push_back(WorkItem{0, 0, 0, 0});
+    while ((P.items.size() - first_item) % ((size_t)VNE_WARPS * seg_ipw)) P.items.push_back(WorkItem{0, 0, 0, 0});
+    if (seg_ipw < P.ipw) {
+        const size_t have = (size_t)VNE_WARPS * seg_ipw, room = (size_t)VNE_WARPS * P.ipw;
+        const std::vector<WorkItem> real(P.items.begin() + first_item, P.items.end());
+        P.items.resize(first_item);
+        for (size_t i = 0; i < real.size(); i += have) {
+            P.items.insert(P.items.end(), real.begin() + i, real.begin() + i + have);
+            P.items.resize(P.items.size() + (room - have), WorkItem{0, 0, 0, 0});
+        }
+    }
     for (size_t i = first_item; i < P.items.size(); i++)
         P.stage_nnz = std::max<int32_t>(P.stage_nnz, P.items[i].nnz_end - P.items[i].nnz_begin);
     SegInfo& sg = P.segs[seg];
@@ -201,7 +213,7 @@ void plan_segment(const int64_t* rowptr, int32_t row_begin, int32_t rows, int32_
     // the passes split further, see Problem::sub), fewer for small segments
     // (at least 16 tiles down to 256 rows) so that the passes spread over the
     // SMs.  At 4096 rows a block of 64 FP32 columns and 150,000 rows made 148
-    // CTAs: 46 us per update, @UPD@ with 1024
+    // CTAs: 46 us per update, 17 with 1024
     const int32_t cap = P.fp64 ? kTileRows : 1024;
     const int32_t trows = std::max<int32_t>(256, std::min<int32_t>(cap, ((rows / 16) + 31) & ~31));
     for (int32_t r = row_begin; r < row_begin + rows; r += trows)
@@ -220,16 +232,41 @@ void problem_upload(vne_ctx* ctx, Problem& P) {
 
 double default_tau(bool fp64) { return fp64 ? 1e-13 : 1e-10; }
 
-int default_item_nnz(const vne_options* o) { return (o && o->item_nnz > 0) ? o->item_nnz : 256; }
+// Built-in schedule of an FP32 matrix that was not autotuned.  Variant 10
+// (four CTAs per SM, eight gathers in flight, staged indices, predicated tails)
+// was the fastest at every size of a sweep (five variants x panel widths x item
+// sizes); the item size follows the nonzeros, so that a small matrix still
+// makes a CTA per SM and a large one pays the CTA's reduction tail rarely.
+// Hutchinson estimates, ms, with the former constants (variant 4, 256
+// nonzeros, one item per warp) and with these:
+//   nnz     5,600 x  5 columns x 20 steps   0.436  0.349   (64)
+//          24,000 x 64 x 40                 0.993  0.719   (64)
+//         160,000 x 64 x 40                 1.66   1.31    (128; 1.52 with 256)
+//       1,600,000 x 100 x 30                5.39   4.89    (512)
+//       8,000,000 x 112 x 20                17.9   14.6    (512, two per warp)
+// FP64 matrices keep 256 nonzeros per item (the order of additions of their
+// conjugate gradients).
+void default_items(bool fp64, int64_t nnz, int* item, int* ipw) {
+    *item = fp64 || (nnz >= 200000 && nnz < 400000) ? 256 : (nnz < 32000 ? 64 : (nnz < 200000 ? 128 : 512));
+    *ipw = fp64 || nnz < 4000000 ? 1 : 2;
+}
 
-
-Sched resolve_sched(const vne_matrix* M, const vne_options* o) {
+Sched resolve_sched(const vne_matrix* M, const vne_options* o, int block_cols) {
     Sched s;
+    int item, ipw;
+    default_items(M->fp64, M->nnz, &item, &ipw);
     s.ks = (o && o->panel > 0) ? o->panel : (M->tuned ? M->tuned_panel : choose_panel(M->fp64, o, M->n));
-    s.item_nnz = (o && o->item_nnz > 0) ? o->item_nnz : (M->tuned ? M->tuned_item_nnz : 256);
-    s.variant = (o && o->step_variant >= 0) ? o->step_variant : (M->tuned ? M->tuned_variant : 4);
+    // a block that is never split by the caller (colour classes, rational
+    // forms) takes panels of 8 where 16 would pad it by 30 % or more: 22 colour
+    // classes of an RGG of 10^6 nodes, 24 columns instead of 32, 4.48 -> 3.72 ms
+    // per 20 steps
+    if (block_cols > 0 && !(o && o->panel > 0) && !M->tuned && !M->fp64 && s.ks == 16 &&
+        10 * ((block_cols + 15) / 16 * 16) >= 13 * ((block_cols + 7) / 8 * 8))
+        s.ks = 8;
+    s.item_nnz = (o && o->item_nnz > 0) ? o->item_nnz : (M->tuned ? M->tuned_item_nnz : item);
+    s.variant = (o && o->step_variant >= 0) ? o->step_variant : (M->tuned ? M->tuned_variant : kDefaultVariant);
     if (M->fp64) s.variant = 0;
-    s.ipw = (o && o->items_per_warp > 0) ? o->items_per_warp : (M->tuned ? M->tuned_ipw : 1);
+    s.ipw = (o && o->items_per_warp > 0) ? o->items_per_warp : (M->tuned ? M->tuned_ipw : ipw);
     s.interleave = (o && o->interleave >= 0) ? (o->interleave != 0) : (M->tuned ? M->tuned_interleave : false);
     s.graph = !(o && o->graphs == 0);
     return s;
@@ -261,7 +298,7 @@ Problem* matrix_problem(vne_matrix* M, const vne_options* opt) {
     s.scale = M->scale;
     s.tau = taurel * M->normM;
     P->segs.push_back(s);
-    plan_segment(M->h_rowptr.data(), 0, (int32_t)M->n, 0, target, *P);
+    plan_segment(M->h_rowptr.data(), 0, (int32_t)M->n, 0, target, sc.ipw, *P);
     problem_upload(M->ctx, *P);
     M->prob = P.release();
     M->prob_item_nnz = target;
@@ -653,10 +690,10 @@ std::vector<double> quadforms(vne_matrix* M, const vne_options* o, StartSource s
                               const double* abs_tol) {
     vne_ctx* ctx = M->ctx;
     Problem* P = matrix_problem(M, o);
-    Sched sc = resolve_sched(M, o);
+    int lim = block_limit(o);
+    Sched sc = resolve_sched(M, o, src.kind == SRC_INDICATOR ? std::min(lim, ncols) : 0);
     int ks = sc.ks;
     check_ks<T>(ctx, ks);
-    int lim = block_limit(o);
     const int reorth = want_reorth(M, o);
     std::vector<double> psi(ncols);
     ctx->last_steps = 0;

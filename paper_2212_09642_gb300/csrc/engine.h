@@ -267,7 +267,8 @@ uint64_t seed_mix(uint64_t seed);
 
 extern const int kTileRows;
 // Work items and row tiles of one segment of a packed CSR.
-void plan_segment(const int64_t* rowptr, int32_t row_begin, int32_t rows, int32_t seg, int target, Problem& P);
+void plan_segment(const int64_t* rowptr, int32_t row_begin, int32_t rows, int32_t seg, int target, int seg_ipw,
+                  Problem& P);
 
 // Device copy of a host vector, owned by the caller (dev_free).
 template <typename T>
@@ -282,7 +283,8 @@ T* dev_copy(vne_ctx* ctx, const std::vector<T>& v) {
 
 void problem_upload(vne_ctx* ctx, Problem& P);
 double default_tau(bool fp64);
-int default_item_nnz(const vne_options* o);
+constexpr int kDefaultVariant = 10;  // step-kernel variant of an FP32 matrix that was not autotuned
+void default_items(bool fp64, int64_t nnz, int* item, int* ipw);
 
 struct Sched {
     int ks, item_nnz, variant, ipw;
@@ -293,7 +295,9 @@ struct Sched {
 int choose_panel(bool fp64, const vne_options* opt, int64_t n);
 // Schedule for a call: explicit options win, then the matrix's autotuned
 // choice, then the built-in defaults.
-Sched resolve_sched(const vne_matrix* M, const vne_options* o);
+// block_cols > 0: the columns of a block whose split the caller does not see
+// (its panel width may then follow them).
+Sched resolve_sched(const vne_matrix* M, const vne_options* o, int block_cols = 0);
 Problem* matrix_problem(vne_matrix* M, const vne_options* opt);
 
 struct BlockOut {

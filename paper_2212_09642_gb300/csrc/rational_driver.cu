@@ -469,9 +469,9 @@ void rational_quadforms(vne_matrix* M, const vne_options* o, StartSource src, in
                         int nshift, std::vector<double>& psi, std::vector<int>& iters, std::vector<double>& resid) {
     vne_ctx* ctx = M->ctx;
     Problem* P = matrix_problem(M, o);
-    Sched sc = resolve_sched(M, o);
-    check_ks<T>(ctx, sc.ks);
     const int lim = std::min(block_limit(o), 128);
+    Sched sc = resolve_sched(M, o, std::min(lim, ncols));
+    check_ks<T>(ctx, sc.ks);
     const double tol = (o && o->cg_tol > 0) ? o->cg_tol : 1e-8;
     const int maxit = (o && o->cg_max_iter > 0) ? o->cg_max_iter : 10000;
     const int n_inf = o ? o->n_inf_poles : 2;
