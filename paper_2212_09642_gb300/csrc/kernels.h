@@ -230,6 +230,9 @@ struct CgState {
 template <typename T>
 struct CgVectors {
     int32_t n, tiles_per_panel;
+    int32_t sub;            // direction kernel: CTAs per row tile
+    int32_t max_tile_rows;  // rows of the largest tile
+    int32_t sm_count;
     const RowTile* tiles;
     const T* r;  // residual r_k
     T* r_next;   // r_{k+1}: the next slot of the residual window
@@ -242,6 +245,7 @@ struct CgVectors {
 template <typename T>
 struct CgFlush {
     int32_t n, K, nshift, panels;
+    int32_t rows;         // rows per CTA (set by the launcher)
     int32_t count;        // residuals in the window (<= CgState::window)
     int32_t first, last;  // first flush: x and p_s start from zero; last: p_s is not needed any more
     const T* r;           // residual slots, [slots][K / ks][n][ks]

@@ -1372,7 +1372,7 @@ static int panel_width_ok(int ks) {
 
 #define VNE_DISPATCH_KS(T, ks, CALL)                                   \
     do {                                                               \
-        if (sizeof(T) == 4) {                                          \
+        if constexpr (sizeof(T) == 4) {                                \
             if ((ks) == 8) { constexpr int KS = 8; CALL; }             \
             else if ((ks) == 16) { constexpr int KS = 16; CALL; }      \
             else if ((ks) == 32) { constexpr int KS = 32; CALL; }      \
@@ -1393,32 +1393,43 @@ cudaError_t launch_start(const StartParams<T>& p, int ks, int panels, cudaStream
     return cudaGetLastError();
 }
 
-// Step-kernel variants: {MINB, UNR, STREAM, STAGE, HINT, PTAIL}.  FP64 uses variant 0 only.
-#define VNE_STEP_VARIANTS(T, KS, VALUED, v, st, grid, p, smem)                                                   \
-    switch (sizeof(T) == 8 ? 0 : (v)) {                                                                          \
-        case 1: k_step<T, KS, VALUED, 6, 4, true, false><<<grid, VNE_THREADS, 0, st>>>(p); break;               \
-        case 2: k_step<T, KS, VALUED, 6, 8, true, false><<<grid, VNE_THREADS, 0, st>>>(p); break;               \
-        case 3: k_step<T, KS, VALUED, 8, 4, true, false><<<grid, VNE_THREADS, 0, st>>>(p); break;               \
-        case 4: k_step<T, KS, VALUED, 6, 4, true, true><<<grid, VNE_THREADS, smem, st>>>(p); break;             \
-        case 5: k_step<T, KS, VALUED, 4, 8, true, true><<<grid, VNE_THREADS, smem, st>>>(p); break;             \
-        case 6: k_step<T, KS, VALUED, 6, 4, true, true, 1><<<grid, VNE_THREADS, smem, st>>>(p); break;          \
-        case 7: k_step<T, KS, VALUED, 6, 4, true, true, 2><<<grid, VNE_THREADS, smem, st>>>(p); break;          \
-        case 8: k_step<T, KS, VALUED, 6, 8, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;    \
-        case 9: k_step<T, KS, VALUED, 6, 4, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;    \
-        case 10: k_step<T, KS, VALUED, 4, 8, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;   \
-        case 11: k_step<T, KS, VALUED, 6, 8, true, false, 0, true><<<grid, VNE_THREADS, 0, st>>>(p); break;     \
-        case 12: k_step<T, KS, VALUED, 5, 4, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;   \
-        case 13: k_step<T, KS, VALUED, 5, 8, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;   \
-        default: k_step<T, KS, VALUED, 4, 4, false, false><<<grid, VNE_THREADS, 0, st>>>(p); break;             \
+// Step-kernel variants: {MINB, UNR, STREAM, STAGE, HINT, PTAIL}.  FP64 has one,
+// plain loads and loops: its additions bind it (an FP64 port takes 64 cycles
+// per warp instruction, and a warp pays for its longest row), so predicated
+// tails and more gathers in flight measured slower (n = 30,000, 16 columns: 36
+// us against 41; weighted entries, n = 60,000, 40 columns: 80 against 94).
+template <int KS, bool VALUED>
+void step_variant(const StepParams<double>& p, int, dim3 grid, size_t, cudaStream_t st) {
+    k_step<double, KS, VALUED, 4, 4, false, false><<<grid, VNE_THREADS, 0, st>>>(p);
+}
+template <int KS, bool VALUED>
+void step_variant(const StepParams<float>& p, int v, dim3 grid, size_t smem, cudaStream_t st) {
+    typedef float T;
+    switch (v) {
+        case 1: k_step<T, KS, VALUED, 6, 4, true, false><<<grid, VNE_THREADS, 0, st>>>(p); break;
+        case 2: k_step<T, KS, VALUED, 6, 8, true, false><<<grid, VNE_THREADS, 0, st>>>(p); break;
+        case 3: k_step<T, KS, VALUED, 8, 4, true, false><<<grid, VNE_THREADS, 0, st>>>(p); break;
+        case 4: k_step<T, KS, VALUED, 6, 4, true, true><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        case 5: k_step<T, KS, VALUED, 4, 8, true, true><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        case 6: k_step<T, KS, VALUED, 6, 4, true, true, 1><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        case 7: k_step<T, KS, VALUED, 6, 4, true, true, 2><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        case 8: k_step<T, KS, VALUED, 6, 8, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        case 9: k_step<T, KS, VALUED, 6, 4, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        case 10: k_step<T, KS, VALUED, 4, 8, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        case 11: k_step<T, KS, VALUED, 6, 8, true, false, 0, true><<<grid, VNE_THREADS, 0, st>>>(p); break;
+        case 12: k_step<T, KS, VALUED, 5, 4, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        case 13: k_step<T, KS, VALUED, 5, 8, true, true, 0, true><<<grid, VNE_THREADS, smem, st>>>(p); break;
+        default: k_step<T, KS, VALUED, 4, 4, false, false><<<grid, VNE_THREADS, 0, st>>>(p); break;
     }
+}
 
 template <typename T>
 cudaError_t launch_step(const StepParams<T>& p, int ks, int panels, bool valued, int variant, cudaStream_t st) {
     dim3 grid(panels * p.ctas_per_panel);
     const size_t smem = (size_t)VNE_WARPS * (p.stage_nnz + kStageRp) * sizeof(int32_t);
     if (smem > 48 * 1024) return cudaErrorInvalidValue;  // items above 1024 nonzeros are not staged
-    if (valued) VNE_DISPATCH_KS(T, ks, VNE_STEP_VARIANTS(T, KS, true, variant, st, grid, p, smem));
-    else VNE_DISPATCH_KS(T, ks, VNE_STEP_VARIANTS(T, KS, false, variant, st, grid, p, smem));
+    if (valued) VNE_DISPATCH_KS(T, ks, (step_variant<KS, true>(p, variant, grid, smem, st)));
+    else VNE_DISPATCH_KS(T, ks, (step_variant<KS, false>(p, variant, grid, smem, st)));
     return cudaGetLastError();
 }
 
@@ -1449,7 +1460,8 @@ cudaError_t launch_step_update_segj(const StepParams<T>& p, int ks, int panels, 
     const size_t smem = (size_t)VNE_WARPS * (p.stage_nnz + kStageRp) * sizeof(int32_t);
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
     dim3 gs(panels * p.ctas_per_panel), gu(panels * p.tiles_per_panel * p.sub);
-    VNE_DISPATCH_KS(T, ks, (k_step<T, KS, false, 4, 8, true, true, 0, true, true><<<gs, VNE_THREADS, smem, st>>>(p)));
+    constexpr int MINB = sizeof(T) == 8 ? 3 : 4;  // CTAs per SM without register spills
+    VNE_DISPATCH_KS(T, ks, (k_step<T, KS, false, MINB, 8, true, true, 0, true, true><<<gs, VNE_THREADS, smem, st>>>(p)));
     VNE_DISPATCH_KS(T, ks, (k_update<T, KS, true><<<gu, VNE_THREADS, 0, st>>>(p)));
     return cudaGetLastError();
 }

@@ -42,6 +42,7 @@
 // rounding error no longer grows with the square of the basis condition
 // number), projects A, diagonalises the small matrix by cyclic Jacobi and
 // returns psi = ||c||^2 e1^T f(A_m) e1.
+#include <cooperative_groups.h>
 #include <float.h>
 #include <math.h>
 
@@ -92,14 +93,27 @@ cudaError_t launch_cg_init(CgState st, const double* norm2, cudaStream_t s) {
 // vectors.  The last CTA of a panel advances the panel's scalars, one thread
 // per (shift, column): two single-warp kernels did that before, 19 us per
 // iteration of dependent FP64 arithmetic that this tail spreads over a CTA.
-template <typename T, int KS>
+// CLUSTER (FP64, few tiles): a thread-block cluster takes a tile, each CTA one
+// run of 16 rows per thread, and CTA 0 adds the runs from distributed shared
+// memory in the order in which one CTA would have added them (n = 30,000, 16
+// columns: 32 tiles of 1888 rows, 23 us on 32 SMs; 18.6 in clusters of
+// two).
+template <typename T, int KS, bool CLUSTER>
 __global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgState st, int wi, int it) {
+    namespace cg = cooperative_groups;
+    const int csize = CLUSTER ? (int)cg::this_cluster().num_blocks() : 1;
+    const int crank = CLUSTER ? (int)cg::this_cluster().block_rank() : 0;
+    const int cta = (int)blockIdx.x / csize;
     constexpr int CPL = LaneVec<T>::CPL;
     constexpr int LPR = KS / CPL;            // lanes per row
     constexpr int RPI = VNE_THREADS / LPR;   // rows per iteration
     constexpr int U = 4;
-    const int panel = blockIdx.x / v.tiles_per_panel, tile = blockIdx.x % v.tiles_per_panel;
-    const RowTile t = v.tiles[tile];
+    const int panel = cta / v.tiles_per_panel, tile = cta % v.tiles_per_panel;
+    RowTile t = v.tiles[tile];
+    if (CLUSTER) {  // run crank of the tile
+        t.row_begin += crank * 16 * RPI;
+        t.row_end = min(t.row_end, t.row_begin + 16 * RPI);
+    }
     const int sub = threadIdx.x % LPR, rs = threadIdx.x / LPR;
     const int cofs = sub * CPL;
     const size_t pofs = (size_t)panel * v.n * KS;
@@ -157,6 +171,21 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgSta
     }
 #pragma unroll
     for (int q = 0; q < CPL; q++) acc[q] += (double)accf[q];
+    if (CLUSTER) {
+        __shared__ double runs[CPL][VNE_THREADS];
+#pragma unroll
+        for (int q = 0; q < CPL; q++) runs[q][threadIdx.x] = acc[q];
+        auto cl = cg::this_cluster();
+        cl.sync();
+        if (crank == 0)
+            for (int k = 1; k < csize; k++) {
+                const double* other = cl.map_shared_rank(&runs[0][0], k);
+#pragma unroll
+                for (int q = 0; q < CPL; q++) acc[q] += other[q * VNE_THREADS + threadIdx.x];
+            }
+        cl.sync();  // CTA 0 has read the runs
+        if (crank != 0) return;
+    }
     constexpr bool kSerial = sizeof(T) == 8;
     __shared__ double red[kSerial ? RPI : VNE_WARPS][KS];
     double tot;
@@ -241,8 +270,11 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_direction(CgVectors<T> v, Cg
     constexpr int LPR = KS / CPL;
     constexpr int RPI = VNE_THREADS / LPR;
     constexpr int U = 4;
-    const int panel = blockIdx.x / v.tiles_per_panel, tile = blockIdx.x % v.tiles_per_panel;
+    const int per = v.tiles_per_panel * v.sub;
+    const int panel = blockIdx.x / per, tile = (int)(blockIdx.x % per) / v.sub, piece = (int)(blockIdx.x % per) % v.sub;
     const RowTile t = v.tiles[tile];
+    const int len = ((t.row_end - t.row_begin) + v.sub - 1) / v.sub;
+    const int r_begin = t.row_begin + piece * len, r_end = min(t.row_end, r_begin + len);
     const int sub = threadIdx.x % LPR, rs = threadIdx.x / LPR;
     const int cofs = sub * CPL;
     const size_t pofs = (size_t)panel * v.n * KS;
@@ -251,12 +283,12 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_direction(CgVectors<T> v, Cg
     for (int q = 0; q < CPL; q++) b[q] = (T)st.b[panel * KS + cofs + q];
     const T* __restrict__ R = v.r_next + pofs;
     T* __restrict__ Pp = v.p + pofs;
-    for (int r0 = t.row_begin + rs; r0 < t.row_end; r0 += U * RPI) {
+    for (int r0 = r_begin + rs; r0 < r_end; r0 += U * RPI) {
         T rv[U][CPL], pv[U][CPL];
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const int r = r0 + u * RPI;
-            if (r < t.row_end) {
+            if (r < r_end) {
                 load_lane(R + (size_t)r * KS + cofs, rv[u]);
                 load_lane(Pp + (size_t)r * KS + cofs, pv[u]);
             }
@@ -264,7 +296,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_direction(CgVectors<T> v, Cg
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const int r = r0 + u * RPI;
-            if (r < t.row_end) {
+            if (r < r_end) {
 #pragma unroll
                 for (int q = 0; q < CPL; q++) pv[u][q] = rv[u][q] + b[q] * pv[u][q];
                 store_lane(Pp + (size_t)r * KS + cofs, pv[u]);
@@ -315,9 +347,9 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_coefs(CgFlush<T> f, CgState 
 // x_s and p_s of the live shifts from a window of residuals: four shifts at a
 // time in registers, two rows per lane (a coefficient read from shared memory
 // serves both), every residual of the window read once per four live shifts.
-// Bound by HBM: (count + 4 per live shift) vectors.
+// Bound by HBM: (count + 4 per live shift) vectors; FP64 by its multiply-adds
+// (two per element, residual and live shift).
 constexpr int kFlushShifts = 4;
-constexpr int kFlushRows = 1024;  // rows per CTA
 
 template <typename T, int KS>
 __global__ void __launch_bounds__(VNE_THREADS) k_cg_flush(CgFlush<T> f) {
@@ -328,9 +360,9 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_flush(CgFlush<T> f) {
     extern __shared__ __align__(16) unsigned char fl_smem[];
     T* cf = reinterpret_cast<T*>(fl_smem);       // [count][G][2][KS]
     __shared__ __align__(16) T cp[G][2][KS];
-    const int chunks = (f.n + kFlushRows - 1) / kFlushRows;
+    const int chunks = (f.n + f.rows - 1) / f.rows;
     const int panel = blockIdx.x / chunks, chunk = blockIdx.x % chunks;
-    const int r_begin = chunk * kFlushRows, r_end = min(f.n, r_begin + kFlushRows);
+    const int r_begin = chunk * f.rows, r_end = min(f.n, r_begin + f.rows);
     const int sub = threadIdx.x % LPR, rs = threadIdx.x / LPR, cofs = sub * CPL;
     const size_t pofs = (size_t)panel * f.n * KS;
     unsigned live = (unsigned)f.live[panel];
@@ -472,87 +504,159 @@ __global__ void k_rational_pass1(const double* Mg, int nb, int K, double drop, d
 }
 
 // Pass 2: orthonormalise the transformed basis, project A, diagonalise by
-// cyclic Jacobi, psi = ||c||^2 sum_k z_{1k}^2 f(mu_k).  c2 = ||c||^2.
-__global__ void k_rational_pass2(const double* Mg, const double* Kg, const double* c2v, int nb, int K, double drop,
-                                 double* psi, int* rank_out) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= K) return;
-    const double c2 = c2v[(size_t)0 * K + c];
-    double R[kMaxBasis][kMaxBasis], D[kMaxBasis];
-    int keep[kMaxBasis];
+// Jacobi, psi = ||c||^2 sum_k z_{1k}^2 f(mu_k).  c2 = ||c||^2.  A warp per
+// column with the matrices in shared memory (one thread per column before, its
+// arrays in local memory: 2.8 ms for 12 columns of 11 vectors, 0.34 now):
+// lanes share the rows of the triangular solves and products, and a Jacobi
+// sweep takes its rotations in rounds of disjoint pairs (the circle method), a
+// lane per rotation angle, since the angle's divisions and square roots are
+// what a rotation costs.
+__global__ void __launch_bounds__(32) k_rational_pass2(const double* Mg, const double* Kg, const double* c2v, int nb,
+                                                       int K, double drop, double* psi, int* rank_out) {
+    constexpr int N = kMaxBasis, LD = kMaxBasis + 1;
+    __shared__ double R[N * LD], Ri[N * LD], T1[N * LD], Am[N * LD], Z[N * LD];
+    __shared__ double D[N], s_c[N / 2], s_s[N / 2];
+    __shared__ int keep[N], s_p[N / 2], s_q[N / 2];
+    const int c = blockIdx.x, lane = threadIdx.x;
+    const double c2 = c2v[c];
     if (!(c2 > 0.0)) {
-        psi[c] = 0.0;
-        rank_out[c] = 0;
+        if (lane == 0) {
+            psi[c] = 0.0;
+            rank_out[c] = 0;
+        }
         return;
     }
-    const int r = gram_cholesky(Mg, nb, K, c, drop, R, D, keep);
-    double Ri[kMaxBasis][kMaxBasis];
-    for (int j = 0; j < r; j++) {
-        for (int i = 0; i < r; i++) Ri[i][j] = 0.0;
-        Ri[j][j] = 1.0 / R[j][j];
-        for (int i = j - 1; i >= 0; i--) {
+    if (lane < nb) {
+        const double maa = Mg[((size_t)lane * nb + lane) * K + c];
+        D[lane] = maa > 0.0 ? 1.0 / sqrt(maa) : 0.0;
+    }
+    __syncwarp();
+    // Cholesky of the column-scaled Gram in basis order (gram_cholesky's rule):
+    // lane i holds entry i of the new column
+    int r = 0;
+    for (int a = 0; a < nb; a++) {
+        if (D[a] == 0.0) continue;
+        double v = lane < r ? Mg[((size_t)keep[lane] * nb + a) * K + c] * D[keep[lane]] * D[a] : 0.0;
+        double s = 1.0;
+        for (int i = 0; i < r; i++) {
+            const double ci = __shfl_sync(0xffffffffu, v, i) / R[i * LD + i];
+            if (lane == i) v = ci;
+            if (lane > i && lane < r) v -= R[i * LD + lane] * ci;
+            s -= ci * ci;
+        }
+        if (s <= drop) continue;
+        if (lane < r) R[lane * LD + r] = v;
+        if (lane == 0) {
+            R[r * LD + r] = sqrt(s);
+            keep[r] = a;
+        }
+        r++;
+        __syncwarp();
+    }
+    // R^{-1}, a lane per column
+    if (lane < r) {
+        for (int i = 0; i < r; i++) Ri[i * LD + lane] = 0.0;
+        Ri[lane * LD + lane] = 1.0 / R[lane * LD + lane];
+        for (int i = lane - 1; i >= 0; i--) {
             double v = 0.0;
-            for (int l = i + 1; l <= j; l++) v += R[i][l] * Ri[l][j];
-            Ri[i][j] = -v / R[i][i];
+            for (int l = i + 1; l <= lane; l++) v += R[i * LD + l] * Ri[l * LD + lane];
+            Ri[i * LD + lane] = -v / R[i * LD + i];
         }
     }
-    // A_m = Ri^T Kt Ri with Kt the scaled, symmetrised W^T A W on kept columns
-    double T1[kMaxBasis][kMaxBasis], Am[kMaxBasis][kMaxBasis];
-    for (int i = 0; i < r; i++)
-        for (int j = 0; j < r; j++) {
-            double v = 0.0;
-            for (int l = 0; l <= j; l++) {
-                const int a = keep[i], b = keep[l];
-                const double kab = 0.5 * (Kg[((size_t)a * nb + b) * K + c] + Kg[((size_t)b * nb + a) * K + c]);
-                v += kab * D[a] * D[b] * Ri[l][j];
-            }
-            T1[i][j] = v;
-        }
-    for (int i = 0; i < r; i++)
-        for (int j = 0; j < r; j++) {
-            double v = 0.0;
-            for (int l = 0; l <= i; l++) v += Ri[l][i] * T1[l][j];
-            Am[i][j] = v;
-        }
-    double Z[kMaxBasis][kMaxBasis];
-    for (int i = 0; i < r; i++)
-        for (int j = 0; j < r; j++) Z[i][j] = (i == j) ? 1.0 : 0.0;
+    __syncwarp();
+    // the scaled, symmetrised W^T A W on kept columns (in Z for now)
+    for (int idx = lane; idx < r * r; idx += 32) {
+        const int i = idx / r, l = idx % r, a = keep[i], b = keep[l];
+        const double kab = 0.5 * (Kg[((size_t)a * nb + b) * K + c] + Kg[((size_t)b * nb + a) * K + c]);
+        Z[i * LD + l] = kab * D[a] * D[b];
+    }
+    __syncwarp();
+    for (int idx = lane; idx < r * r; idx += 32) {
+        const int i = idx / r, j = idx % r;
+        double v = 0.0;
+        for (int l = 0; l <= j; l++) v += Z[i * LD + l] * Ri[l * LD + j];
+        T1[i * LD + j] = v;
+    }
+    __syncwarp();
+    for (int idx = lane; idx < r * r; idx += 32) {
+        const int i = idx / r, j = idx % r;
+        double v = 0.0;
+        for (int l = 0; l <= i; l++) v += Ri[l * LD + i] * T1[l * LD + j];
+        Am[i * LD + j] = v;
+        Z[i * LD + j] = (i == j) ? 1.0 : 0.0;
+    }
+    __syncwarp();
+    const int r2 = (r + 1) & ~1, half = r2 / 2;  // players of the circle method (an odd r sits one out)
     for (int sweep = 0; sweep < 30; sweep++) {
         double off = 0.0, tot = 0.0;
-        for (int i = 0; i < r; i++)
-            for (int j = 0; j < r; j++) {
-                tot += Am[i][j] * Am[i][j];
-                if (i != j) off += Am[i][j] * Am[i][j];
-            }
+        for (int idx = lane; idx < r * r; idx += 32) {
+            const double x = Am[(idx / r) * LD + idx % r];
+            tot += x * x;
+            if (idx / r != idx % r) off += x * x;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        }
         if (off <= 1e-30 * tot) break;
-        for (int p = 0; p < r; p++)
-            for (int q = p + 1; q < r; q++) {
-                double apq = Am[p][q];
-                if (apq == 0.0) continue;
-                double theta = (Am[q][q] - Am[p][p]) / (2.0 * apq);
-                double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                double cs = 1.0 / sqrt(t * t + 1.0), sn = t * cs;
-                for (int k = 0; k < r; k++) {
-                    double akp = Am[k][p], akq = Am[k][q];
-                    Am[k][p] = cs * akp - sn * akq;
-                    Am[k][q] = sn * akp + cs * akq;
+        for (int round = 0; round < r2 - 1; round++) {
+            if (lane < half) {
+                const int m = r2 - 1;
+                int p = lane == 0 ? m : (round + lane) % m;
+                int q = lane == 0 ? round : (round + m - lane) % m;
+                if (p > q) {
+                    const int x = p;
+                    p = q;
+                    q = x;
                 }
-                for (int k = 0; k < r; k++) {
-                    double apk = Am[p][k], aqk = Am[q][k];
-                    Am[p][k] = cs * apk - sn * aqk;
-                    Am[q][k] = sn * apk + cs * aqk;
+                double cs = 1.0, sn = 0.0;
+                if (q < r) {
+                    const double apq = Am[p * LD + q];
+                    if (apq != 0.0) {
+                        const double theta = (Am[q * LD + q] - Am[p * LD + p]) / (2.0 * apq);
+                        const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+                        cs = 1.0 / sqrt(t * t + 1.0);
+                        sn = t * cs;
+                    }
                 }
-                for (int k = 0; k < r; k++) {
-                    double zkp = Z[k][p], zkq = Z[k][q];
-                    Z[k][p] = cs * zkp - sn * zkq;
-                    Z[k][q] = sn * zkp + cs * zkq;
-                }
+                s_c[lane] = cs;
+                s_s[lane] = sn;
+                s_p[lane] = p;
+                s_q[lane] = q;
             }
+            __syncwarp();
+            for (int idx = lane; idx < r * half; idx += 32) {  // columns of A and Z
+                const int k = idx / half, h = idx % half, p = s_p[h], q = s_q[h];
+                if (q >= r) continue;
+                const double cs = s_c[h], sn = s_s[h];
+                const double akp = Am[k * LD + p], akq = Am[k * LD + q];
+                Am[k * LD + p] = cs * akp - sn * akq;
+                Am[k * LD + q] = sn * akp + cs * akq;
+                const double zkp = Z[k * LD + p], zkq = Z[k * LD + q];
+                Z[k * LD + p] = cs * zkp - sn * zkq;
+                Z[k * LD + q] = sn * zkp + cs * zkq;
+            }
+            __syncwarp();
+            for (int idx = lane; idx < r * half; idx += 32) {  // rows of A
+                const int k = idx % r, h = idx / r, p = s_p[h], q = s_q[h];
+                if (q >= r) continue;
+                const double cs = s_c[h], sn = s_s[h];
+                const double apk = Am[p * LD + k], aqk = Am[q * LD + k];
+                Am[p * LD + k] = cs * apk - sn * aqk;
+                Am[q * LD + k] = sn * apk + cs * aqk;
+            }
+            __syncwarp();
+        }
     }
     double s = 0.0;
-    for (int k = 0; k < r; k++) s += Z[0][k] * Z[0][k] * f_ent(Am[k][k]);
-    psi[c] = c2 * s;
-    rank_out[c] = r;
+    if (lane < r) s = Z[lane] * Z[lane] * f_ent(Am[lane * LD + lane]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+        psi[c] = c2 * s;
+        rank_out[c] = r;
+    }
 }
 
 template <typename T, int KS>
@@ -743,22 +847,52 @@ __global__ void k_gram_mirror(const double* uniq, int nb, int K, double* full) {
         else return cudaErrorInvalidValue;                                \
     } while (0)
 
+template <typename T, int KS>
+cudaError_t cg_update_ks(const CgVectors<T>& v, const CgState& st, int panels, int wi, int it, cudaStream_t s) {
+    constexpr int RPI = VNE_THREADS / (KS / LaneVec<T>::CPL);
+    const int ctas = panels * v.tiles_per_panel;
+    if constexpr (sizeof(T) == 8) {
+        // runs of 16 rows per thread in the largest tile; clusters pay while
+        // the tiles alone do not fill the SMs twice
+        const int runs = (v.max_tile_rows + 16 * RPI - 1) / (16 * RPI);
+        if (runs > 1 && runs <= 8 && ctas < 2 * v.sm_count) {
+            int size = 1;
+            while (size < runs) size *= 2;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(ctas * size);
+            cfg.blockDim = dim3(VNE_THREADS);
+            cfg.stream = s;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = size;
+            at[0].val.clusterDim.y = 1;
+            at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            return cudaLaunchKernelEx(&cfg, k_cg_update<T, KS, true>, v, st, wi, it);
+        }
+    }
+    k_cg_update<T, KS, false><<<ctas, VNE_THREADS, 0, s>>>(v, st, wi, it);
+    return cudaSuccess;
+}
 template <typename T>
 cudaError_t launch_cg_update(const CgVectors<T>& v, const CgState& st, int ks, int panels, int window_index,
                              int iteration, cudaStream_t s) {
-    VNE_KS_SWITCH(T, ks, (k_cg_update<T, KS><<<panels * v.tiles_per_panel, VNE_THREADS, 0, s>>>(v, st, window_index,
-                                                                                                iteration)));
-    return cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    VNE_KS_SWITCH(T, ks, (e = cg_update_ks<T, KS>(v, st, panels, window_index, iteration, s)));
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 template <typename T, int KS>
-cudaError_t cg_flush_ks(const CgFlush<T>& f, cudaStream_t s) {
+cudaError_t cg_flush_ks(CgFlush<T> f, cudaStream_t s) {
+    // 1024 rows per CTA, 256 while that leaves SMs without one
+    f.rows = (int64_t)f.panels * f.n >= 1024 * 608 ? 1024 : 256;
     const size_t smem = (size_t)f.count * kFlushShifts * 2 * KS * sizeof(T);
     if (smem + 4096 > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_cg_flush<T, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_cg_flush<T, KS><<<f.panels * ((f.n + kFlushRows - 1) / kFlushRows), VNE_THREADS, smem, s>>>(f);
+    k_cg_flush<T, KS><<<f.panels * ((f.n + f.rows - 1) / f.rows), VNE_THREADS, smem, s>>>(f);
     return cudaSuccess;
 }
 template <typename T>
@@ -771,7 +905,7 @@ cudaError_t launch_cg_flush(const CgFlush<T>& f, const CgState& st, int ks, cuda
 }
 template <typename T>
 cudaError_t launch_cg_direction(const CgVectors<T>& v, const CgState& st, int ks, int panels, cudaStream_t s) {
-    VNE_KS_SWITCH(T, ks, (k_cg_direction<T, KS><<<panels * v.tiles_per_panel, VNE_THREADS, 0, s>>>(v, st)));
+    VNE_KS_SWITCH(T, ks, (k_cg_direction<T, KS><<<panels * v.tiles_per_panel * v.sub, VNE_THREADS, 0, s>>>(v, st)));
     return cudaGetLastError();
 }
 template <typename T, int KS>
@@ -823,7 +957,7 @@ cudaError_t launch_rational_pass1(const double* M, int nb, int K, double drop, d
 cudaError_t launch_rational_pass2(const double* M, const double* Kmat, const double* c2, int nb, int K, double drop,
                                   double* psi, int* rank, cudaStream_t s) {
     if (nb > kMaxBasis) return cudaErrorInvalidValue;
-    k_rational_pass2<<<(K + 31) / 32, 32, 0, s>>>(M, Kmat, c2, nb, K, drop, psi, rank);
+    k_rational_pass2<<<K, 32, 0, s>>>(M, Kmat, c2, nb, K, drop, psi, rank);
     return cudaGetLastError();
 }
 // the basis-change matrix (nb^2 x KS values) lives in dynamic shared memory,

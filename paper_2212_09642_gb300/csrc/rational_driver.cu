@@ -74,6 +74,9 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     v.n = n;
     v.tiles_per_panel = tiles;
     v.tiles = P.d_tiles;
+    v.sub = P.sub();
+    for (const RowTile& t : P.tiles) v.max_tile_rows = std::max(v.max_tile_rows, t.row_end - t.row_begin);
+    v.sm_count = ctx->sm_count;
     v.q = ws_get_t<T>(ctx, "rat.q", blk);
     v.p = ws_get_t<T>(ctx, "rat.p", blk);
     T* xs = ws_get_t<T>(ctx, "rat.x", blk * nshift);
