@@ -50,6 +50,11 @@ extern "C" vne_status vne_ctx_destroy(vne_ctx* ctx) {
         if (e) cudaEventDestroy(e);
     for (auto& kv : ctx->graphs) cudaGraphExecDestroy(kv.second.exec);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
+    for (int g = 0; g + 1 < vne_ctx::kMaxGroups; g++) {
+        if (ctx->aux[g]) cudaStreamDestroy(ctx->aux[g]);
+        if (ctx->join_ev[g]) cudaEventDestroy(ctx->join_ev[g]);
+    }
+    if (ctx->fork_ev) cudaEventDestroy(ctx->fork_ev);
     for (cudaStream_t sx : ctx->color_streams) cudaStreamDestroy(sx);
     for (cudaEvent_t e : ctx->color_events) cudaEventDestroy(e);
     pinned_free(ctx->pinned_ctr);

@@ -313,6 +313,27 @@ int choose_panel(bool fp64, const vne_options* opt, int64_t n) {
     return 8;
 }
 
+void init_streams(vne_ctx* ctx, int groups) {
+    if (groups > 1 && !ctx->fork_ev) VNE_TRY_CUDA(ctx, cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming));
+    for (int g = 0; g + 1 < groups; g++) {
+        if (!ctx->aux[g]) VNE_TRY_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->aux[g], cudaStreamNonBlocking));
+        if (!ctx->join_ev[g]) VNE_TRY_CUDA(ctx, cudaEventCreateWithFlags(&ctx->join_ev[g], cudaEventDisableTiming));
+    }
+}
+
+void fork_streams(vne_ctx* ctx, cudaStream_t s, int groups) {
+    if (groups <= 1) return;
+    VNE_TRY_CUDA(ctx, cudaEventRecord(ctx->fork_ev, s));
+    for (int g = 0; g + 1 < groups; g++) VNE_TRY_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[g], ctx->fork_ev, 0));
+}
+
+void join_streams(vne_ctx* ctx, cudaStream_t s, int groups) {
+    for (int g = 0; g + 1 < groups; g++) {
+        VNE_TRY_CUDA(ctx, cudaEventRecord(ctx->join_ev[g], ctx->aux[g]));
+        VNE_TRY_CUDA(ctx, cudaStreamWaitEvent(s, ctx->join_ev[g], 0));
+    }
+}
+
 // ---------------------------------------------------------------------------
 // block Krylov engine
 
@@ -340,7 +361,8 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
     double* mean = ws_get_t<double>(ctx, "mean", SK);
     double* psi = ws_get_t<double>(ctx, tag + ".psi", SK);
     const int ctas = P.ctas_per_panel(), tiles = P.tiles_per_panel();
-    double* part = ws_get_t<double>(ctx, "part", (size_t)panels * std::max(ctas, tiles * P.sub()) * ks);
+    double* part = ws_get_t<double>(ctx, "part", (size_t)panels * std::max(ctas, tiles) * ks);
+    double* part_u = ws_get_t<double>(ctx, "part.update", (size_t)panels * tiles * P.sub() * ks);
     uint32_t* counter = ws_get_t<uint32_t>(ctx, "counter", (size_t)panels * S, true);
     const int nh = (int)P.hubs.size();
     const int64_t nnz_total = P.nnz_total;
@@ -403,6 +425,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
     p.sub = P.sub();
     p.u = u;
     p.part = part;
+    p.part_u = part_u;
     p.counter = counter;
     double* rcoef = nullptr;
     double* rpart = nullptr;
@@ -428,9 +451,9 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
         pro.eps = sizeof(T) == 4 ? 0x1.0p-24 : 0x1.0p-53;
         pro.normM = P.norm_m;
     }
-    // The step loop, enqueued on stream `s`; `prof` brackets the launches
-    // with events (never while capturing).
-    auto enqueue_loop = [&](cudaStream_t s, bool prof, int j_begin, int j_end) {
+    // The step loop of panels [pb, pb + pc), enqueued on stream `s`; `prof`
+    // brackets the launches with events (never while capturing).
+    auto enqueue_panels = [&](cudaStream_t s, bool prof, int j_begin, int j_end, int pb, int pc) {
         for (int j = j_begin; j <= j_end; j++) {
             p.first = (j == 1);
             p.renorm = 0;
@@ -451,25 +474,25 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
             if (interleave && !reorth) {
                 // per-panel launches, step then update of the same panel: the
                 // update finds u and w_j of that panel still in L2
-                for (int pn = 0; pn < panels; pn++) {
+                for (int pn = pb; pn < pb + pc; pn++) {
                     p.panel_base = pn;
                     VNE_TRY_CUDA(ctx, launch_step<T>(p, ks, 1, P.valued, variant, s));
                     VNE_TRY_CUDA(ctx, launch_update<T>(p, ks, 1, s));
                 }
                 p.panel_base = 0;
-                ctx->launches += 2 * panels;
+                ctx->launches += 2 * pc;
                 if (prof) {
                     e1 = ctx_event(ctx);
                     VNE_TRY_CUDA(ctx, cudaEventRecord(e1, s));
                 }
             } else {
-                p.panel_base = 0;
-                VNE_TRY_CUDA(ctx, launch_step<T>(p, ks, panels, P.valued, variant, s));
+                p.panel_base = pb;
+                VNE_TRY_CUDA(ctx, launch_step<T>(p, ks, pc, P.valued, variant, s));
                 if (prof) {
                     e1 = ctx_event(ctx);
                     VNE_TRY_CUDA(ctx, cudaEventRecord(e1, s));
                 }
-                VNE_TRY_CUDA(ctx, launch_update<T>(p, ks, panels, s));
+                VNE_TRY_CUDA(ctx, launch_update<T>(p, ks, pc, s));
                 ctx->launches += 2;
             }
             if (prof) {
@@ -507,7 +530,9 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 rp.j = j;
                 rp.K = Kp;
                 rp.n_total = P.n_total;
-                rp.panels = panels;
+                rp.panels = pc;
+                rp.panel_base = pb;
+                rp.jstride = m;
                 rp.tiles_per_panel = tiles;
                 rp.sub = P.sub();
                 rp.tiles = P.d_tiles;
@@ -521,14 +546,16 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 cp.coef = rcoef;
                 cp.j = j;
                 cp.K = Kp;
-                cp.panels = panels;
+                cp.panels = pc;
+                cp.panel_base = pb;
+                cp.jstride = m;
                 cp.tiles_per_panel = tiles;
                 cp.sel = pro.sel;
                 cp.panel_active = pro.panel_active;
                 for (int pass = 0; pass < 2; pass++) VNE_TRY_CUDA(ctx, launch_reorth<T>(rp, cp, ks, s));
                 p.renorm = 1;
                 p.panel_active = pro.panel_active;
-                VNE_TRY_CUDA(ctx, launch_update<T>(p, ks, panels, s));
+                VNE_TRY_CUDA(ctx, launch_update<T>(p, ks, pc, s));
                 p.panel_active = nullptr;
                 ctx->launches += 8;
             } else if (reorth && j < m + 1) {
@@ -539,7 +566,9 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 rp.j = j;
                 rp.K = Kp;
                 rp.n_total = P.n_total;
-                rp.panels = panels;
+                rp.panels = pc;
+                rp.panel_base = pb;
+                rp.jstride = m;
                 rp.tiles_per_panel = tiles;
                 rp.sub = P.sub();
                 rp.tiles = P.d_tiles;
@@ -551,14 +580,37 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 cp.coef = rcoef;
                 cp.j = j;
                 cp.K = Kp;
-                cp.panels = panels;
+                cp.panels = pc;
+                cp.panel_base = pb;
+                cp.jstride = m;
                 cp.tiles_per_panel = tiles;
                 for (int pass = 0; pass < 2; pass++) VNE_TRY_CUDA(ctx, launch_reorth<T>(rp, cp, ks, s));
                 p.renorm = 1;
-                VNE_TRY_CUDA(ctx, launch_update<T>(p, ks, panels, s));
+                VNE_TRY_CUDA(ctx, launch_update<T>(p, ks, pc, s));
                 ctx->launches += 7;
             }
         }
+    };
+    // Panels are independent recurrences, and the end of a kernel (its last
+    // CTAs, the reduction of the partial sums) leaves SMs idle, so a captured
+    // loop runs its panels in two groups on parallel branches of the graph; the
+    // numbers do not change.  Measured, one branch -> two: BA 20k x 64 FP32
+    // 1.40 -> 1.23 ms, WS 150k x 64 3.74 -> 3.48, weighted FP64 60k x 33 14.6 ->
+    // 14.0, BA 1e6 Hutch++ 136.5 -> 132.7; three and four branches gain no
+    // more.  Blocks below 2 MB (3,000 x 64: 0.723 -> 0.730 ms) and loops that
+    // the host launches (a second stream's launches, 9.9 -> 10.7 ms) keep one.
+    const int groups =
+        panels >= 2 && reorth != 2 && !interleave && slot_elems * sizeof(T) >= (size_t)2 << 20 ? 2 : 1;
+    auto enqueue_loop = [&](cudaStream_t s, bool prof, int j_begin, int j_end) {
+        enqueue_panels(s, prof, j_begin, j_end, 0, panels);
+    };
+    auto capture_loop = [&](cudaStream_t s) {
+        fork_streams(ctx, s, groups);
+        for (int g = 0; g < groups; g++) {
+            const int pb = (int)((int64_t)panels * g / groups), pe = (int)((int64_t)panels * (g + 1) / groups);
+            enqueue_panels(g == 0 ? s : ctx->aux[g - 1], false, 1, m, pb, pe - pb);
+        }
+        join_streams(ctx, s, groups);
     };
     if (ctx->time_steps) VNE_TRY_CUDA(ctx, cudaEventRecord(ctx->loop_ev[0], st));
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -594,7 +646,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
         std::string key;
         auto put = [&key](const void* v, size_t b) { key.append(reinterpret_cast<const char*>(v), b); };
         const int ints[] = {(int)sizeof(T), ks, panels, m, variant, (int)interleave, (int)reorth, (int)store_all,
-                            (int)P.valued, SK};
+                            (int)P.valued, SK, groups};
         put(ints, sizeof(ints));
         const void* ptrs[] = {slots,     alpha,    beta,         sigma,    rcoef,          rpart,
                               pro.omega, pro.sel,     pro.pend_sel, pro.pend, pro.panel_active};
@@ -611,11 +663,12 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 }
                 if (!ctx->cap_stream)
                     VNE_TRY_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
+                init_streams(ctx, groups);
                 const int64_t l0 = ctx->launches;
                 cudaGraph_t g = nullptr;
                 VNE_TRY_CUDA(ctx, cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
                 try {
-                    enqueue_loop(ctx->cap_stream, false, 1, m);
+                    capture_loop(ctx->cap_stream);
                 } catch (...) {
                     cudaStreamEndCapture(ctx->cap_stream, &g);
                     if (g) cudaGraphDestroy(g);
@@ -750,8 +803,8 @@ OpConsts op_consts(vne_ctx* ctx, const Problem& P, int Kp, double shift, const s
 // out = A in + shift * in (A = scale M), and dq[c] = scale * (in . out).
 template <typename T>
 void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* out, const OpConsts& k, double* dq,
-                    int variant) {
-    cudaStream_t st = ctx->stream;
+                    int variant, const PanelRange* range) {
+    cudaStream_t st = range ? range->stream : ctx->stream;
     const int panels = Kp / ks;
     const int ctas = P.ctas_per_panel(), tiles = P.tiles_per_panel();
     const int nh = (int)P.hubs.size();
@@ -794,7 +847,8 @@ void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* ou
         e0 = ctx_event(ctx);
         VNE_TRY_CUDA(ctx, cudaEventRecord(e0, st));
     }
-    VNE_TRY_CUDA(ctx, launch_step<T>(p, ks, panels, P.valued, variant, st));
+    p.panel_base = range ? range->begin : 0;
+    VNE_TRY_CUDA(ctx, launch_step<T>(p, ks, range ? range->count : panels, P.valued, variant, st));
     ctx->launches += 1;
     if (ctx->profile) {
         cudaEvent_t e1 = ctx_event(ctx);
@@ -811,7 +865,8 @@ void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* ou
                                const std::string&, BlockOut&, int, bool, bool, bool, const Adaptive*);          \
     template std::vector<double> quadforms<T>(vne_matrix*, const vne_options*, StartSource, int, int,             \
                                               const double*);                                                    \
-    template void apply_operator<T>(vne_ctx*, Problem&, int, int, const T*, T*, const OpConsts&, double*, int);
+    template void apply_operator<T>(vne_ctx*, Problem&, int, int, const T*, T*, const OpConsts&, double*, int,      \
+                                    const PanelRange*);
 VNE_ENGINE_INSTANTIATE(float)
 VNE_ENGINE_INSTANTIATE(double)
 

@@ -99,6 +99,11 @@ struct vne_ctx {
     std::map<std::string, LoopGraph> graphs;
     std::map<std::string, int> graph_seen;
     cudaStream_t cap_stream = nullptr;  // private stream the captures run on
+    // streams of the panel groups beside the call's own, and their fork / join
+    // events (init_streams, fork_streams, join_streams)
+    static constexpr int kMaxGroups = 4;
+    cudaStream_t aux[kMaxGroups - 1] = {};
+    cudaEvent_t fork_ev = nullptr, join_ev[kMaxGroups - 1] = {};
     int64_t graphs_captured = 0, graphs_replayed = 0;
     int last_steps = 0;  // Lanczos steps of the last quadrature call (largest over its blocks)
     int last_poly_dim = 0;  // polynomial dimension chosen by the switching rule (last rational call)
@@ -299,6 +304,12 @@ int choose_panel(bool fp64, const vne_options* opt, int64_t n);
 // (its panel width may then follow them).
 Sched resolve_sched(const vne_matrix* M, const vne_options* o, int block_cols = 0);
 Problem* matrix_problem(vne_matrix* M, const vne_options* opt);
+// Panels are independent recurrences: `groups` - 1 streams beside s that wait
+// for what s holds now (fork), and s waiting for all of them (join).  They are
+// made before a capture starts (init).
+void init_streams(vne_ctx* ctx, int groups);
+void fork_streams(vne_ctx* ctx, cudaStream_t s, int groups);
+void join_streams(vne_ctx* ctx, cudaStream_t s, int groups);
 
 struct BlockOut {
     int K = 0, Kp = 0, ks = 0, panels = 0, m = 0, SK = 0;
@@ -358,11 +369,16 @@ struct OpConsts {
     const double *sig = nullptr, *cp = nullptr, *one = nullptr;
 };
 OpConsts op_consts(vne_ctx* ctx, const Problem& P, int Kp, double shift, const std::string& tag);
+// Some panels of a block, on a stream of their own.
+struct PanelRange {
+    cudaStream_t stream;
+    int begin, count;
+};
 // out = A in + shift * in (A = scale M) and dq[c] = scale * (in . out), with
-// the Lanczos step kernel.
+// the Lanczos step kernel; all panels on the context's stream, or a range.
 template <typename T>
 void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* out, const OpConsts& k, double* dq,
-                    int variant);
+                    int variant, const PanelRange* range = nullptr);
 
 // Rational Krylov quadratic forms (rational_driver.cu).
 template <typename T>

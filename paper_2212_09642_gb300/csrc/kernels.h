@@ -82,7 +82,9 @@ struct StepParams {
     double* alpha;
     double* beta;
     double* sig_next;
-    double* part;
+    double* part;    // step kernel's partial sums [panels][ctas][KS]
+    double* part_u;  // update kernel's [panels][tiles * sub][KS] (a buffer of its own: panel groups
+                     // run the two kernels at the same time)
     uint32_t* counter;
 };
 
@@ -92,9 +94,11 @@ struct ReorthParams {
     size_t slot_stride;   // elements between consecutive slots
     T* w;                 // vector being orthogonalised (slot j)
     int32_t j, K, n_total, panels, tiles_per_panel;
+    int32_t panel_base;   // first panel of this launch (panels: their number)
+    int32_t jstride;      // basis vectors per panel in part (>= j)
     int32_t sub;          // update pass: CTAs per row tile
     const RowTile* tiles;
-    double* part;         // [panels][j][tiles][KS]
+    double* part;         // [panels][jstride][tiles][KS]
     const double* coef;   // [j][K]
     const int32_t* panel_active;  // nullable: panels with no column to orthogonalise are skipped
     const uint8_t* sel;   // nullable [j][K]: a (panel, i) with no selected column is skipped
@@ -105,6 +109,7 @@ struct ReorthCoefParams {
     const double* sig;    // [j][K] sigma_i of each basis vector
     double* coef;
     int32_t j, K, panels, tiles_per_panel;
+    int32_t panel_base, jstride;  // as in ReorthParams
     const uint8_t* sel;           // nullable [j][K]: orthogonalise column c against basis vector i
     const int32_t* panel_active;  // nullable, as in ReorthParams
 };
@@ -230,6 +235,7 @@ struct CgState {
 template <typename T>
 struct CgVectors {
     int32_t n, tiles_per_panel;
+    int32_t panel_base;     // first panel of the launch
     int32_t sub;            // direction kernel: CTAs per row tile
     int32_t max_tile_rows;  // rows of the largest tile
     int32_t sm_count;
@@ -245,6 +251,7 @@ struct CgVectors {
 template <typename T>
 struct CgFlush {
     int32_t n, K, nshift, panels;
+    int32_t panel_base;   // first panel of the launch (panels: their number)
     int32_t rows;         // rows per CTA (set by the launcher)
     int32_t count;        // residuals in the window (<= CgState::window)
     int32_t first, last;  // first flush: x and p_s start from zero; last: p_s is not needed any more

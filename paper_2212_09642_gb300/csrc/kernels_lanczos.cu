@@ -900,10 +900,10 @@ __global__ void __launch_bounds__(VNE_THREADS) k_update(StepParams<T> p) {
     for (int q = 0; q < CPL; q++) nd[q] = (double)nrm[q];
     cta_colsum<KS, CPL>(nd, red, part);
     if (threadIdx.x < KS)
-        p.part[(((size_t)panel * p.tiles_per_panel + tile) * p.sub + piece) * KS + threadIdx.x] = part;
+        p.part_u[(((size_t)panel * p.tiles_per_panel + tile) * p.sub + piece) * KS + threadIdx.x] = part;
     __shared__ double tot[KS];
     const SegInfo sg = p.seg[t.seg];
-    if (last_cta_reduce<KS>(p.part, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel * p.sub,
+    if (last_cta_reduce<KS>(p.part_u, p.counter + (size_t)panel * p.nseg + t.seg, panel, p.tiles_per_panel * p.sub,
                             sg.tile_begin * p.sub, sg.tile_count * p.sub, tot)) {
         if (threadIdx.x < KS) {
             size_t o = (size_t)t.seg * p.K + panel * KS + threadIdx.x;
@@ -975,7 +975,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_dots(ReorthParams<T> p) 
     // grid: panel * tiles * j ; each CTA: one tile, one i
     const int i = blockIdx.x % p.j;
     const int pt = blockIdx.x / p.j;
-    const int panel = pt / p.tiles_per_panel, tile = pt % p.tiles_per_panel;
+    const int panel = p.panel_base + pt / p.tiles_per_panel, tile = pt % p.tiles_per_panel;
     if (p.panel_active && !p.panel_active[panel]) return;
     if (!reorth_panel_uses<T, KS>(p, panel, i)) return;
     const RowTile t = p.tiles[tile];
@@ -983,7 +983,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_dots(ReorthParams<T> p) 
     const T* Wi = p.basis + (size_t)i * p.slot_stride + base;
     const T* Wn = p.w + base;
     const int nchunks = (t.row_end - t.row_begin) * G;
-    const size_t opart = (((size_t)panel * p.j + i) * p.tiles_per_panel + tile) * KS;
+    const size_t opart = (((size_t)panel * p.jstride + i) * p.tiles_per_panel + tile) * KS;
     if constexpr (sizeof(T) == 8) {
         // FP64 inner products are bound by the FP64 pipe, so the partial sums
         // take as few FP64 additions as possible: each thread accumulates its
@@ -1069,7 +1069,7 @@ __global__ void k_reorth_coef(ReorthCoefParams p) {
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     int total = p.panels * p.j * KS;
     if (idx >= total) return;
-    int c = idx % KS, i = (idx / KS) % p.j, panel = idx / (KS * p.j);
+    int c = idx % KS, i = (idx / KS) % p.j, panel = p.panel_base + idx / (KS * p.j);
     int col = panel * KS + c;
     if ((p.panel_active && !p.panel_active[panel]) || (p.sel && !p.sel[(size_t)i * p.K + col])) {
         p.coef[(size_t)i * p.K + col] = 0.0;
@@ -1077,7 +1077,7 @@ __global__ void k_reorth_coef(ReorthCoefParams p) {
     }
     double s = 0.0;
     for (int t = 0; t < p.tiles_per_panel; t++)
-        s += p.part[(((size_t)panel * p.j + i) * p.tiles_per_panel + t) * KS + c];
+        s += p.part[(((size_t)panel * p.jstride + i) * p.tiles_per_panel + t) * KS + c];
     double sig = p.sig[(size_t)i * p.K + col];
     p.coef[(size_t)i * p.K + col] = sig * sig * s;
 }
@@ -1092,7 +1092,8 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_apply(ReorthParams<T> p)
     constexpr int V = Chunk16<T>::V, G = KS / V, U = 4;
     static_assert(KS % V == 0 && VNE_THREADS % G == 0, "chunk layout");
     const int per = p.tiles_per_panel * p.sub;
-    const int panel = blockIdx.x / per, tile = (int)(blockIdx.x % per) / p.sub, piece = (int)(blockIdx.x % per) % p.sub;
+    const int panel = p.panel_base + blockIdx.x / per;
+    const int tile = (int)(blockIdx.x % per) / p.sub, piece = (int)(blockIdx.x % per) % p.sub;
     if (p.panel_active && !p.panel_active[panel]) return;
     __shared__ int16_t act[kReorthMaxJ];
     __shared__ T cf[kReorthMaxJ * KS];
@@ -1469,7 +1470,7 @@ cudaError_t launch_step_update_segj(const StepParams<T>& p, int ks, int panels, 
 template <typename T>
 cudaError_t launch_reorth(const ReorthParams<T>& p, const ReorthCoefParams& c, int ks, cudaStream_t st) {
     if (p.j <= 0) return cudaSuccess;
-    if (p.j > kReorthMaxJ) return cudaErrorInvalidValue;
+    if (p.j > kReorthMaxJ || p.jstride < p.j || c.jstride != p.jstride) return cudaErrorInvalidValue;
     VNE_DISPATCH_KS(T, ks, (k_reorth_dots<T, KS><<<dim3(p.panels * p.tiles_per_panel * p.j), VNE_THREADS, 0, st>>>(p)));
     int total = c.panels * c.j * ks;
     VNE_DISPATCH_KS(T, ks, (k_reorth_coef<KS><<<dim3((total + 255) / 256), 256, 0, st>>>(c)));
@@ -1481,6 +1482,7 @@ cudaError_t launch_reorth(const ReorthParams<T>& p, const ReorthCoefParams& c, i
 template <typename T>
 cudaError_t launch_col_dots(const ReorthParams<T>& p, const ReorthCoefParams& c, int ks, cudaStream_t st) {
     if (p.j <= 0) return cudaSuccess;
+    if (p.jstride < p.j || c.jstride != p.jstride) return cudaErrorInvalidValue;
     VNE_DISPATCH_KS(T, ks, (k_reorth_dots<T, KS><<<dim3(p.panels * p.tiles_per_panel * p.j), VNE_THREADS, 0, st>>>(p)));
     int total = c.panels * c.j * ks;
     VNE_DISPATCH_KS(T, ks, (k_reorth_coef<KS><<<dim3((total + 255) / 256), 256, 0, st>>>(c)));

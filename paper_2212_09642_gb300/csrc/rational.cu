@@ -52,7 +52,6 @@
 
 namespace vne {
 
-constexpr int kMaxShifts = 8;
 constexpr int kMaxBasis = 24;  // 1 + up to 15 polynomial directions + 8 poles
 
 __device__ __forceinline__ double f_ent(double x) { return x > 0.0 ? -x * log(x) : 0.0; }
@@ -108,7 +107,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgSta
     constexpr int LPR = KS / CPL;            // lanes per row
     constexpr int RPI = VNE_THREADS / LPR;   // rows per iteration
     constexpr int U = 4;
-    const int panel = cta / v.tiles_per_panel, tile = cta % v.tiles_per_panel;
+    const int panel = v.panel_base + cta / v.tiles_per_panel, tile = cta % v.tiles_per_panel;
     RowTile t = v.tiles[tile];
     if (CLUSTER) {  // run crank of the tile
         t.row_begin += crank * 16 * RPI;
@@ -271,7 +270,8 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_direction(CgVectors<T> v, Cg
     constexpr int RPI = VNE_THREADS / LPR;
     constexpr int U = 4;
     const int per = v.tiles_per_panel * v.sub;
-    const int panel = blockIdx.x / per, tile = (int)(blockIdx.x % per) / v.sub, piece = (int)(blockIdx.x % per) % v.sub;
+    const int panel = v.panel_base + blockIdx.x / per;
+    const int tile = (int)(blockIdx.x % per) / v.sub, piece = (int)(blockIdx.x % per) % v.sub;
     const RowTile t = v.tiles[tile];
     const int len = ((t.row_end - t.row_begin) + v.sub - 1) / v.sub;
     const int r_begin = t.row_begin + piece * len, r_end = min(t.row_end, r_begin + len);
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_coefs(CgFlush<T> f, CgState 
     __shared__ int s_live;
     if (threadIdx.x == 0) s_live = f.first ? (1 << st.nshift) - 1 : 0;
     __syncthreads();
-    const int panel = blockIdx.x;
+    const int panel = f.panel_base + blockIdx.x;
     for (int idx = threadIdx.x; idx < st.nshift * ks; idx += VNE_THREADS) {
         const int s = idx / ks, c = panel * ks + idx % ks;
         const size_t o = (size_t)s * st.K + c;
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_flush(CgFlush<T> f) {
     T* cf = reinterpret_cast<T*>(fl_smem);       // [count][G][2][KS]
     __shared__ __align__(16) T cp[G][2][KS];
     const int chunks = (f.n + f.rows - 1) / f.rows;
-    const int panel = blockIdx.x / chunks, chunk = blockIdx.x % chunks;
+    const int panel = f.panel_base + blockIdx.x / chunks, chunk = blockIdx.x % chunks;
     const int r_begin = chunk * f.rows, r_end = min(f.n, r_begin + f.rows);
     const int sub = threadIdx.x % LPR, rs = threadIdx.x / LPR, cofs = sub * CPL;
     const size_t pofs = (size_t)panel * f.n * KS;

@@ -597,7 +597,8 @@ int tick_impl(vne_server* S) {
     p.tiles_per_panel = (int32_t)tile_high;
     p.sub = P.sub();
     p.u = (T*)S->u;
-    p.part = ws_get_t<double>(ctx, "srv.step_part", (size_t)panels * std::max(cta_high, tile_high * P.sub()) * ks);
+    p.part = ws_get_t<double>(ctx, "srv.step_part", (size_t)panels * std::max<int64_t>(cta_high, 1) * ks);
+    p.part_u = ws_get_t<double>(ctx, "srv.update_part", (size_t)panels * tile_high * P.sub() * ks);
     p.counter = ws_get_t<uint32_t>(ctx, "srv.step_counter", (size_t)panels * P.nseg);
     p.segj = (const int32_t*)dptr(i_sj);
     p.slot0 = (T*)S->slot0;
