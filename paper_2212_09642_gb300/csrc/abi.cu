@@ -336,8 +336,12 @@ extern "C" vne_status vne_quadform_batch(vne_matrix* M, const double* vectors, i
     int ks = sc.ks;
     const int reorth = want_reorth(M, &o);
     int lim = block_limit(&o);
+    // a schedule that the caller asked for (or tuned) is the multi-CTA kernels'
+    const bool auto_sched = o.panel <= 0 && o.item_nnz <= 0 && o.step_variant < 0 && o.interleave < 0 &&
+                            o.items_per_warp <= 0 && !M->tuned && !ctx->profile;
     for (int b0 = 0; b0 < k; b0 += lim) {
         int K = std::min(lim, k - b0);
+        const bool small = auto_sched && small_lanczos_wins(M, *P, K, m, reorth);
         StartSource s{};
         s.kind = SRC_DENSE64;
         s.ncols = K;
@@ -347,11 +351,11 @@ extern "C" vne_status vne_quadform_batch(vne_matrix* M, const double* vectors, i
         if (M->fp64) {
             check_ks<double>(ctx, ks);
             run_block<double>(ctx, *P, s, nullptr, K, ks, m, reorth, false, M->desing, "q", out, sc.variant,
-                              sc.interleave, sc.graph);
+                              sc.interleave, sc.graph, true, nullptr, small);
         } else {
             check_ks<float>(ctx, ks);
             run_block<float>(ctx, *P, s, nullptr, K, ks, m, reorth, false, M->desing, "q", out, sc.variant,
-                             sc.interleave, sc.graph);
+                             sc.interleave, sc.graph, true, nullptr, small);
         }
         std::vector<double> h = download(ctx, out.psi, K);
         std::copy(h.begin(), h.end(), psi + b0);

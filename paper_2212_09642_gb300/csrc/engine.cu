@@ -339,17 +339,59 @@ void join_streams(vne_ctx* ctx, cudaStream_t s, int groups) {
 
 
 
+bool small_lanczos_wins(vne_matrix* M, Problem& P, int K, int m, int reorth) {
+    if (M->n > 25000 || small_lanczos_smem((int)M->n, M->fp64) > 200 * 1024) return false;
+    if (P.nlong == -1) {  // once per schedule: the rows that whole warps take
+        std::vector<int32_t> rows;
+        for (int64_t r = 0; r < M->n; r++)
+            if (M->h_rowptr[r + 1] - M->h_rowptr[r] > kSmallLongRow) rows.push_back((int32_t)r);
+        if (rows.size() > 256) {
+            P.nlong = -2;
+        } else {
+            if (!rows.empty()) {
+                P.d_long = dev_copy(M->ctx, rows);
+                P.owned.push_back(P.d_long);
+            }
+            P.nlong = (int32_t)rows.size();
+        }
+    }
+    if (P.nlong < 0) return false;
+    // Times in ms of both forms, fitted to a sweep over n = 300 .. 14,000 (mean
+    // degree 8, ER and BA), 1 to 160 columns, 20 and 30 steps; columns beyond
+    // one per SM take another wave.  FP32, n = 700, 5 columns, 20 steps: 0.35
+    // with the multi-CTA kernels, 0.17; n = 5,000, 64, 30: 0.62, 0.43; n =
+    // 14,000, 64, 30: 0.73, 0.96.  FP64 with full reorthogonalisation, n = 700,
+    // 64, 30: 1.76, 0.85; n = 2,000, 64, 30: 2.19, 1.80; n = 5,000: 3.5, 3.9.
+    const double n = (double)M->n, nnz = (double)M->nnz, steps = m;
+    const double waves = (double)((K + M->ctx->sm_count - 1) / std::max(M->ctx->sm_count, 1));
+    if (!M->fp64 && reorth == 0) {
+        const double mine = 0.10 + waves * steps * (0.0035 + 0.7e-6 * n + 0.15e-6 * nnz);
+        const double theirs = 0.10 + steps * (0.0125 + 1e-6 * n);
+        return 1.1 * mine < theirs;
+    }
+    if (M->fp64 && reorth == 1) {
+        // the Gram-Schmidt passes: 2 m^2 n multiply-adds per column at 3.36e6
+        // per ms and SM, or spread over the chip at three quarters of that
+        const double gs = 2.0 * steps * steps * n;
+        const double mine = 1.2 * (0.10 + waves * (steps * (0.0045 + 4.8e-7 * nnz) + gs / 3.36e6));
+        const double theirs = 0.20 + 0.045 * steps + gs * K / 3.8e8;
+        return mine < theirs;
+    }
+    return false;
+}
+
 template <typename T>
 void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_src, int K, int ks, int m,
                int reorth, bool keep_basis, bool desing, const std::string& tag, BlockOut& out, int variant,
-               bool interleave, bool graph, bool want_psi, const Adaptive* ad) {
+               bool interleave, bool graph, bool want_psi, const Adaptive* ad, bool small) {
     cudaStream_t st = ctx->stream;
     const int panels = (K + ks - 1) / ks;
     const int Kp = panels * ks;
     const int S = P.nseg;
     const int SK = S * Kp;
     const size_t slot_elems = (size_t)Kp * P.n_total;
-    const bool store_all = keep_basis || reorth != 0;
+    small = small && S == 1 && !keep_basis && reorth <= 1 && !ad;
+    const bool store_all = !small && (keep_basis || reorth != 0);
     const int nslots = store_all ? m + 1 : 2;
     VNE_REQUIRE(ctx, reorth == 0 || S == 1, VNE_EUNSUPPORTED, "reorthogonalisation needs a single matrix");
     T* slots = ws_get_t<T>(ctx, tag + ".slots", slot_elems * nslots);
@@ -429,7 +471,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
     p.counter = counter;
     double* rcoef = nullptr;
     double* rpart = nullptr;
-    if (reorth) {
+    if (reorth && !small) {
         rcoef = ws_get_t<double>(ctx, "reorth.coef", (size_t)m * Kp);
         rpart = ws_get_t<double>(ctx, "reorth.part", (size_t)panels * m * tiles * ks);
     }
@@ -616,7 +658,26 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cap = cudaStreamCaptureStatusActive;
     int m_run = m;  // steps actually taken
-    if (ad && ad->tol > 0.0 && want_psi) {
+    if (small) {
+        SmallLanczos<T> sl{};
+        sl.rowptr = P.rowptr;
+        sl.col = P.col;
+        sl.vals = P.valued ? (const T*)P.vals : nullptr;
+        sl.long_rows = P.d_long;
+        sl.nlong = P.nlong;
+        sl.n = P.n_total;
+        sl.ks = ks;
+        sl.m = m;
+        sl.SK = SK;
+        sl.tau = P.segs[0].tau;
+        sl.w1 = slot(1);
+        sl.basis = reorth ? ws_get_t<T>(ctx, "small.basis", (size_t)K * m * P.n_total) : nullptr;
+        sl.alpha = alpha;
+        sl.beta = beta;
+        sl.sigma = sigma;
+        VNE_TRY_CUDA(ctx, launch_lanczos_small<T>(sl, K, reorth != 0, st));
+        ctx->launches += 1;
+    } else if (ad && ad->tol > 0.0 && want_psi) {
         // adaptive: chunks of `check` steps launched directly, each followed
         // by the quadratures and error estimates of all columns
         double* est = ws_get_t<double>(ctx, tag + ".est", 3 * (size_t)SK);
@@ -862,7 +923,7 @@ void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* ou
 
 #define VNE_ENGINE_INSTANTIATE(T)                                                                                \
     template void run_block<T>(vne_ctx*, Problem&, const StartSource&, const T*, int, int, int, int, bool, bool,  \
-                               const std::string&, BlockOut&, int, bool, bool, bool, const Adaptive*);          \
+                               const std::string&, BlockOut&, int, bool, bool, bool, const Adaptive*, bool);    \
     template std::vector<double> quadforms<T>(vne_matrix*, const vne_options*, StartSource, int, int,             \
                                               const double*);                                                    \
     template void apply_operator<T>(vne_ctx*, Problem&, int, int, const T*, T*, const OpConsts&, double*, int,      \

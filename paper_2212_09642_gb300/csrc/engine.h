@@ -170,6 +170,10 @@ struct Problem {
     int32_t hub_slots = 0;
     int32_t stage_nnz = 0;   // largest item (nonzeros)
     int32_t ipw = 1;         // work items per warp (CTA = VNE_WARPS * ipw items)
+    // rows longer than kSmallLongRow, for the kernel that keeps a column on an
+    // SM (single matrix; -1: not counted yet, -2: too many of them)
+    int32_t nlong = -1;
+    int32_t* d_long = nullptr;  // in `owned`
     double norm_m = 0.0;     // Gershgorin bound of the stored operator (single matrix)
     // device copies (owned)
     SegInfo* d_segs = nullptr;
@@ -343,7 +347,13 @@ struct Adaptive {
 template <typename T>
 void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_src, int K, int ks, int m,
                int reorth, bool keep_basis, bool desing, const std::string& tag, BlockOut& out, int variant = 0,
-               bool interleave = false, bool graph = true, bool want_psi = true, const Adaptive* ad = nullptr);
+               bool interleave = false, bool graph = true, bool want_psi = true, const Adaptive* ad = nullptr,
+               bool small = false);
+// Whether a block of K columns and m steps runs faster with a CTA per column
+// (lanczos_small.cu; reorth 0 or 1), `small` of run_block.  The rule weighs
+// the columns too, so it is for callers whose columns are not compared across
+// blocks of other widths.
+bool small_lanczos_wins(vne_matrix* M, Problem& P, int K, int m, int reorth);
 
 // Reorthogonalisation policy of a call: 0 none, 1 full, 2 partial.
 int want_reorth(const vne_matrix* M, const vne_options* o);

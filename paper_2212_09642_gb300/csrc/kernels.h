@@ -210,6 +210,26 @@ template <typename T>
 cudaError_t launch_select_columns(const T* in, int n, int ks, const int32_t* src_cols, int k, int Kp, T* out,
                                   cudaStream_t st);
 
+// ---- small graphs: a CTA per column, all steps in one launch (lanczos_small.cu) ----
+constexpr int kSmallMaxSteps = 128;  // Lanczos steps of a launch
+constexpr int kSmallLongRow = 64;    // longer rows are taken by whole warps
+template <typename T>
+struct SmallLanczos {
+    const int32_t* rowptr;
+    const int32_t* col;
+    const T* vals;             // nullable: pattern (graph Laplacian)
+    const int32_t* long_rows;  // rows longer than kSmallLongRow
+    int32_t nlong;
+    int32_t n, ks, m, SK;      // SK: columns of the scalar arrays
+    double tau;                // breakdown threshold on beta
+    const T* w1;               // start vectors, panel-major
+    T* basis;                  // [columns][m][n], with reorthogonalisation
+    double *alpha, *beta, *sigma;  // [m][SK], sigma [m + 1][SK]; sigma row 0 set, the rest zero
+};
+size_t small_lanczos_smem(int n, bool fp64);
+template <typename T>
+cudaError_t launch_lanczos_small(const SmallLanczos<T>&, int cols, bool reorth, cudaStream_t);
+
 // ---- multi-shift CG and rational projection (rational.cu) ----
 // v *= 1 / sqrt(rem2[col]) where rem2 > drop^2 orig2 (a kept direction),
 // else v = 0 (a dependent one): the last step of one Gram-Schmidt
