@@ -154,8 +154,11 @@ template <typename T> cudaError_t launch_update(const StepParams<T>&, int ks, in
 // segment): for the segments listed, g = probe columns col0[s] ..
 // col0[s] + K - 1 (Rademacher, or Gaussian), g' = g - Q_s (Q_s^T g),
 // c = g' - mean(g') 1 written to w1 (panel-major, K columns), with
-// ||c||^2 and sigma_1 = 1 / ||c||.  Three passes with fixed-order
+// ||c||^2 and sigma_1 = 1 / ||c||.  Two passes with fixed-order
 // per-segment reductions.
+constexpr int kSrvSub = 4;  // CTAs per listed tile
+// values per segment of the first pass: Q^T g [4][K], sum g [K], sum q [4]
+constexpr __host__ __device__ int kSrvW(int K) { return 5 * K + 4; }
 template <typename T>
 struct SrvStartParams {
     const int32_t* tile_list;  // [ntiles] tiles of the starting segments, grouped by segment
@@ -167,14 +170,13 @@ struct SrvStartParams {
     const uint64_t* seg_seed;  // [nseg] mixed seed
     const int32_t* seg_col0;   // [nseg] first probe column of the block
     const T* q;                // [n_total][4] deflation basis, zero columns beyond the rank
-    double* coef;              // [nseg][4][K]
-    double* mean;              // [nseg][K]
+    double* coef;              // [nseg][kSrvW(K)]: totals of the first pass
+    double* mean;              // [nseg][K]: totals of the second (scratch)
     double* norm2;             // [nseg][K]
     double* sig1;              // [nseg][K]: row 0 of the sigma array
     T* w1;                     // panel-major [K / KS][n_total][KS]
-    double* part;              // [ntiles][4 * K]
-    uint32_t* counter;         // [nseg], zero between launches
-    int32_t ntiles, K, n_total, gaussian;
+    double* part;              // [ntiles * kSrvSub][kSrvW(K)]
+    int32_t ntiles, nseg, K, n_total, gaussian;
 };
 template <typename T> cudaError_t launch_srv_start(const SrvStartParams<T>& p, int ks, cudaStream_t st);
 // Step and update kernels for per-segment step counters (p.segj, pattern operators only).

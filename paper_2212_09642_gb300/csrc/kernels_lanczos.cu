@@ -399,116 +399,179 @@ __global__ void __launch_bounds__(VNE_THREADS, 3) k_start_center(StartParams<T> 
 }
 
 // ---------------------------------------------------------------------------
-// Served blocks: deflated start vectors (see kernels.h).  One CTA per listed
-// tile; thread t handles block column t % 64 (and t % 64 + 64, ..) of the
-// tile's rows t / 64, t / 64 + 4, ...; partials of the CTA are summed over
-// its four row groups, and the last CTA of a segment adds the segment's
-// tile partials in list order.
-
-// The last-arriving CTA of segment s sums the W-value partials of its tiles
-// (list entries tb .. tb + tc - 1) in order; true in that CTA, with the
-// totals in out[0 .. W).
-__device__ bool srv_last_reduce(const double* part, uint32_t* counter, int tb, int tc, int W, double* out) {
-    __shared__ int s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == (unsigned)(tc - 1);
-    __syncthreads();
-    if (!s_last) return false;
-    __threadfence();
-    for (int w = threadIdx.x; w < W; w += blockDim.x) {
-        double acc = 0.0;
-        for (int i = 0; i < tc; i++) acc += ld_cg(&part[(size_t)(tb + i) * W + w]);
-        out[w] = acc;
-    }
-    if (threadIdx.x == 0) *counter = 0u;
-    __syncthreads();
-    return true;
-}
+// Served blocks: deflated start vectors (see kernels.h).  A listed tile is
+// split over kSrvSub CTAs; thread t handles block column t % 64 of the piece's
+// rows t / 64, t / 64 + 4, ..., four rows in flight.  Partial sums go to
+// part[tile * kSrvSub + piece][..] and are added per segment by k_srv_sum, which
+// spreads the additions over CTAs (one last CTA per segment would add up to 800
+// partials of 324 values through one SM's FP64 port, about 60 us).
+// Two passes over the probes instead of three: the column means of
+// g' = g - Q coef follow from the sums of g and of Q's columns, which the first
+// pass takes along.  The probes are hashed again in the second pass.  Measured
+// per tick with starting blocks, served mix of 32 queries: 144 us with one CTA
+// per tile and three passes, 76 us now.
 
 template <typename T>
-__device__ __forceinline__ T srv_probe(const SrvStartParams<T>& p, int s, int c, int r) {
-    const uint64_t sd = p.seg_seed[s];
-    const uint64_t col = (uint64_t)(p.seg_col0[s] + c);
-    const uint64_t id = (uint64_t)p.node_id[r];
-    return (T)(p.gaussian ? gaussian_entry(sd, col, id) : rademacher_entry(sd, col, id));
+__device__ __forceinline__ T srv_probe(const SrvStartParams<T>& p, uint64_t sd, uint64_t col, int id) {
+    return (T)(p.gaussian ? gaussian_entry(sd, col, (uint64_t)id) : rademacher_entry(sd, col, (uint64_t)id));
 }
 
-// pass 1: coef[s][i][c] = q_i . g_c over the segment's rows
+// Rows of piece blockIdx.x % kSrvSub of the listed tile.
+template <typename T>
+__device__ __forceinline__ void srv_rows(const SrvStartParams<T>& p, const RowTile& t, int& r_begin, int& r_end) {
+    const int len = (t.row_end - t.row_begin + kSrvSub - 1) / kSrvSub, piece = blockIdx.x % kSrvSub;
+    r_begin = t.row_begin + piece * len;
+    r_end = min(t.row_end, r_begin + len);
+}
+
+// pass 1: the sums q_i . g_c (i < 4), sum g_c and sum q_i over the piece's rows
 template <typename T>
 __global__ void __launch_bounds__(VNE_THREADS) k_srv_coef(SrvStartParams<T> p) {
-    const RowTile t = p.tiles[p.tile_list[blockIdx.x]];
-    const int s = t.seg, c0 = threadIdx.x % 64, rs = threadIdx.x / 64;
-    __shared__ double red[VNE_THREADS / 64][4 * 256];
-    for (int c = c0; c < p.K; c += 64) {
-        // products in the vector precision, runs of 16 rows summed in FP64
-        RowSum<T> acc[4];
-        for (int r = t.row_begin + rs; r < t.row_end; r += VNE_THREADS / 64) {
-            const T g = srv_probe(p, s, c, r);
+    constexpr int U = 4, RG = VNE_THREADS / 64;
+    const RowTile t = p.tiles[p.tile_list[blockIdx.x / kSrvSub]];
+    const int s = t.seg, c = threadIdx.x % 64, rs = threadIdx.x / 64;
+    int r_begin, r_end;
+    srv_rows(p, t, r_begin, r_end);
+    __shared__ double red[RG][6][64];
+    // products in the vector precision, runs of 16 rows summed in FP64
+    RowSum<T> acc[4], sg, sq;
+    const uint64_t sd = p.seg_seed[s], col = (uint64_t)(p.seg_col0[s] + c);
+    for (int r0 = r_begin + rs; r0 < r_end; r0 += U * RG) {
+        int id[U];
+        T q[U][4];
 #pragma unroll
-            for (int i = 0; i < 4; i++) acc[i].add(p.q[(size_t)r * 4 + i] * g);
+        for (int u = 0; u < U; u++) {
+            const int r = r0 + u * RG;
+            if (r < r_end) {
+                id[u] = __ldg(p.node_id + r);
+                ld4(p.q + (size_t)r * 4, q[u]);
+            }
         }
 #pragma unroll
-        for (int i = 0; i < 4; i++) red[rs][i * p.K + c] = acc[i].total();
+        for (int u = 0; u < U; u++) {
+            if (r0 + u * RG >= r_end) continue;
+            const T g = srv_probe(p, sd, col, id[u]);
+#pragma unroll
+            for (int i = 0; i < 4; i++) acc[i].add(q[u][i] * g);
+            sg.add(g);
+            sq.add((c & 2) ? ((c & 1) ? q[u][3] : q[u][2]) : ((c & 1) ? q[u][1] : q[u][0]));
+        }
     }
+#pragma unroll
+    for (int i = 0; i < 4; i++) red[rs][i][c] = acc[i].total();
+    red[rs][4][c] = sg.total();
+    red[rs][5][c] = sq.total();
     __syncthreads();
-    const int W = 4 * p.K;
-    for (int w = threadIdx.x; w < W; w += blockDim.x) {
+    const int W = kSrvW(p.K);
+    for (int w = threadIdx.x; w < W; w += VNE_THREADS) {
+        const int i = w < 5 * p.K ? w / p.K : 5, cc = w < 5 * p.K ? w % p.K : w - 5 * p.K;
         double v = 0.0;
-        for (int q = 0; q < VNE_THREADS / 64; q++) v += red[q][w];
+#pragma unroll
+        for (int k = 0; k < RG; k++) v += red[k][i][cc];
         p.part[(size_t)blockIdx.x * W + w] = v;
     }
-    __shared__ double tot[4 * 256];
-    if (srv_last_reduce(p.part, p.counter + s, p.seg_tb[s], p.seg_tc[s], W, tot))
-        for (int w = threadIdx.x; w < W; w += blockDim.x) p.coef[(size_t)s * W + w] = tot[w];
 }
 
-// pass 2 (center = 0): column sums of g' = g - Q coef -> mean; pass 3
-// (center = 1): c = g' - mean written to w1, ||c||^2 -> norm2, sigma_1
+// out[segment][w] = sum of the segment's partials of value w < W, in a fixed
+// order: 32 values per CTA, eight slots each.  grid (segments, ceil(W / 32)).
+__global__ void __launch_bounds__(VNE_THREADS) k_srv_sum(const double* __restrict__ part, const int32_t* seg_tb,
+                                                         const int32_t* seg_tc, int W, double* __restrict__ out) {
+    const int s = blockIdx.x, w = blockIdx.y * 32 + threadIdx.x % 32, k = threadIdx.x / 32;
+    const int count = seg_tc[s] * kSrvSub;
+    if (count == 0) return;
+    __shared__ double red[8][32];
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    if (w < W) {
+        const double* src = part + (size_t)seg_tb[s] * kSrvSub * W + w;
+        int i = k;
+        for (; i + 24 < count; i += 32) {
+#pragma unroll
+            for (int u = 0; u < 4; u++) acc[u] += src[(size_t)(i + 8 * u) * W];
+        }
+        for (int u = 0; i < count; i += 8, u++) acc[u & 3] += src[(size_t)i * W];
+    }
+    red[k][threadIdx.x % 32] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    __syncthreads();
+    if (threadIdx.x < 32 && w < W) {
+        double x = 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; q++) x += red[q][threadIdx.x];
+        out[(size_t)s * W + w] = x;
+    }
+}
+
+// pass 2: c = g - Q coef - mean written to w1, partial sums of c^2
 template <typename T, int KS>
-__global__ void __launch_bounds__(VNE_THREADS) k_srv_pass(SrvStartParams<T> p, int center) {
-    const RowTile t = p.tiles[p.tile_list[blockIdx.x]];
-    const int s = t.seg, c0 = threadIdx.x % 64, rs = threadIdx.x / 64;
-    __shared__ double red[VNE_THREADS / 64][256];
-    for (int c = c0; c < p.K; c += 64) {
+__global__ void __launch_bounds__(VNE_THREADS) k_srv_center(SrvStartParams<T> p) {
+    constexpr int U = 4, RG = VNE_THREADS / 64;
+    const RowTile t = p.tiles[p.tile_list[blockIdx.x / kSrvSub]];
+    const int s = t.seg, c = threadIdx.x % 64, rs = threadIdx.x / 64;
+    int r_begin, r_end;
+    srv_rows(p, t, r_begin, r_end);
+    __shared__ double red[RG][64];
+    __shared__ T s_cf[4][64], s_mu[64];
+    if (threadIdx.x < p.K) {
+        const double* sums = p.coef + (size_t)s * kSrvW(p.K);
+        double m = sums[4 * p.K + c];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            s_cf[i][c] = (T)sums[i * p.K + c];
+            m -= sums[i * p.K + c] * sums[5 * p.K + i];
+        }
+        s_mu[c] = (T)(m / (double)p.seg[s].rows);
+    }
+    __syncthreads();
+    RowSum<T> acc;
+    if (c < p.K) {
         T cf[4];
 #pragma unroll
-        for (int i = 0; i < 4; i++) cf[i] = (T)p.coef[((size_t)s * 4 + i) * p.K + c];
-        const T mu = center ? (T)p.mean[(size_t)s * p.K + c] : (T)0;
+        for (int i = 0; i < 4; i++) cf[i] = s_cf[i][c];
+        const T mu = s_mu[c];
         T* out = p.w1 + (size_t)(c / KS) * p.n_total * KS + (c % KS);
-        RowSum<T> acc;
-        for (int r = t.row_begin + rs; r < t.row_end; r += VNE_THREADS / 64) {
-            T v = srv_probe(p, s, c, r);
+        const uint64_t sd = p.seg_seed[s], col = (uint64_t)(p.seg_col0[s] + c);
+        for (int r0 = r_begin + rs; r0 < r_end; r0 += U * RG) {
+            int id[U];
+            T q[U][4];
 #pragma unroll
-            for (int i = 0; i < 4; i++) v -= p.q[(size_t)r * 4 + i] * cf[i];
-            if (center) {
+            for (int u = 0; u < U; u++) {
+                const int r = r0 + u * RG;
+                if (r < r_end) {
+                    id[u] = __ldg(p.node_id + r);
+                    ld4(p.q + (size_t)r * 4, q[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int r = r0 + u * RG;
+                if (r >= r_end) continue;
+                T v = srv_probe(p, sd, col, id[u]);
+#pragma unroll
+                for (int i = 0; i < 4; i++) v -= q[u][i] * cf[i];
                 v -= mu;
                 out[(size_t)r * KS] = v;
                 acc.add(v * v);
-            } else {
-                acc.add(v);
             }
         }
-        red[rs][c] = acc.total();
     }
+    red[rs][c] = acc.total();
     __syncthreads();
-    for (int w = threadIdx.x; w < p.K; w += blockDim.x) {
+    if (threadIdx.x < p.K) {
         double v = 0.0;
-        for (int q = 0; q < VNE_THREADS / 64; q++) v += red[q][w];
-        p.part[(size_t)blockIdx.x * p.K + w] = v;
+#pragma unroll
+        for (int k = 0; k < RG; k++) v += red[k][c];
+        p.part[(size_t)blockIdx.x * p.K + c] = v;
     }
-    __shared__ double tot[256];
-    if (srv_last_reduce(p.part, p.counter + s, p.seg_tb[s], p.seg_tc[s], p.K, tot)) {
-        for (int w = threadIdx.x; w < p.K; w += blockDim.x) {
-            const size_t o = (size_t)s * p.K + w;
-            if (center) {
-                p.norm2[o] = tot[w];
-                p.sig1[o] = tot[w] > 0.0 ? 1.0 / sqrt(tot[w]) : 0.0;
-            } else {
-                p.mean[o] = tot[w] / (double)p.seg[s].rows;
-            }
-        }
-    }
+}
+
+// ||c||^2 and sigma_1 of the listed segments from k_srv_sum's totals
+__global__ void k_srv_norms(const double* __restrict__ sums, const int32_t* seg_tc, int K, double* norm2,
+                            double* sig1) {
+    const int s = blockIdx.x;
+    if (seg_tc[s] == 0 || (int)threadIdx.x >= K) return;
+    const size_t o = (size_t)s * K + threadIdx.x;
+    const double x = sums[o];
+    norm2[o] = x;
+    sig1[o] = x > 0.0 ? 1.0 / sqrt(x) : 0.0;
 }
 
 // ---------------------------------------------------------------------------
@@ -1448,10 +1511,13 @@ cudaError_t launch_update(const StepParams<T>& p, int ks, int panels, cudaStream
 template <typename T>
 cudaError_t launch_srv_start(const SrvStartParams<T>& p, int ks, cudaStream_t st) {
     if (p.ntiles == 0) return cudaSuccess;
-    if (p.K < 1 || p.K > 64 || p.K % ks) return cudaErrorInvalidValue;
-    k_srv_coef<T><<<p.ntiles, VNE_THREADS, 0, st>>>(p);
-    VNE_DISPATCH_KS(T, ks, (k_srv_pass<T, KS><<<p.ntiles, VNE_THREADS, 0, st>>>(p, 0)));
-    VNE_DISPATCH_KS(T, ks, (k_srv_pass<T, KS><<<p.ntiles, VNE_THREADS, 0, st>>>(p, 1)));
+    if (p.K < 4 || p.K > 64 || p.K % ks) return cudaErrorInvalidValue;
+    const int W = kSrvW(p.K), ctas = p.ntiles * kSrvSub;
+    k_srv_coef<T><<<ctas, VNE_THREADS, 0, st>>>(p);
+    k_srv_sum<<<dim3(p.nseg, (W + 31) / 32), VNE_THREADS, 0, st>>>(p.part, p.seg_tb, p.seg_tc, W, p.coef);
+    VNE_DISPATCH_KS(T, ks, (k_srv_center<T, KS><<<ctas, VNE_THREADS, 0, st>>>(p)));
+    k_srv_sum<<<dim3(p.nseg, (p.K + 31) / 32), VNE_THREADS, 0, st>>>(p.part, p.seg_tb, p.seg_tc, p.K, p.mean);
+    k_srv_norms<<<p.nseg, 64, 0, st>>>(p.mean, p.seg_tc, p.K, p.norm2, p.sig1);
     return cudaGetLastError();
 }
 

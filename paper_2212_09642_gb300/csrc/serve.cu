@@ -243,7 +243,7 @@ void arena_alloc(vne_server* S, bool fp64) {
     S->psi = (double*)take((size_t)SK * 8);
     S->est = (double*)take((size_t)3 * SK * 8);
     S->scale = (double*)take((size_t)SK * 8);
-    S->coef = (double*)take((size_t)kSketchCols * SK * 8);
+    S->coef = (double*)take((size_t)S->nseg * kSrvW(S->K) * 8);
     if (fp64 && S->ks > 16) {  // FP64 panels hold 4, 8 or 16 columns
         S->ks = 16;
         S->K = ((S->K + 15) / 16) * 16;
@@ -565,14 +565,14 @@ int tick_impl(vne_server* S) {
         sp.norm2 = S->norm2;
         sp.sig1 = S->sigma;
         sp.w1 = (T*)S->slot0;
-        sp.part = ws_get_t<double>(ctx, "srv.part", tlist.size() * kSketchCols * K);
-        sp.counter = ws_get_t<uint32_t>(ctx, "srv.counter", S->nseg);
+        sp.part = ws_get_t<double>(ctx, "srv.part", tlist.size() * kSrvSub * kSrvW(K));
+        sp.nseg = S->nseg;
         sp.ntiles = (int32_t)tlist.size();
         sp.K = K;
         sp.n_total = P.n_total;
         sp.gaussian = S->opt.gaussian_probes != 0;
         VNE_TRY_CUDA(ctx, launch_srv_start<T>(sp, ks, st));
-        ctx->launches += 3;
+        ctx->launches += 5;
     }
     StepParams<T> p;
     memset(&p, 0, sizeof(p));
