@@ -108,26 +108,27 @@ __device__ __forceinline__ T source_value_t(const StartSource& S, const T* panel
 }
 
 // Per-thread sum over its rows: FP64 throughout for FP64 blocks; for FP32
-// blocks FP32 partial sums of 16 rows, added in FP64 (a Rademacher column's
-// partial sums are exact).
+// blocks FP32 partial sums of at most kRun rows, which the caller's loop hands to
+// the FP64 sum by flush() (a Rademacher column's partial sums are exact).  The
+// loops are nested for it: a flush under a condition on a counter is compiled to
+// a predicated FP64 addition per row, and a predicated-off FP64 instruction
+// holds the FP64 port for its 64 cycles like any other (the served first pass,
+// six sums: 54 us with the counter, 11 with nested loops; centring 150,000 x 64
+// FP32 entries: 62 us, 19).
+constexpr int kRun = 16;
 template <typename T>
 struct RowSum {
     double acc = 0.0;
     T part = (T)0;
-    int cnt = 0;
     __device__ __forceinline__ void add(T v) {
-        if (sizeof(T) == 8) {
-            acc += (double)v;
-            return;
-        }
-        part += v;
-        if (++cnt == 16) {
-            acc += (double)part;
-            part = (T)0;
-            cnt = 0;
-        }
+        if (sizeof(T) == 8) acc += (double)v;
+        else part += v;
     }
-    __device__ __forceinline__ double total() const { return acc + (double)part; }
+    __device__ __forceinline__ void flush() {
+        if (sizeof(T) == 8) return;
+        acc += (double)part;
+        part = (T)0;
+    }
 };
 
 // Four consecutive entries of one row of a panel (16-byte aligned: the
@@ -260,18 +261,23 @@ __global__ void __launch_bounds__(VNE_THREADS, 4) k_start_mean(StartParams<T> p)
         for (int j = 0; j < 4; j++) sum[j] = rq.live[j] ? (double)(rows - 2 * neg[j]) : 0.0;
     } else {
         RowSum<T> rs[4];
-        for (int r = t.row_begin + rsub; r < t.row_end; r += RPP) {
-            const int id = p.node_id ? __ldg(p.node_id + r) : r - sg.row_begin;
-            T v[4];
+        for (int r0 = t.row_begin + rsub; r0 < t.row_end; r0 += kRun * RPP) {
+            const int r1 = min(t.row_end, r0 + kRun * RPP);
+            for (int r = r0; r < r1; r += RPP) {
+                const int id = p.node_id ? __ldg(p.node_id + r) : r - sg.row_begin;
+                T v[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                v[j] = source_value_t<T, KS>(p.src, p.panel_src, r, id, gc0 + j, p.n_total, t.seg);
-                rs[j].add(v[j]);
+                for (int j = 0; j < 4; j++) {
+                    v[j] = source_value_t<T, KS>(p.src, p.panel_src, r, id, gc0 + j, p.n_total, t.seg);
+                    rs[j].add(v[j]);
+                }
+                st4(out + (size_t)r * KS + c0, v);
             }
-            st4(out + (size_t)r * KS + c0, v);
+#pragma unroll
+            for (int j = 0; j < 4; j++) rs[j].flush();
         }
 #pragma unroll
-        for (int j = 0; j < 4; j++) sum[j] = rs[j].total();
+        for (int j = 0; j < 4; j++) sum[j] = rs[j].acc;
     }
     cta_column_partials<KS, sizeof(T) == 8>(sum, rsub, c0, p.part + ((size_t)panel * p.tiles_per_panel + tile) * KS);
     __shared__ double tot[KS];
@@ -341,28 +347,34 @@ __global__ void __launch_bounds__(VNE_THREADS, 3) k_start_center(StartParams<T> 
             }
         } else {
             RowSum<T> rs[4];
-            for (int r0 = t.row_begin + rsub; r0 < t.row_end; r0 += 4 * RPP) {
-                T v[4][4];
+            for (int rb = t.row_begin + rsub; rb < t.row_end; rb += kRun * RPP) {
+                const int re = min(t.row_end, rb + kRun * RPP);
+#pragma unroll 1
+                for (int r0 = rb; r0 < re; r0 += 4 * RPP) {
+                    T v[4][4];
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const int r = r0 + u * RPP;
-                    if (r < t.row_end) ld4(out + (size_t)r * KS + c0, v[u]);
-                }
+                    for (int u = 0; u < 4; u++) {
+                        const int r = r0 + u * RPP;
+                        if (r < re) ld4(out + (size_t)r * KS + c0, v[u]);
+                    }
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const int r = r0 + u * RPP;
-                    if (r < t.row_end) {
+                    for (int u = 0; u < 4; u++) {
+                        const int r = r0 + u * RPP;
+                        if (r < re) {
 #pragma unroll
-                        for (int j = 0; j < 4; j++) {
-                            v[u][j] = live[j] ? v[u][j] - mu[j] : (T)0;
-                            rs[j].add(v[u][j] * v[u][j]);
+                            for (int j = 0; j < 4; j++) {
+                                v[u][j] = live[j] ? v[u][j] - mu[j] : (T)0;
+                                rs[j].add(v[u][j] * v[u][j]);
+                            }
+                            st4(out + (size_t)r * KS + c0, v[u]);
                         }
-                        st4(out + (size_t)r * KS + c0, v[u]);
                     }
                 }
+#pragma unroll
+                for (int j = 0; j < 4; j++) rs[j].flush();
             }
 #pragma unroll
-            for (int j = 0; j < 4; j++) sum[j] = rs[j].total();
+            for (int j = 0; j < 4; j++) sum[j] = rs[j].acc;
         }
     } else if (p.src.kind == SRC_RADEMACHER && !p.src.gaussian) {
         const RadQuad rq(p.src, t.seg, gc0);
@@ -372,18 +384,23 @@ __global__ void __launch_bounds__(VNE_THREADS, 3) k_start_center(StartParams<T> 
         for (int j = 0; j < 4; j++) sum[j] = rq.live[j] ? (double)rows : 0.0;
     } else {
         RowSum<T> rs[4];
-        for (int r = t.row_begin + rsub; r < t.row_end; r += RPP) {
-            const int id = p.node_id ? __ldg(p.node_id + r) : r - sg.row_begin;
-            T v[4];
+        for (int r0 = t.row_begin + rsub; r0 < t.row_end; r0 += kRun * RPP) {
+            const int r1 = min(t.row_end, r0 + kRun * RPP);
+            for (int r = r0; r < r1; r += RPP) {
+                const int id = p.node_id ? __ldg(p.node_id + r) : r - sg.row_begin;
+                T v[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                v[j] = source_value_t<T, KS>(p.src, p.panel_src, r, id, gc0 + j, p.n_total, t.seg);
-                rs[j].add(v[j] * v[j]);
+                for (int j = 0; j < 4; j++) {
+                    v[j] = source_value_t<T, KS>(p.src, p.panel_src, r, id, gc0 + j, p.n_total, t.seg);
+                    rs[j].add(v[j] * v[j]);
+                }
+                st4(out + (size_t)r * KS + c0, v);
             }
-            st4(out + (size_t)r * KS + c0, v);
+#pragma unroll
+            for (int j = 0; j < 4; j++) rs[j].flush();
         }
 #pragma unroll
-        for (int j = 0; j < 4; j++) sum[j] = rs[j].total();
+        for (int j = 0; j < 4; j++) sum[j] = rs[j].acc;
     }
     cta_column_partials<KS, sizeof(T) == 8>(sum, rsub, c0, p.part + ((size_t)panel * p.tiles_per_panel + tile) * KS);
     __shared__ double tot[KS];
@@ -409,7 +426,7 @@ __global__ void __launch_bounds__(VNE_THREADS, 3) k_start_center(StartParams<T> 
 // g' = g - Q coef follow from the sums of g and of Q's columns, which the first
 // pass takes along.  The probes are hashed again in the second pass.  Measured
 // per tick with starting blocks, served mix of 32 queries: 144 us with one CTA
-// per tile and three passes, 76 us now.
+// per tile and three passes, 27 us now.
 
 template <typename T>
 __device__ __forceinline__ T srv_probe(const SrvStartParams<T>& p, uint64_t sd, uint64_t col, int id) {
@@ -436,31 +453,39 @@ __global__ void __launch_bounds__(VNE_THREADS) k_srv_coef(SrvStartParams<T> p) {
     // products in the vector precision, runs of 16 rows summed in FP64
     RowSum<T> acc[4], sg, sq;
     const uint64_t sd = p.seg_seed[s], col = (uint64_t)(p.seg_col0[s] + c);
-    for (int r0 = r_begin + rs; r0 < r_end; r0 += U * RG) {
-        int id[U];
-        T q[U][4];
+    for (int rb = r_begin + rs; rb < r_end; rb += kRun * RG) {
+        const int re = min(r_end, rb + kRun * RG);
+#pragma unroll 1
+        for (int r0 = rb; r0 < re; r0 += U * RG) {
+            int id[U];
+            T q[U][4];
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int r = r0 + u * RG;
-            if (r < r_end) {
-                id[u] = __ldg(p.node_id + r);
-                ld4(p.q + (size_t)r * 4, q[u]);
+            for (int u = 0; u < U; u++) {
+                const int r = r0 + u * RG;
+                if (r < re) {
+                    id[u] = __ldg(p.node_id + r);
+                    ld4(p.q + (size_t)r * 4, q[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (r0 + u * RG >= re) continue;
+                const T g = srv_probe(p, sd, col, id[u]);
+#pragma unroll
+                for (int i = 0; i < 4; i++) acc[i].add(q[u][i] * g);
+                sg.add(g);
+                sq.add((c & 2) ? ((c & 1) ? q[u][3] : q[u][2]) : ((c & 1) ? q[u][1] : q[u][0]));
             }
         }
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-            if (r0 + u * RG >= r_end) continue;
-            const T g = srv_probe(p, sd, col, id[u]);
-#pragma unroll
-            for (int i = 0; i < 4; i++) acc[i].add(q[u][i] * g);
-            sg.add(g);
-            sq.add((c & 2) ? ((c & 1) ? q[u][3] : q[u][2]) : ((c & 1) ? q[u][1] : q[u][0]));
-        }
+        for (int i = 0; i < 4; i++) acc[i].flush();
+        sg.flush();
+        sq.flush();
     }
 #pragma unroll
-    for (int i = 0; i < 4; i++) red[rs][i][c] = acc[i].total();
-    red[rs][4][c] = sg.total();
-    red[rs][5][c] = sq.total();
+    for (int i = 0; i < 4; i++) red[rs][i][c] = acc[i].acc;
+    red[rs][4][c] = sg.acc;
+    red[rs][5][c] = sq.acc;
     __syncthreads();
     const int W = kSrvW(p.K);
     for (int w = threadIdx.x; w < W; w += VNE_THREADS) {
@@ -529,31 +554,36 @@ __global__ void __launch_bounds__(VNE_THREADS) k_srv_center(SrvStartParams<T> p)
         const T mu = s_mu[c];
         T* out = p.w1 + (size_t)(c / KS) * p.n_total * KS + (c % KS);
         const uint64_t sd = p.seg_seed[s], col = (uint64_t)(p.seg_col0[s] + c);
-        for (int r0 = r_begin + rs; r0 < r_end; r0 += U * RG) {
-            int id[U];
-            T q[U][4];
+        for (int rb = r_begin + rs; rb < r_end; rb += kRun * RG) {
+            const int re = min(r_end, rb + kRun * RG);
+#pragma unroll 1
+            for (int r0 = rb; r0 < re; r0 += U * RG) {
+                int id[U];
+                T q[U][4];
 #pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int r = r0 + u * RG;
-                if (r < r_end) {
-                    id[u] = __ldg(p.node_id + r);
-                    ld4(p.q + (size_t)r * 4, q[u]);
+                for (int u = 0; u < U; u++) {
+                    const int r = r0 + u * RG;
+                    if (r < re) {
+                        id[u] = __ldg(p.node_id + r);
+                        ld4(p.q + (size_t)r * 4, q[u]);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const int r = r0 + u * RG;
+                    if (r >= re) continue;
+                    T v = srv_probe(p, sd, col, id[u]);
+#pragma unroll
+                    for (int i = 0; i < 4; i++) v -= q[u][i] * cf[i];
+                    v -= mu;
+                    out[(size_t)r * KS] = v;
+                    acc.add(v * v);
                 }
             }
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int r = r0 + u * RG;
-                if (r >= r_end) continue;
-                T v = srv_probe(p, sd, col, id[u]);
-#pragma unroll
-                for (int i = 0; i < 4; i++) v -= q[u][i] * cf[i];
-                v -= mu;
-                out[(size_t)r * KS] = v;
-                acc.add(v * v);
-            }
+            acc.flush();
         }
     }
-    red[rs][c] = acc.total();
+    red[rs][c] = acc.acc;
     __syncthreads();
     if (threadIdx.x < p.K) {
         double v = 0.0;

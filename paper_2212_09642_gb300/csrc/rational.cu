@@ -136,40 +136,40 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgSta
         acc[q] = 0.0;
         accf[q] = (T)0;
     }
-    int cnt = 0;
-    for (int r0 = t.row_begin + rs; r0 < t.row_end; r0 += U * RPI) {
-        T rv[U][CPL], qv[U][CPL];
+    // runs of 16 rows as a loop of its own: a flush under a condition would be a
+    // predicated FP64 addition per iteration, which holds the FP64 port
+    for (int rb = t.row_begin + rs; rb < t.row_end; rb += 16 * RPI) {
+        const int re = min(t.row_end, rb + 16 * RPI);
+#pragma unroll 1
+        for (int r0 = rb; r0 < re; r0 += U * RPI) {
+            T rv[U][CPL], qv[U][CPL];
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int r = r0 + u * RPI;
-            if (r < t.row_end) {
-                load_lane(R + (size_t)r * KS + cofs, rv[u]);
-                load_lane_stream(Q + (size_t)r * KS + cofs, qv[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            const int r = r0 + u * RPI;
-            if (r < t.row_end) {
-#pragma unroll
-                for (int q = 0; q < CPL; q++) {
-                    rv[u][q] -= a[q] * qv[u][q];
-                    accf[q] += rv[u][q] * rv[u][q];
+            for (int u = 0; u < U; u++) {
+                const int r = r0 + u * RPI;
+                if (r < re) {
+                    load_lane(R + (size_t)r * KS + cofs, rv[u]);
+                    load_lane_stream(Q + (size_t)r * KS + cofs, qv[u]);
                 }
-                store_lane(Rn + (size_t)r * KS + cofs, rv[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int r = r0 + u * RPI;
+                if (r < re) {
+#pragma unroll
+                    for (int q = 0; q < CPL; q++) {
+                        rv[u][q] -= a[q] * qv[u][q];
+                        accf[q] += rv[u][q] * rv[u][q];
+                    }
+                    store_lane(Rn + (size_t)r * KS + cofs, rv[u]);
+                }
             }
         }
-        if ((cnt += U) == 16) {
 #pragma unroll
-            for (int q = 0; q < CPL; q++) {
-                acc[q] += (double)accf[q];
-                accf[q] = (T)0;
-            }
-            cnt = 0;
+        for (int q = 0; q < CPL; q++) {
+            acc[q] += (double)accf[q];
+            accf[q] = (T)0;
         }
     }
-#pragma unroll
-    for (int q = 0; q < CPL; q++) acc[q] += (double)accf[q];
     if (CLUSTER) {
         __shared__ double runs[CPL][VNE_THREADS];
 #pragma unroll
