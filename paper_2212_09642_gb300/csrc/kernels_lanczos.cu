@@ -21,6 +21,7 @@
 // CTAs; the cross-CTA sums are done by the last CTA to arrive for each
 // (panel, segment), in a fixed order, so results are bit-reproducible.
 #include "common.cuh"
+#include "gauss.cuh"
 #include "kernels.h"
 #include "reduce.cuh"
 
@@ -46,8 +47,7 @@ __device__ __forceinline__ double gaussian_entry(uint64_t s, uint64_t col, uint6
     const uint64_t h1 = mix64((((col << 32) | node) ^ s) + 0x9E3779B97F4A7C15ULL);
     const uint64_t h2 = mix64(h1 + 0x9E3779B97F4A7C15ULL);
     const double u1 = ((double)(h1 >> 11) + 0.5) * 0x1.0p-53;
-    const double u2 = (double)(h2 >> 11) * 0x1.0p-53;
-    return sqrt(-2.0 * log(u1)) * cos(6.283185307179586 * u2);
+    return gauss_sqrt(2.0 * gauss_neg_log(u1)) * gauss_cos(h2 >> 11);
 }
 
 // Start-vector source value for packed row r (local node id `id`, segment
