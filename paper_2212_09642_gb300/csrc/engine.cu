@@ -499,6 +499,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
         for (int j = j_begin; j <= j_end; j++) {
             p.first = (j == 1);
             p.renorm = 0;
+            p.no_norm = reorth == 1;
             p.w_cur = slot(j);
             p.w_prev = (j > 1) ? slot(j - 1) : slot(j);
             p.w_next = slot(j + 1);
@@ -626,10 +627,15 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 cp.panel_base = pb;
                 cp.jstride = m;
                 cp.tiles_per_panel = tiles;
-                for (int pass = 0; pass < 2; pass++) VNE_TRY_CUDA(ctx, launch_reorth<T>(rp, cp, ks, s));
-                p.renorm = 1;
-                VNE_TRY_CUDA(ctx, launch_update<T>(p, ks, pc, s));
-                ctx->launches += 7;
+                VNE_TRY_CUDA(ctx, launch_reorth<T>(rp, cp, ks, s));
+                rp.norm_beta = p.beta;  // the second pass takes the norm
+                rp.norm_sig_next = p.sig_next;
+                rp.norm_sig = p.sig_cur;
+                rp.norm_tau = P.segs[0].tau;
+                rp.norm_part = part_u;
+                rp.norm_counter = counter;
+                VNE_TRY_CUDA(ctx, launch_reorth<T>(rp, cp, ks, s));
+                ctx->launches += 6;
             }
         }
     };

@@ -72,6 +72,7 @@ struct StepParams {
     int32_t panel_base; // first panel of this launch (per-panel launches)
     int32_t first;   // j == 1: no previous vector
     int32_t renorm;  // update kernel: only recompute the norm of w_next in place
+    int32_t no_norm; // update kernel: leave the norm to the reorthogonalisation's last pass
     const T* w_cur;
     const T* w_prev;
     T* u;
@@ -102,6 +103,13 @@ struct ReorthParams {
     const double* coef;   // [j][K]
     const int32_t* panel_active;  // nullable: panels with no column to orthogonalise are skipped
     const uint8_t* sel;   // nullable [j][K]: a (panel, i) with no selected column is skipped
+    // launch_reorth's last pass with the norm (norm_beta set): beta_j = ||w||, sigma_{j+1}
+    double* norm_beta;     // nullable [K]
+    double* norm_sig_next; // [K]
+    const double* norm_sig; // [K] sigma_j
+    double norm_tau;       // breakdown threshold
+    double* norm_part;     // [panels][tiles * sub][KS]
+    uint32_t* norm_counter; // [panels]
 };
 
 struct ReorthCoefParams {
