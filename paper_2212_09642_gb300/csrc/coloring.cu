@@ -42,15 +42,25 @@ namespace {
 
 constexpr int kCWarps = 4;          // warps per CTA
 constexpr int kWin = 1024;          // colours per mex window (32 words of 32 bits)
-constexpr int kHashSlots = 2048;    // d >= 3: de-duplication table per warp
-constexpr int kBallCap = 1024;      // d >= 3: nodes of levels 2..d-1 kept as frontiers
+// d >= 3, per warp in shared memory: a de-duplication table of 2^TB entries (at
+// most three quarters in use) and the nodes of levels 2..d-1 kept as frontiers.
+// The table is cleared for every search and its size sets the warps per SM, and
+// the searches are chains of dependent loads, so the smallest table that cannot
+// overflow is taken (ball_table_bits).  RGG of 10^6 nodes (mean degree 6), d =
+// 3, 80 rounds: 13.4 ms with 2^11 entries (16 warps per SM), 10.0 with 2^9.
+template <int TB>
+struct BallTable {
+    static constexpr int kSlots = 1 << TB;
+    static constexpr int kBall = TB == 11 ? 1024 : kSlots * 3 / 4;
+    static constexpr int kWords = kSlots + kBall;
+};
 
 __device__ __forceinline__ int ld_color(const int32_t* p) { return __ldcg(p); }
 __device__ __forceinline__ void st_color(int32_t* p, int v) { __stcg(p, v); }
 
+template <int TB>
 __device__ __forceinline__ uint32_t hash_node(int32_t w) {
-    uint32_t x = (uint32_t)w * 0x9E3779B1u;
-    return x >> 21;  // 11 bits: kHashSlots = 2048
+    return ((uint32_t)w * 0x9E3779B1u) >> (32 - TB);
 }
 
 // The stored node of a key: its low half is the caller's id, mapped back to
@@ -103,8 +113,10 @@ __device__ __forceinline__ void visit(int32_t w, const uint64_t* __restrict__ ke
 }
 
 // Insert w into the warp's table: 1 = new, 0 = present, -1 = table full.
+template <int TB>
 __device__ __forceinline__ int table_insert(int32_t* table, int32_t w) {
-    uint32_t h = hash_node(w);
+    constexpr int kHashSlots = BallTable<TB>::kSlots;
+    uint32_t h = hash_node<TB>(w);
     for (int probe = 0; probe < kHashSlots; probe++) {
         const int32_t old = atomicCAS(&table[h], -1, w);
         if (old == -1) return 1;
@@ -119,6 +131,7 @@ __device__ __forceinline__ int table_insert(int32_t* table, int32_t w) {
 // table, new nodes are inserted and, if `append`, stored in ball[] as the
 // next frontier.  Returns true (warp-uniform) once the table overflowed or,
 // with `early`, once a blocker has been seen.
+template <int TB>
 __device__ __forceinline__ bool expand(const int32_t* fr, int cnt, const int32_t* __restrict__ rowptr,
                        const int32_t* __restrict__ col, const uint64_t* __restrict__ key, const int32_t* color,
                        BallCtx& b, WarpScratch& ws, int32_t* table, bool append, int32_t* ball, int* nball,
@@ -152,15 +165,15 @@ __device__ __forceinline__ bool expand(const int32_t* fr, int cnt, const int32_t
                 const int32_t w = col[ws.start[j] + t - ws.excl[j]];
                 visit(w, key, color, b, ws);
                 if (table) {
-                    const int r = table_insert(table, w);
+                    const int r = table_insert<TB>(table, w);
                     if (r < 0) {
                         overflow = true;
                     } else if (r == 1) {
                         const int q = atomicAdd(nins, 1);
-                        if (q >= kHashSlots * 3 / 4) overflow = true;
+                        if (q >= BallTable<TB>::kSlots * 3 / 4) overflow = true;
                         if (append) {
                             const int pos = atomicAdd(nball, 1);
-                            if (pos < kBallCap) ball[pos] = w;
+                            if (pos < BallTable<TB>::kBall) ball[pos] = w;
                             else overflow = true;
                         }
                     }
@@ -176,6 +189,7 @@ __device__ __forceinline__ bool expand(const int32_t* fr, int cnt, const int32_t
 // One search of v's d-ball with mex window [base, base + kWin).  Returns the
 // colour (>= 0), -1 when a blocker was found (*blocker set), -2 when the ball
 // did not fit the per-warp table, -3 when every colour of the window is used.
+template <int TB>
 __device__ __forceinline__ int search_ball(int32_t v, int d, int base, const int32_t* __restrict__ rowptr,
                            const int32_t* __restrict__ col, const uint64_t* __restrict__ key, const int32_t* color,
                            WarpScratch& ws, int32_t* table, int32_t* ball, int* nball, int* nins, int32_t* self,
@@ -185,35 +199,35 @@ __device__ __forceinline__ int search_ball(int32_t v, int d, int base, const int
     ws.win[lane] = 0u;
     const bool dedup = d >= 3;
     if (dedup) {
-        for (int i = lane; i < kHashSlots; i += 32) table[i] = -1;
+        for (int i = lane; i < BallTable<TB>::kSlots; i += 32) table[i] = -1;
         if (lane == 0) {
             *nball = 0;
             *nins = 0;
             *self = v;
         }
         __syncwarp();
-        if (lane == 0) table_insert(table, v);
+        if (lane == 0) table_insert<TB>(table, v);
     } else if (lane == 0) {
         *self = v;
     }
     __syncwarp();
     bool overflow = false;
-    bool stop = expand(self, 1, rowptr, col, key, color, b, ws, dedup ? table : nullptr, false, ball, nball, nins,
+    bool stop = expand<TB>(self, 1, rowptr, col, key, color, b, ws, dedup ? table : nullptr, false, ball, nball, nins,
                        overflow, early);
     if (!stop && d >= 2) {
         const int32_t rb = rowptr[v];
-        stop = expand(col + rb, rowptr[v + 1] - rb, rowptr, col, key, color, b, ws, dedup ? table : nullptr, d > 2,
+        stop = expand<TB>(col + rb, rowptr[v + 1] - rb, rowptr, col, key, color, b, ws, dedup ? table : nullptr, d > 2,
                       ball, nball, nins, overflow, early);
     }
     int lb = 0;
     for (int lev = 3; lev <= d && !stop; lev++) {
         __syncwarp();
-        const int le = min(*nball, kBallCap);
+        const int le = min(*nball, BallTable<TB>::kBall);
         if (le == lb) break;  // the ball is exhausted
         // level lev - 1 lives in ball[lb, le); the new level is appended after it
         // the last level is only visited: no insertion, so the table holds
         // the nodes within distance d - 1
-        stop = expand(ball + lb, le - lb, rowptr, col, key, color, b, ws, lev < d ? table : nullptr, lev < d, ball,
+        stop = expand<TB>(ball + lb, le - lb, rowptr, col, key, color, b, ws, lev < d ? table : nullptr, lev < d, ball,
                       nball, nins, overflow, early);
         lb = le;
     }
@@ -241,8 +255,9 @@ __device__ __forceinline__ int search_ball(int32_t v, int d, int base, const int
 // slots: round r reads cnt[r % 3], appends the nodes that stay uncoloured to
 // cnt[(r + 1) % 3] and clears cnt[(r + 2) % 3] (the input of round r - 1 and
 // the output of round r + 1).
-__global__ void __launch_bounds__(kCWarps * 32) k_color_round(ColorRound p) {
-    extern __shared__ int32_t dyn[];  // d >= 3: per warp kHashSlots table + kBallCap ball
+template <int TB>
+__global__ void __launch_bounds__(kCWarps * 32, TB == 9 ? 12 : 8) k_color_round(ColorRound p) {
+    extern __shared__ int32_t dyn[];  // d >= 3: per warp the table and the ball
     __shared__ WarpScratch ws_all[kCWarps];
     __shared__ int nball_all[kCWarps], nins_all[kCWarps];
     __shared__ int32_t self_all[kCWarps];
@@ -264,8 +279,8 @@ __global__ void __launch_bounds__(kCWarps * 32) k_color_round(ColorRound p) {
     const int32_t* in = (r & 1) ? p.list[1] : p.list[0];
     int32_t* out = (r & 1) ? p.list[0] : p.list[1];
     WarpScratch& ws = ws_all[warp];
-    int32_t* table = p.d >= 3 ? dyn + warp * (kHashSlots + kBallCap) : nullptr;
-    int32_t* ball = p.d >= 3 ? table + kHashSlots : nullptr;
+    int32_t* table = p.d >= 3 ? dyn + warp * BallTable<TB>::kWords : nullptr;
+    int32_t* ball = p.d >= 3 ? table + BallTable<TB>::kSlots : nullptr;
     const int nw = gridDim.x * kCWarps;
     // 32 list entries per warp step: each lane re-checks its node's blocker
     // (the common case, one load each; survivors appended with one atomic per
@@ -300,7 +315,7 @@ __global__ void __launch_bounds__(kCWarps * 32) k_color_round(ColorRound p) {
             int32_t blocker = -1;
             const int tries = p.tries[u];
             for (;;) {
-                res = search_ball(u, p.d, base, p.rowptr, p.col, p.key, p.color, ws, table, ball, &nball_all[warp],
+                res = search_ball<TB>(u, p.d, base, p.rowptr, p.col, p.key, p.color, ws, table, ball, &nball_all[warp],
                                   &nins_all[warp], &self_all[warp], p.inv, tries < 2, &blocker);
                 // every colour of the window is taken: the next window (the
                 // ball has at most n nodes, so this ends)
@@ -571,17 +586,54 @@ cudaError_t launch_color_init(const int32_t* rowptr, const int32_t* node_id, int
     return cudaGetLastError();
 }
 
-size_t color_round_smem(int d) { return d >= 3 ? (size_t)kCWarps * (kHashSlots + kBallCap) * sizeof(int32_t) : 0; }
+// Largest number of nodes within distance 2 of a node, from above: 1 + the sum of
+// its neighbours' degrees (each neighbour's list holds the node itself once).
+__global__ void k_ball2_bound(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col, int64_t n,
+                              int32_t* __restrict__ bound) {
+    int best = 0;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+        int64_t s = 1;
+        for (int k = rowptr[v]; k < rowptr[v + 1]; k++) {
+            const int32_t u = col[k];
+            s += rowptr[u + 1] - rowptr[u];
+        }
+        best = max(best, (int)min(s, (int64_t)1 << 30));
+    }
+    best = __reduce_max_sync(0xffffffffu, best);
+    if ((threadIdx.x & 31) == 0) atomicMax(bound, best);
+}
 
-cudaError_t launch_color_round(const ColorRound& p, cudaStream_t st) {
-    const size_t smem = color_round_smem(p.d);
+cudaError_t launch_ball2_bound(const int32_t* rowptr, const int32_t* col, int64_t n, int32_t* bound,
+                               cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_ball2_bound<<<flat_grid(n), 256, 0, st>>>(rowptr, col, n, bound);
+    return cudaGetLastError();
+}
+
+// Table for a search of distance d whose 2-balls hold at most `ball2` nodes
+// (<= 0: unknown): at d = 3 exactly the 2-ball is inserted, so a table whose
+// three quarters hold it never overflows; larger distances keep the largest.
+int ball_table_bits(int d, int ball2) {
+    if (d != 3 || ball2 <= 0) return 11;
+    return ball2 < BallTable<9>::kSlots * 3 / 4 ? 9 : (ball2 < BallTable<10>::kSlots * 3 / 4 ? 10 : 11);
+}
+
+template <int TB>
+static cudaError_t color_round_tb(const ColorRound& p, int ctas_per_sm, cudaStream_t st) {
+    const int smem = p.d >= 3 ? kCWarps * BallTable<TB>::kWords * (int)sizeof(int32_t) : 0;
     if (smem) {
-        cudaError_t e = cudaFuncSetAttribute(k_color_round, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_color_round<TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    const int grid = sm_count() * (p.d >= 3 ? 4 : 8);
-    k_color_round<<<grid, kCWarps * 32, smem, st>>>(p);
+    k_color_round<TB><<<sm_count() * ctas_per_sm, kCWarps * 32, smem, st>>>(p);
     return cudaGetLastError();
+}
+
+cudaError_t launch_color_round(const ColorRound& p, cudaStream_t st) {
+    if (p.d < 3) return color_round_tb<9>(p, 12, st);
+    if (p.table_bits == 9) return color_round_tb<9>(p, 12, st);
+    if (p.table_bits == 10) return color_round_tb<10>(p, 7, st);
+    return color_round_tb<11>(p, 4, st);
 }
 
 int color_big_ctas() { return sm_count(); }

@@ -141,6 +141,7 @@ struct vne_matrix {
     int tuned_panel = 0, tuned_item_nnz = 0, tuned_variant = 0, tuned_ipw = 1;
     bool tuned_interleave = false;
     int64_t maxdeg = 0;
+    int32_t ball2 = -1;             // bound of the nodes within distance 2 (made by the first d = 3 colouring)
     ~vne_matrix();  // frees the device arrays and the cached schedule (engine.cu)
 };
 

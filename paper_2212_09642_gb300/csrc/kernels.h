@@ -363,10 +363,14 @@ struct ColorRound {
     int32_t* bigball;   // per CTA: frontier storage
     uint32_t* epoch;    // per CTA: search counter (table entries of older searches count as empty)
     int32_t d, round;
+    int32_t table_bits;  // d >= 3: size of the per-warp table (ball_table_bits)
 };
 cudaError_t launch_color_init(const int32_t* rowptr, const int32_t* node_id, int64_t n, uint64_t* key,
                               int32_t* inv, int32_t* tries, int32_t* color, int32_t* blk, int32_t* list,
                               cudaStream_t st);
+// *bound (zeroed) = an upper bound of the nodes within distance 2 of a node.
+cudaError_t launch_ball2_bound(const int32_t* rowptr, const int32_t* col, int64_t n, int32_t* bound, cudaStream_t);
+int ball_table_bits(int d, int ball2);
 cudaError_t launch_color_round(const ColorRound& p, cudaStream_t st);
 // d >= 3: the nodes of biglist, one CTA each, with a table in global memory.
 cudaError_t launch_color_big(const ColorRound& p, cudaStream_t st);

@@ -45,6 +45,17 @@ void device_colorings(vne_matrix* M, std::vector<ColorJob>& jobs) {
         }
     }
     const int32_t n32 = (int32_t)n;
+    bool d3 = false;
+    for (const ColorJob& J : jobs) d3 = d3 || J.d == 3;
+    if (d3 && M->ball2 < 0) {
+        int32_t* b = ws_get_t<int32_t>(ctx, "col.ball2", 1, true);
+        VNE_TRY_CUDA(ctx, launch_ball2_bound(M->d_rowptr, M->d_col, n, b, ctx->stream));
+        ctx->launches++;
+        int32_t h = 0;
+        VNE_TRY_CUDA(ctx, cudaMemcpyAsync(&h, b, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+        VNE_TRY_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        M->ball2 = h;
+    }
     for (int i = 0; i < nj; i++) {
         ColorJob& J = jobs[i];
         J.st = i == 0 ? ctx->stream : ctx->color_streams[i - 1];
@@ -79,6 +90,7 @@ void device_colorings(vne_matrix* M, std::vector<ColorJob>& jobs) {
         p.ncolors = J.ctr + 3;
         p.overflow = J.ctr + 4;
         p.d = J.d;
+        p.table_bits = ball_table_bits(J.d, M->ball2);
         if (J.d >= 3) {
             // balls too large for a warp's shared-memory table go to one CTA
             // each (k_color_big); the tables start empty (epoch 0 everywhere)

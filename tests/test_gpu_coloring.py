@@ -76,6 +76,35 @@ def test_large_balls_searched_by_a_cta(vctx):
     assert s == int(want.max()) + 1
 
 
+@pytest.mark.parametrize("spokes,degree", [(2, 191), (383, 1), (2, 383), (13, 59), (1, 1535), (3, 512)])
+@pytest.mark.parametrize("d", [3, 4])
+def test_table_sizes_of_the_ball_search(vctx, spokes, degree, d):
+    """The table of a d = 3 search holds exactly the nodes within distance 2, and
+    its size is chosen by their largest number: a root with `spokes` neighbours
+    of `degree` neighbours each has 1 + spokes * degree (383, 384, 767, 768,
+    1536 and 1537: both sides of three quarters of 2^9, 2^10 and 2^11 entries),
+    joined with a small graph whose balls are much smaller."""
+    mids = 1 + np.arange(spokes)
+    leaves = 1 + spokes + np.arange(spokes * (degree - 1))
+    src = np.concatenate([np.zeros(spokes, dtype=np.int64), np.repeat(mids, degree - 1)])
+    dst = np.concatenate([mids, leaves])
+    n0 = 1 + spokes * degree
+    ws = graphs.watts_strogatz(300, 6, 0.3, 4)
+    rows = np.repeat(np.arange(ws.n), np.diff(ws.rowptr))
+    keep = rows < ws.col
+    g = graphs.from_edges(n0 + ws.n, np.concatenate([src, n0 + rows[keep]]),
+                          np.concatenate([dst, n0 + np.asarray(ws.col)[keep]]))
+    want = coloring.greedy_distance_coloring(g, d)
+    mat = vne.matrix_from_graph(vctx, g, reorder=True)
+    try:
+        got, s, rounds = vne.vne_matrix_coloring(vctx, mat, g.n, d)
+    finally:
+        vne.vne_matrix_destroy(mat)
+    assert rounds > 0
+    assert np.array_equal(got, want), int(np.sum(got != want))
+    assert s == int(want.max()) + 1
+
+
 def test_ball_beyond_the_cta_table_is_refused(vctx):
     """A hub with 200,000 neighbours at d = 3: the radius-2 ball of every leaf
     holds the whole graph, more than a CTA's table; the call reports
