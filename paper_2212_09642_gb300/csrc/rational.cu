@@ -92,13 +92,19 @@ cudaError_t launch_cg_init(CgState st, const double* norm2, cudaStream_t s) {
 // vectors.  The last CTA of a panel advances the panel's scalars, one thread
 // per (shift, column): two single-warp kernels did that before, 19 us per
 // iteration of dependent FP64 arithmetic that this tail spreads over a CTA.
+// In FP32 a CTA is short (two batches of four rows per thread), so what it does
+// before and after them counts: the first rows are loaded before the step
+// lengths are formed, and 64 registers keep four CTAs per SM (n = 10^6, 22
+// columns: 70 us at three per SM; 61 us so; loading the next rows ahead as well
+// takes 96 registers and 80 us).
 // CLUSTER (FP64, few tiles): a thread-block cluster takes a tile, each CTA one
 // run of 16 rows per thread, and CTA 0 adds the runs from distributed shared
 // memory in the order in which one CTA would have added them (n = 30,000, 16
 // columns: 32 tiles of 1888 rows, 23 us on 32 SMs; 18.6 in clusters of
 // two).
 template <typename T, int KS, bool CLUSTER>
-__global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgState st, int wi, int it) {
+__global__ void __launch_bounds__(VNE_THREADS, sizeof(T) == 8 ? 1 : 4)
+    k_cg_update(CgVectors<T> v, CgState st, int wi, int it) {
     namespace cg = cooperative_groups;
     const int csize = CLUSTER ? (int)cg::this_cluster().num_blocks() : 1;
     const int crank = CLUSTER ? (int)cg::this_cluster().block_rank() : 0;
@@ -107,7 +113,11 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgSta
     constexpr int LPR = KS / CPL;            // lanes per row
     constexpr int RPI = VNE_THREADS / LPR;   // rows per iteration
     constexpr int U = 4;
-    const int panel = v.panel_base + cta / v.tiles_per_panel, tile = cta % v.tiles_per_panel;
+    // panels in reverse order: the step kernel walked them forwards, so the last
+    // panel's q is still in L2 when this starts, and the direction pass begins
+    // on the panel whose residual this wrote last
+    const int np = (int)gridDim.x / csize / v.tiles_per_panel;
+    const int panel = v.panel_base + np - 1 - cta / v.tiles_per_panel, tile = cta % v.tiles_per_panel;
     RowTile t = v.tiles[tile];
     if (CLUSTER) {  // run crank of the tile
         t.row_begin += crank * 16 * RPI;
@@ -116,6 +126,24 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgSta
     const int sub = threadIdx.x % LPR, rs = threadIdx.x / LPR;
     const int cofs = sub * CPL;
     const size_t pofs = (size_t)panel * v.n * KS;
+    const T* __restrict__ R = v.r + pofs;
+    T* __restrict__ Rn = v.r_next + pofs;
+    const T* __restrict__ Q = v.q + pofs;
+    T rv[U][CPL], qv[U][CPL];
+    auto fetch = [&](int r0, int re) {
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int r = r0 + u * RPI;
+            if (r < re) {
+                load_lane(R + (size_t)r * KS + cofs, rv[u]);
+                load_lane_stream(Q + (size_t)r * KS + cofs, qv[u]);
+            }
+        }
+    };
+    // the first rows are on their way while the step lengths are formed (two
+    // FP64 divisions behind two loads)
+    int rb = t.row_begin + rs;
+    if (rb < t.row_end) fetch(rb, min(t.row_end, rb + 16 * RPI));
     __shared__ double s_a[KS];
     if (threadIdx.x < KS) {
         const int c = panel * KS + threadIdx.x;
@@ -126,9 +154,6 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgSta
     T a[CPL];
 #pragma unroll
     for (int q = 0; q < CPL; q++) a[q] = (T)s_a[cofs + q];
-    const T* __restrict__ R = v.r + pofs;
-    T* __restrict__ Rn = v.r_next + pofs;
-    const T* __restrict__ Q = v.q + pofs;
     double acc[CPL];
     T accf[CPL];
 #pragma unroll
@@ -138,19 +163,11 @@ __global__ void __launch_bounds__(VNE_THREADS) k_cg_update(CgVectors<T> v, CgSta
     }
     // runs of 16 rows as a loop of its own: a flush under a condition would be a
     // predicated FP64 addition per iteration, which holds the FP64 port
-    for (int rb = t.row_begin + rs; rb < t.row_end; rb += 16 * RPI) {
+    for (; rb < t.row_end; rb += 16 * RPI) {
         const int re = min(t.row_end, rb + 16 * RPI);
 #pragma unroll 1
         for (int r0 = rb; r0 < re; r0 += U * RPI) {
-            T rv[U][CPL], qv[U][CPL];
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int r = r0 + u * RPI;
-                if (r < re) {
-                    load_lane(R + (size_t)r * KS + cofs, rv[u]);
-                    load_lane_stream(Q + (size_t)r * KS + cofs, qv[u]);
-                }
-            }
+            if (r0 != t.row_begin + rs) fetch(r0, re);
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 const int r = r0 + u * RPI;
