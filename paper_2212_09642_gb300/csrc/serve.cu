@@ -167,6 +167,7 @@ struct vne_server {
     cudaEvent_t stage_ev = nullptr;  // recorded after each tick's staging copy
     char* pin = nullptr;             // pinned staging of a tick's host arrays
     size_t pin_cap = 0;
+    double* pin_out = nullptr;  // pinned destination of an evaluation's results
     struct Req {
         vne_matrix* M;
         double eps;
@@ -200,6 +201,7 @@ struct vne_server {
         dev_free(d_segs);
         if (stage_ev) cudaEventDestroy(stage_ev);
         pinned_free(pin);
+        pinned_free(pin_out);
     }
 };
 
@@ -240,8 +242,8 @@ void arena_alloc(vne_server* S, bool fp64) {
     S->sigma = (double*)take((size_t)(S->m + 1) * SK * 8);
     S->norm2 = (double*)take((size_t)SK * 8);
     S->mean = (double*)take((size_t)SK * 8);
-    S->psi = (double*)take((size_t)SK * 8);
-    S->est = (double*)take((size_t)3 * SK * 8);
+    S->est = (double*)take((size_t)4 * SK * 8);
+    S->psi = S->est + 3 * (size_t)SK;  // next to the estimates: one copy brings both
     S->scale = (double*)take((size_t)SK * 8);
     S->coef = (double*)take((size_t)S->nseg * kSrvW(S->K) * 8);
     if (fp64 && S->ks > 16) {  // FP64 panels hold 4, 8 or 16 columns
@@ -533,6 +535,9 @@ int tick_impl(vne_server* S) {
                  i_qc = add(LA.qcols.data(), LA.qcols.size() * 4), i_qm = add(LA.qm.data(), LA.qm.size() * 4),
                  i_bc = add(LA.bcols.data(), LA.bcols.size() * 4), i_bm = add(LA.bm.data(), LA.bm.size() * 4),
                  i_bl = add(LA.blam.data(), LA.blam.size() * 8);
+    // room for the second evaluation's lists (copied when they are known)
+    const size_t first_bytes = total;
+    const size_t i_b2 = add(nullptr, checking.size() * (size_t)(K - kFirst) * 16);
     if (S->stage_ev) VNE_TRY_CUDA(ctx, cudaEventSynchronize(S->stage_ev));
     if (S->pin_cap < total) {
         pinned_free(S->pin);
@@ -541,11 +546,12 @@ int tick_impl(vne_server* S) {
         VNE_TRY_CUDA(ctx, pinned_malloc((void**)&S->pin, 2 * total));
         S->pin_cap = 2 * total;
     }
+    if (!S->pin_out) VNE_TRY_CUDA(ctx, pinned_malloc((void**)&S->pin_out, (size_t)2 * SK * 8));
     char* pin = S->pin;
     for (const Part& q : parts)
-        if (q.bytes) memcpy(pin + q.off, q.src, q.bytes);
+        if (q.src && q.bytes) memcpy(pin + q.off, q.src, q.bytes);
     char* dstage = (char*)ws_get(ctx, "srv.stage", total);
-    VNE_TRY_CUDA(ctx, cudaMemcpyAsync(dstage, pin, total, cudaMemcpyHostToDevice, st));
+    VNE_TRY_CUDA(ctx, cudaMemcpyAsync(dstage, pin, first_bytes, cudaMemcpyHostToDevice, st));
     if (!S->stage_ev) VNE_TRY_CUDA(ctx, cudaEventCreateWithFlags(&S->stage_ev, cudaEventDisableTiming));
     VNE_TRY_CUDA(ctx, cudaEventRecord(S->stage_ev, st));
     auto dptr = [&](size_t i) { return (void*)(dstage + parts[i].off); };
@@ -610,7 +616,9 @@ int tick_impl(vne_server* S) {
         VNE_TRY_CUDA(ctx, launch_step_update_segj<T>(p, ks, panels, st));
         ctx->launches += 2;
     }
-    std::vector<double> hp, he;
+    // results of an evaluation: estimates, then quadratures, in pinned memory
+    // (two copies into pageable memory took 25 us of an idle GPU each time)
+    const double *he = S->pin_out, *hp = S->pin_out + SK;
     auto evaluate = [&](const Lists& L, const int32_t* qc, const int32_t* qm, const int32_t* bc, const int32_t* bm,
                         const double* bl) {
         if (L.qcols.empty() && L.bcols.empty()) return;
@@ -627,9 +635,11 @@ int tick_impl(vne_server* S) {
                                                          bc, bm, bl, mx, SK, 0.0, 1.0, S->grid, S->est,
                                                          S->est + SK, S->est + 2 * SK, S->psi, st));
             ctx->launches += 1;
-            he = download(ctx, S->est + 2 * SK, SK);
         }
-        hp = download(ctx, S->psi, SK);
+        VNE_TRY_CUDA(ctx, cudaMemcpyAsync(S->pin_out, S->est + 2 * (size_t)SK, (size_t)2 * SK * 8,
+                                          cudaMemcpyDeviceToHost, st));
+        VNE_TRY_CUDA(ctx, cudaStreamSynchronize(st));
+        if (!ctx->pending.empty()) ctx_flush_profile(ctx);
     };
     auto passes = [&](const vne_server::Req& rq, int c_begin, int c_end) {
         for (int c = c_begin; c < c_end; c++) {
@@ -649,8 +659,14 @@ int tick_impl(vne_server* S) {
     // of the first evaluation for every other column)
     if (!candidates.empty() && kFirst < K) {
         Lists LB = make_lists({}, candidates, kFirst, K);
-        evaluate(LB, nullptr, nullptr, upload(ctx, "srv.bcols", LB.bcols), upload(ctx, "srv.bm", LB.bm),
-                 upload(ctx, "srv.blam", LB.blam));
+        const size_t nb = LB.bcols.size(), ob = parts[i_b2].off;
+        memcpy(pin + ob, LB.blam.data(), nb * 8);
+        memcpy(pin + ob + nb * 8, LB.bcols.data(), nb * 4);
+        memcpy(pin + ob + nb * 12, LB.bm.data(), nb * 4);
+        VNE_TRY_CUDA(ctx, cudaMemcpyAsync(dstage + ob, pin + ob, nb * 16, cudaMemcpyHostToDevice, st));
+        VNE_TRY_CUDA(ctx, cudaEventRecord(S->stage_ev, st));
+        evaluate(LB, nullptr, nullptr, (const int32_t*)(dstage + ob + nb * 8), (const int32_t*)(dstage + ob + nb * 12),
+                 (const double*)(dstage + ob));
     }
     for (int ri : candidates)
         if (passes(S->reqs[ri], kFirst, K)) block_done[ri] = 1;
