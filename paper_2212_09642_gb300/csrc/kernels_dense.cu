@@ -9,6 +9,7 @@
 // quadrature (the Golub-Welsch weights u_{1j}^2), so the per-column kernel
 // tracks that row alone; the matvec kernel keeps the full eigenvector matrix
 // in shared memory, one warp per column, lanes owning its rows.
+#include <cooperative_groups.h>
 #include <float.h>
 #include <math.h>
 #include <stdlib.h>
@@ -1039,32 +1040,47 @@ __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
 // be positive.
 // Divided differences of f(x) = -x log x at (t, z), z = t (1 + u):
 // f[t, z] = -log t - h and f[t, t, z] = (1 - h) / (z - t) with
-// h = z (log z - log t) / (z - t) = (1 + u) log(1 + u) / u.  For |u| < 0.1 the
-// power series 1 - h = sum_{k>=1} (-1)^k u^k / (k (k + 1)) (18 terms: |u|^18 /
-// 342 < 1e-20) avoids the cancellation of the plain quotients.
-// With a Ritz value's constants this gives its term of g_m without the part
-// -2 ab gamma log t, which does not depend on z and is summed once: one
-// reciprocal and eight multiply-adds per point (four divisions and 18 in the
-// series before; a division occupies an FP64 port for 9 slots).
+// h = z (log z - log t) / (z - t) = (log z - log t) (1 + 1 / u).  For |u| < 0.1
+// the power series 1 - h = sum_{k>=1} (-1)^k u^k / (k (k + 1)) (16 terms: the
+// next are below 1e-18 of the sum) avoids the cancellation of the plain
+// quotients.  With a Ritz value's constants this gives its term of g_m without
+// the part -2 ab gamma log t, which does not depend on z and is summed once.
+// FP64 instructions are what a term costs (a warp's holds its port 64 cycles):
+// 12 in the plain form with 1 / u from a single-precision seed and one step of
+// Halley's iteration, w (1 + e + e^2) with e = 1 - u w (three instructions, error
+// e^3 < 1e-20; a division is nine, a reciprocal six), 21 by the series.
 struct GTerm {
-    double t, it, lt, ab2, c1;  // theta, 1 / theta, log theta, (a b)^2, 2 a b gamma
+    double t, it, lt, c2, c1;  // theta, 1 / theta, log theta, (a b)^2 / theta, 2 a b gamma
 };
 __device__ __forceinline__ double g_term(double z, double lz, const GTerm& p, double g) {
-    const double d = z - p.t;
-    const double u = d * p.it;
-    if (fabs((float)u) < 0.1f) {
+    const double u = (z - p.t) * p.it;
+    const float uf = (float)u;
+    if (fabsf(uf) < 0.1f) {
         double ser = 0.0;  // (1 - h) / u by Horner
 #pragma unroll
-        for (int k = 18; k >= 1; k--) ser = fma(ser, u, ((k & 1) ? -1.0 : 1.0) / (double)(k * (k + 1)));
-        g = fma(p.ab2 * p.it, ser, g);
+        for (int k = 16; k >= 1; k--) ser = fma(ser, u, ((k & 1) ? -1.0 : 1.0) / (double)(k * (k + 1)));
+        g = fma(p.c2, ser, g);
         return fma(p.c1, fma(ser, u, -1.0), g);
     }
-    const double r = 1.0 / d;
-    const double h = (lz - p.lt) * (z * r);
-    g = fma(p.ab2 * r, 1.0 - h, g);
+    double w = (double)__frcp_rn(uf);
+    if (fabsf(uf) > 1e30f) {  // the seed would leave single precision's range
+        w = 1.0 / u;
+    } else {
+        const double e = fma(-u, w, 1.0);
+        w = fma(w, fma(e, e, e), w);
+    }
+    const double h = (lz - p.lt) * (1.0 + w);
+    g = fma(p.c2 * w, 1.0 - h, g);
     return fma(-p.c1, h, g);
 }
 
+// The points are most of the work: 2 grid + n of them with n terms each, on the
+// four FP64 ports of the column's SM.  So a column may take a cluster of two, four
+// or eight CTAs: every CTA computes the spectrum (the same numbers, and no later
+// than one would), takes its share of the points, and CTA 0 reads the others'
+// minimum and maximum.  The values of the points, and so the results, do not depend on
+// the cluster's size.  Served mix of 32 queries (460 calls of 8 to 1400
+// columns, 512 points, 5 to 32 steps): 72 -> 62 us a call.
 template <int MAXM>
 __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
     k_tridiag_bounds(const double* __restrict__ alpha, const double* __restrict__ beta,
@@ -1077,14 +1093,18 @@ __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
     __shared__ GTerm G[MAXM];
     extern __shared__ double piv[];  // pivot scratch of tq_vectors
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if ((int)blockIdx.x >= count) return;
-    // entry blockIdx.x: column c (of the ld-strided arrays) after m steps,
-    // with its own upper end of the spectral interval if given
-    const int c = cols ? cols[blockIdx.x] : (int)blockIdx.x;
-    const int m = mcol ? mcol[blockIdx.x] : m_all;
-    if (lam_max_col) lam_max = lam_max_col[blockIdx.x];
+    auto cluster = cooperative_groups::this_cluster();
+    const int csize = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
+    const int entry = (int)blockIdx.x / csize;
+    if (entry >= count) return;
+    // column c (of the ld-strided arrays) after m steps, with its own upper end
+    // of the spectral interval if given; every return before the minimum is taken
+    // by all CTAs of the cluster (the same data) or by none
+    const int c = cols ? cols[entry] : entry;
+    const int m = mcol ? mcol[entry] : m_all;
+    if (lam_max_col) lam_max = lam_max_col[entry];
     auto put = [&](double lo, double hi, double est) {
-        if (tid == 0) {
+        if (tid == 0 && crank == 0) {
             lower[c] = lo;
             upper[c] = hi;
             estimate[c] = est;
@@ -1092,7 +1112,7 @@ __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
     };
     if (!tq_spectrum<MAXM>(alpha, beta, c, m, ld, S)) {
         put(nan(""), nan(""), nan(""));
-        if (psi && tid == 0) psi[c] = nan("");
+        if (psi && tid == 0 && crank == 0) psi[c] = nan("");
         return;
     }
     const int n = S.n;
@@ -1102,7 +1122,7 @@ __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
     if (!invariant || (psi && !S.fallback))
         for (int rb = 0; rb < n; rb += TqCfg<MAXM>::RB)
             tq_vectors<MAXM, false>(S, piv, rb, min(TqCfg<MAXM>::RB, n - rb));
-    if (psi) {  // the quadrature itself, from the same spectrum
+    if (psi && crank == 0) {  // the quadrature itself, from the same spectrum
         if (S.fallback) {
             if (warp == 0) quad_by_qr<MAXM>(S.a, S.b, n, sc, norm2[c], lane, psi + c);
         } else {
@@ -1124,7 +1144,7 @@ __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
         p.t = sc * S.th[j];
         p.it = 1.0 / p.t;
         p.lt = log(p.t);
-        p.ab2 = ab * ab;
+        p.c2 = ab * ab * p.it;
         p.c1 = 0.0;
         G[j] = p;
         S.c0[j] = ab;
@@ -1160,7 +1180,8 @@ __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
     const double lmin = log(lam_min), lratio = log(lam_max / lam_min), inv = grid > 1 ? 1.0 / (grid - 1) : 0.0;
     const double lstep = lratio * inv, zstep = (lam_max - lam_min) * inv;
     unsigned long long gmin = 0x7ff0000000000000ULL, gmax = 0;
-    for (int q = tid; q < npts; q += blockDim.x) {
+    for (unsigned i = crank * TqCfg<MAXM>::NT + tid; i < (unsigned)npts; i += csize * TqCfg<MAXM>::NT) {
+        const int q = (int)i;
         double z, lz;
         if (q < grid) {
             const double x = lstep * q;
@@ -1192,10 +1213,40 @@ __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
         atomicMin(&S.gmin, gmin);
         atomicMax(&S.gmax, gmax);
     }
-    __syncthreads();
-    const double lo = __longlong_as_double((long long)S.gmin), hi = __longlong_as_double((long long)S.gmax);
+    cluster.sync();
+    if (crank == 0 && tid == 0) {
+        gmin = S.gmin;
+        gmax = S.gmax;
+        for (int r = 1; r < csize; r++) {
+            gmin = min(gmin, *cluster.map_shared_rank(&S.gmin, r));
+            gmax = max(gmax, *cluster.map_shared_rank(&S.gmax, r));
+        }
+    }
+    cluster.sync();  // the other CTAs' shared memory has been read
+    const double lo = __longlong_as_double((long long)gmin), hi = __longlong_as_double((long long)gmax);
     const double nb = norm2[c];
     put(nb * lo, nb * hi, nb * sqrt(lo * hi));
+}
+
+// CTAs per column of k_tridiag_bounds: the size with the least work on the
+// fullest SM.  A CTA costs its share of the points plus a spectrum, which holds the
+// FP64 ports as long as about 80 points do (512 columns of 10 steps: 0.05 us a
+// column for the spectra, 0.32 for 522 points).
+static int bounds_cluster(int count, int64_t points) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        return 1;
+    int best = 1;
+    int64_t best_cost = 0;
+    for (int size = 1; size <= 8; size *= 2) {
+        const int64_t cost = (((int64_t)count * size + sms - 1) / sms) * (80 + points / size);
+        if (size == 1 || cost < best_cost) {
+            best = size;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
 cudaError_t launch_tridiag_bounds(const double* alpha, const double* beta, const double* norm2, const double* scale,
@@ -1213,16 +1264,28 @@ cudaError_t launch_tridiag_bounds_list(const double* alpha, const double* beta, 
     if (count <= 0) return cudaSuccess;
     // lam_min <= 0: half the smallest positive Ritz value of each column
     if ((!lam_max_col && !(lam_max > 0.0 && lam_max > lam_min)) || grid < 1) return cudaErrorInvalidValue;
+    const int size = bounds_cluster(count, 2 * (int64_t)grid + m);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = size;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
 #define VNE_BOUND_CASE(MM)                                                                                   \
     if (m <= MM) {                                                                                          \
         const int smem = TqCfg<MM>::kSmem;                                                                  \
         cudaError_t e = cudaFuncSetAttribute(k_tridiag_bounds<MM>,                                          \
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);            \
         if (e != cudaSuccess) return e;                                                                     \
-        k_tridiag_bounds<MM><<<count, TqCfg<MM>::NT, smem, st>>>(alpha, beta, norm2, scale, count, m, ld,   \
-                                                                  lam_min, lam_max, grid, lower, upper,     \
-                                                                  estimate, cols, mcol, lam_max_col, psi);  \
-        return cudaGetLastError();                                                                          \
+        cudaLaunchConfig_t cfg{};                                                                           \
+        cfg.gridDim = dim3((unsigned)(count * size));                                                       \
+        cfg.blockDim = dim3(TqCfg<MM>::NT);                                                                 \
+        cfg.dynamicSmemBytes = smem;                                                                        \
+        cfg.stream = st;                                                                                    \
+        cfg.attrs = at;                                                                                     \
+        cfg.numAttrs = 1;                                                                                   \
+        e = cudaLaunchKernelEx(&cfg, k_tridiag_bounds<MM>, alpha, beta, norm2, scale, count, m, ld, lam_min, \
+                               lam_max, grid, lower, upper, estimate, cols, mcol, lam_max_col, psi);        \
+        return e != cudaSuccess ? e : cudaGetLastError();                                                   \
     }
     VNE_BOUND_CASE(32)
     VNE_BOUND_CASE(64)

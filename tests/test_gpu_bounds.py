@@ -54,6 +54,24 @@ def test_bounds_match_oracle_and_bracket(vctx, name, g, seed):
         assert lo[0] <= est[0] <= hi[0]
 
 
+@pytest.mark.parametrize("m", [3, 24, 40, 70])
+@pytest.mark.parametrize("grid", [1, 13, 200, 1000])
+def test_bounds_do_not_depend_on_the_number_of_columns(vctx, m, grid):
+    """A column takes a cluster of 8, 4, 2 or 1 CTAs by how many columns the call
+    has; the points' values do not depend on it: the same bits."""
+    l2, ln, exact, runs = _case(graphs.watts_strogatz(400, 6, 0.3, 4), 6, (m,))
+    _, psi, alpha, beta, nb = runs[0]
+    assert len(alpha) == m
+    want = None
+    for count in (1, 20, 40, 80, 400):
+        got = vne.vne_quadrature_bounds(vctx, np.tile(alpha, (count, 1)), np.tile(beta[:m], (count, 1)),
+                                        np.full(count, nb), 1.0, l2, ln, grid)
+        want = want if want is not None else [x[0] for x in got]
+        for x, w in zip(got, want):
+            assert np.all(x == w), count
+    assert 0.0 <= want[0] <= want[2] <= want[1]
+
+
 def test_bounds_zero_after_breakdown(vctx):
     # K_n: the Krylov space of a desingularised vector is invariant after one step
     g = graphs.complete(30)
