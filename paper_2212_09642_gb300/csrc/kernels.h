@@ -268,6 +268,7 @@ struct CgVectors {
     int32_t panel_base;     // first panel of the launch
     int32_t sub;            // direction kernel: CTAs per row tile
     int32_t max_tile_rows;  // rows of the largest tile
+    int32_t group;          // update kernel: row tiles per CTA (set by the launcher)
     int32_t sm_count;
     const RowTile* tiles;
     const T* r;  // residual r_k

@@ -92,11 +92,12 @@ cudaError_t launch_cg_init(CgState st, const double* norm2, cudaStream_t s) {
 // vectors.  The last CTA of a panel advances the panel's scalars, one thread
 // per (shift, column): two single-warp kernels did that before, 19 us per
 // iteration of dependent FP64 arithmetic that this tail spreads over a CTA.
-// In FP32 a CTA is short (two batches of four rows per thread), so what it does
-// before and after them counts: the first rows are loaded before the step
-// lengths are formed, and 64 registers keep four CTAs per SM (n = 10^6, 22
-// columns: 70 us at three per SM; 61 us so; loading the next rows ahead as well
-// takes 96 registers and 80 us).
+// In FP32 a tile is short (two batches of four rows per thread), so what a CTA
+// does before and after the rows counts: the first rows are loaded before the
+// step lengths are formed, 64 registers keep four CTAs per SM (n = 10^6, 22
+// columns: 70 us at three per SM; 62 so; loading the next rows ahead as well
+// takes 96 registers and 80 us), and a CTA takes several tiles of a long panel
+// (cg_update_ks).
 // CLUSTER (FP64, few tiles): a thread-block cluster takes a tile, each CTA one
 // run of 16 rows per thread, and CTA 0 adds the runs from distributed shared
 // memory in the order in which one CTA would have added them (n = 30,000, 16
@@ -116,9 +117,11 @@ __global__ void __launch_bounds__(VNE_THREADS, sizeof(T) == 8 ? 1 : 4)
     // panels in reverse order: the step kernel walked them forwards, so the last
     // panel's q is still in L2 when this starts, and the direction pass begins
     // on the panel whose residual this wrote last
-    const int np = (int)gridDim.x / csize / v.tiles_per_panel;
-    const int panel = v.panel_base + np - 1 - cta / v.tiles_per_panel, tile = cta % v.tiles_per_panel;
-    RowTile t = v.tiles[tile];
+    const int tiles = (v.tiles_per_panel + v.group - 1) / v.group;  // CTAs per panel
+    const int np = (int)gridDim.x / csize / tiles;
+    const int panel = v.panel_base + np - 1 - cta / tiles, tile = cta % tiles;
+    RowTile t = v.tiles[tile * v.group];
+    t.row_end = v.tiles[min(v.tiles_per_panel, (tile + 1) * v.group) - 1].row_end;
     if (CLUSTER) {  // run crank of the tile
         t.row_begin += crank * 16 * RPI;
         t.row_end = min(t.row_end, t.row_begin + 16 * RPI);
@@ -207,25 +210,25 @@ __global__ void __launch_bounds__(VNE_THREADS, sizeof(T) == 8 ? 1 : 4)
     double tot;
     if (kSerial) cta_colsum_serial<KS, CPL>(acc, red, tot);
     else cta_colsum<KS, CPL>(acc, red, tot);
-    if (threadIdx.x < KS) v.part[((size_t)panel * v.tiles_per_panel + tile) * KS + threadIdx.x] = tot;
+    if (threadIdx.x < KS) v.part[((size_t)panel * tiles + tile) * KS + threadIdx.x] = tot;
     __shared__ double s_rho[KS];
     if (kSerial) {
         __shared__ int s_last;
         __threadfence();
         __syncthreads();
-        if (threadIdx.x == 0) s_last = (atomicAdd(v.counter + panel, 1u) == (unsigned)(v.tiles_per_panel - 1));
+        if (threadIdx.x == 0) s_last = (atomicAdd(v.counter + panel, 1u) == (unsigned)(tiles - 1));
         __syncthreads();
         if (!s_last) return;
         __threadfence();
         if (threadIdx.x < KS) {
             double sum = 0.0;
-            for (int i = 0; i < v.tiles_per_panel; i++)
-                sum += __ldcg(&v.part[((size_t)panel * v.tiles_per_panel + i) * KS + threadIdx.x]);
+            for (int i = 0; i < tiles; i++)
+                sum += __ldcg(&v.part[((size_t)panel * tiles + i) * KS + threadIdx.x]);
             s_rho[threadIdx.x] = sum;
         }
         if (threadIdx.x == 0) v.counter[panel] = 0u;
         __syncthreads();
-    } else if (!last_cta_reduce<KS>(v.part, v.counter + panel, panel, v.tiles_per_panel, 0, v.tiles_per_panel, s_rho)) {
+    } else if (!last_cta_reduce<KS>(v.part, v.counter + panel, panel, tiles, 0, tiles, s_rho)) {
         return;
     }
     int any = 0;
@@ -865,9 +868,13 @@ __global__ void k_gram_mirror(const double* uniq, int nb, int K, double* full) {
     } while (0)
 
 template <typename T, int KS>
-cudaError_t cg_update_ks(const CgVectors<T>& v, const CgState& st, int panels, int wi, int it, cudaStream_t s) {
+cudaError_t cg_update_ks(CgVectors<T> v, const CgState& st, int panels, int wi, int it, cudaStream_t s) {
     constexpr int RPI = VNE_THREADS / (KS / LaneVec<T>::CPL);
-    const int ctas = panels * v.tiles_per_panel;
+    // three row tiles per CTA where that leaves the SMs more than one wave of four
+    // (n = 10^6, 22 columns, per launch: 62 us with one, 57 with two, 53 with
+    // three, 59 with four, 54 with five)
+    v.group = sizeof(T) == 4 && (int64_t)panels * v.tiles_per_panel >= 16 * (int64_t)v.sm_count ? 3 : 1;
+    const int ctas = panels * ((v.tiles_per_panel + v.group - 1) / v.group);
     if constexpr (sizeof(T) == 8) {
         // runs of 16 rows per thread in the largest tile; clusters pay while
         // the tiles alone do not fill the SMs twice

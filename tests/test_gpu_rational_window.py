@@ -28,3 +28,22 @@ def test_windowed_shifts(vctx, fp64, panel, n, shifts, k):
     ref = np.array([rational.rational_quadform(A, X[:, j], sh) for j in range(k)])
     assert np.max(np.abs(psi - ref) / np.abs(ref)) <= (1e-10 if fp64 else 1e-5)
     assert np.all(res <= tol_cg * 1.0000001)
+
+
+@pytest.mark.parametrize("n", [303 * 1024 + 1, 305 * 1024])
+def test_update_over_several_tiles(vctx, n):
+    """FP32 blocks of many row tiles take three of them per CTA of the update
+    (64 columns of 304 or 305 tiles, one or two tiles in the last CTA); eight of
+    the columns alone take one.  Each is within 1e-5 of the exact value."""
+    g = graphs.watts_strogatz(n, 6, 0.2, 3)
+    sh = np.array([1e-6, 1e-5])
+    X = rng.rademacher(5, g.n, 0, 64)
+    mat = vne.matrix_from_graph(vctx, g, fp64=False)
+    opt = vne.options(cg_tol=1e-8, panel=8)
+    try:
+        psi, its, res = vne.vne_quadform_rational(vctx, mat, X, sh, opt=opt)
+        alone, _, _ = vne.vne_quadform_rational(vctx, mat, X[:, 24:32], sh, opt=opt)
+    finally:
+        vne.vne_matrix_destroy(mat)
+    assert np.all(res <= 1e-8 * 1.0000001)
+    assert np.max(np.abs(psi[24:32] - alone) / np.abs(alone)) <= 2e-5
