@@ -631,7 +631,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 rp.norm_beta = p.beta;  // the second pass takes the norm
                 rp.norm_sig_next = p.sig_next;
                 rp.norm_sig = p.sig_cur;
-                rp.norm_tau = P.segs[0].tau;
+                rp.seg = P.d_segs;
                 rp.norm_part = part_u;
                 rp.norm_counter = counter;
                 VNE_TRY_CUDA(ctx, launch_reorth<T>(rp, cp, ks, s));
@@ -709,7 +709,10 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
     } else if (!graph || ctx->profile || cap != cudaStreamCaptureStatusNone) {
         enqueue_loop(st, ctx->profile, 1, m);
     } else {
-        // Graph key: every value the loop's launches depend on.
+        // Graph key: every value the loop's launches depend on.  What belongs to
+        // the matrix or its schedule (thresholds, structure) is either read from
+        // device memory or in the key: another matrix can come to lie at the same
+        // addresses.
         std::string key;
         auto put = [&key](const void* v, size_t b) { key.append(reinterpret_cast<const char*>(v), b); };
         const int ints[] = {(int)sizeof(T), ks, panels, m, variant, (int)interleave, (int)reorth, (int)store_all,
@@ -719,6 +722,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                               pro.omega, pro.sel,     pro.pend_sel, pro.pend, pro.panel_active};
         put(ptrs, sizeof(ptrs));
         put(&slot_elems, sizeof(slot_elems));
+        put(&pro.normM, sizeof(pro.normM));
         put(&p, sizeof(p));
         auto it = ctx->graphs.find(key);
         if (it == ctx->graphs.end()) {

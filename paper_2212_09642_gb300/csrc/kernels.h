@@ -99,6 +99,7 @@ struct ReorthParams {
     int32_t jstride;      // basis vectors per panel in part (>= j)
     int32_t sub;          // update pass: CTAs per row tile
     const RowTile* tiles;
+    const SegInfo* seg;   // the matrix's segment (its breakdown threshold)
     double* part;         // [panels][jstride][tiles][KS]
     const double* coef;   // [j][K]
     const int32_t* panel_active;  // nullable: panels with no column to orthogonalise are skipped
@@ -107,7 +108,6 @@ struct ReorthParams {
     double* norm_beta;     // nullable [K]
     double* norm_sig_next; // [K]
     const double* norm_sig; // [K] sigma_j
-    double norm_tau;       // breakdown threshold
     double* norm_part;     // [panels][tiles * sub][KS]
     uint32_t* norm_counter; // [panels]
 };

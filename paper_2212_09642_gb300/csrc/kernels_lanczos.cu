@@ -1315,7 +1315,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_apply(ReorthParams<T> p)
         if (threadIdx.x < KS) {
             const int c = panel * KS + threadIdx.x;
             const double b = sqrt(tot[threadIdx.x]);
-            const bool stop = !(b > p.norm_tau) || p.norm_sig[c] == 0.0;
+            const bool stop = !(b > p.seg[0].tau) || p.norm_sig[c] == 0.0;
             p.norm_beta[c] = stop ? 0.0 : b;
             p.norm_sig_next[c] = stop ? 0.0 : 1.0 / b;
         }
