@@ -71,6 +71,8 @@ void set_err(vne_ctx* ctx, const char* fmt, ...) {
 
 void* ws_get(vne_ctx* ctx, const std::string& name, size_t bytes, bool zero) {
     WsBuf& b = ctx->ws[name];
+    VNE_REQUIRE(ctx, !ctx->forked || (b.bytes >= bytes && !zero), VNE_EDEVICE,
+                "workspace %s is made or cleared while several streams run", name.c_str());
     if (b.bytes < bytes) {
         dev_free(b.ptr);
         b.ptr = nullptr;
@@ -325,9 +327,11 @@ void fork_streams(vne_ctx* ctx, cudaStream_t s, int groups) {
     if (groups <= 1) return;
     VNE_TRY_CUDA(ctx, cudaEventRecord(ctx->fork_ev, s));
     for (int g = 0; g + 1 < groups; g++) VNE_TRY_CUDA(ctx, cudaStreamWaitEvent(ctx->aux[g], ctx->fork_ev, 0));
+    ctx->forked = true;
 }
 
 void join_streams(vne_ctx* ctx, cudaStream_t s, int groups) {
+    ctx->forked = false;
     for (int g = 0; g + 1 < groups; g++) {
         VNE_TRY_CUDA(ctx, cudaEventRecord(ctx->join_ev[g], ctx->aux[g]));
         VNE_TRY_CUDA(ctx, cudaStreamWaitEvent(s, ctx->join_ev[g], 0));
@@ -741,6 +745,7 @@ void run_block(vne_ctx* ctx, Problem& P, const StartSource& src, const T* panel_
                 try {
                     capture_loop(ctx->cap_stream);
                 } catch (...) {
+                    ctx->forked = false;
                     cudaStreamEndCapture(ctx->cap_stream, &g);
                     if (g) cudaGraphDestroy(g);
                     ctx->launches = l0;
@@ -870,6 +875,18 @@ OpConsts op_consts(vne_ctx* ctx, const Problem& P, int Kp, double shift, const s
     return k;
 }
 
+template <typename T>
+OpWork<T> op_work(vne_ctx* ctx, const Problem& P, int ks, int Kp) {
+    const size_t panels = (size_t)(Kp / ks), nh = std::max<size_t>(P.hubs.size(), 1);
+    OpWork<T> w;
+    w.hub_part = ws_get_t<T>(ctx, "hub_part", panels * std::max(P.hub_slots, 1) * ks);
+    w.hub_cnt = ws_get_t<uint32_t>(ctx, "op.hub_cnt", panels * nh);
+    w.hub_dot = ws_get_t<double>(ctx, "hub_dot", panels * nh * ks);
+    w.part = ws_get_t<double>(ctx, "op.part", panels * std::max(P.ctas_per_panel(), P.tiles_per_panel()) * ks);
+    w.counter = ws_get_t<uint32_t>(ctx, "op.counter", panels);
+    return w;
+}
+
 // Apply the operator to a panel-major block with the Lanczos step kernel:
 // out = A in + shift * in (A = scale M), and dq[c] = scale * (in . out).
 template <typename T>
@@ -894,9 +911,10 @@ void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* ou
     p.hubs = P.d_hubs;
     p.nhubs = std::max(nh, 1);
     p.hub_slots = std::max(P.hub_slots, 1);
-    p.hub_part = ws_get_t<T>(ctx, "hub_part", (size_t)panels * std::max(P.hub_slots, 1) * ks);
-    p.hub_cnt = ws_get_t<uint32_t>(ctx, "op.hub_cnt", (size_t)panels * std::max(nh, 1));
-    p.hub_dot = ws_get_t<double>(ctx, "hub_dot", (size_t)panels * std::max(nh, 1) * ks);
+    const OpWork<T> w = op_work<T>(ctx, P, ks, Kp);
+    p.hub_part = w.hub_part;
+    p.hub_cnt = w.hub_cnt;
+    p.hub_dot = w.hub_dot;
     p.stage_nnz = std::max(P.stage_nnz, 1);
     p.ipw = P.ipw;
     p.tiles = P.d_tiles;
@@ -911,8 +929,8 @@ void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* ou
     p.beta_prev = k.cp;
     p.sig_prev = k.one;
     p.alpha = dq;
-    p.part = ws_get_t<double>(ctx, "op.part", (size_t)panels * std::max(ctas, tiles) * ks);
-    p.counter = ws_get_t<uint32_t>(ctx, "op.counter", (size_t)panels);
+    p.part = w.part;
+    p.counter = w.counter;
     cudaEvent_t e0 = nullptr;
     if (ctx->profile) {
         e0 = ctx_event(ctx);
@@ -937,7 +955,8 @@ void apply_operator(vne_ctx* ctx, Problem& P, int ks, int Kp, const T* in, T* ou
     template std::vector<double> quadforms<T>(vne_matrix*, const vne_options*, StartSource, int, int,             \
                                               const double*);                                                    \
     template void apply_operator<T>(vne_ctx*, Problem&, int, int, const T*, T*, const OpConsts&, double*, int,      \
-                                    const PanelRange*);
+                                    const PanelRange*);                                                          \
+    template OpWork<T> op_work<T>(vne_ctx*, const Problem&, int, int);
 VNE_ENGINE_INSTANTIATE(float)
 VNE_ENGINE_INSTANTIATE(double)
 

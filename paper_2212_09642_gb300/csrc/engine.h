@@ -104,6 +104,7 @@ struct vne_ctx {
     static constexpr int kMaxGroups = 4;
     cudaStream_t aux[kMaxGroups - 1] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[kMaxGroups - 1] = {};
+    bool forked = false;  // between fork and join: no workspace is made or cleared (ws_get refuses)
     int64_t graphs_captured = 0, graphs_replayed = 0;
     int last_steps = 0;  // Lanczos steps of the last quadrature call (largest over its blocks)
     int last_poly_dim = 0;  // polynomial dimension chosen by the switching rule (last rational call)
@@ -243,7 +244,9 @@ void set_err(vne_ctx* ctx, const char* fmt, ...);
 // Workspace buffers grow on demand and are kept for the life of the context,
 // so the hot loop never allocates.  New allocations are zero-filled (the
 // cross-CTA counters rely on starting at zero; the kernels reset them after
-// use).  zero = true clears the requested bytes on every call.
+// use).  zero = true clears the requested bytes on every call.  The clearing is
+// ordered on the context's stream only, so every buffer that work on another
+// stream uses is made before the fork (VNE_EDEVICE otherwise).
 void* ws_get(vne_ctx* ctx, const std::string& name, size_t bytes, bool zero = false);
 
 template <typename T>
@@ -311,7 +314,8 @@ Sched resolve_sched(const vne_matrix* M, const vne_options* o, int block_cols = 
 Problem* matrix_problem(vne_matrix* M, const vne_options* opt);
 // Panels are independent recurrences: `groups` - 1 streams beside s that wait
 // for what s holds now (fork), and s waiting for all of them (join).  They are
-// made before a capture starts (init).
+// made before a capture starts (init).  The work between fork and join finds its
+// workspace made.
 void init_streams(vne_ctx* ctx, int groups);
 void fork_streams(vne_ctx* ctx, cudaStream_t s, int groups);
 void join_streams(vne_ctx* ctx, cudaStream_t s, int groups);
@@ -385,6 +389,17 @@ struct PanelRange {
     cudaStream_t stream;
     int begin, count;
 };
+// Workspace of apply_operator for blocks of Kp columns (a caller that applies it on
+// several streams makes it before they fork).
+template <typename T>
+struct OpWork {
+    T* hub_part;
+    uint32_t* hub_cnt;
+    double *hub_dot, *part;
+    uint32_t* counter;
+};
+template <typename T>
+OpWork<T> op_work(vne_ctx* ctx, const Problem& P, int ks, int Kp);
 // out = A in + shift * in (A = scale M) and dq[c] = scale * (in . out), with
 // the Lanczos step kernel; all panels on the context's stream, or a range.
 template <typename T>

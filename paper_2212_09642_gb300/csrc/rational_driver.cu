@@ -269,10 +269,12 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     };
     // the call's stream waits for the other group whatever happens, so that
     // later work on it (and the reuse of the workspace) comes after
+    op_work<T>(ctx, P, ks, Kp);  // its clearing is ordered before the second group, too
     fork_streams(ctx, st, groups);
     try {
         iterate();
     } catch (...) {
+        ctx->forked = false;
         if (groups > 1) cudaStreamSynchronize(ctx->aux[0]);
         throw;
     }

@@ -1,0 +1,34 @@
+"""Work on streams beside the call's own: what it uses is made before the streams
+fork, and the call's stream continues after all of them."""
+import numpy as np
+import pytest
+
+from oracle import rng
+from paper_2212_09642_gb300 import graphs, vne
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+def test_first_rational_call_of_a_context(fp64):
+    """Conjugate gradients of a small block run their panels in two groups.  The
+    first call of a context, and a later one whose workspace grows, equal the
+    same calls on one stream (a profiled context) bit for bit: three and seven
+    panels of 8, a graph with rows of several work items."""
+    g = graphs.barabasi_albert(30000, 4, 5)
+    assert g.degrees.max() > 2 * 256
+    X = rng.rademacher(7, g.n, 0, 56)
+    out = []
+    for profiled in (False, True):
+        ctx = vne.vne_ctx_create(0)
+        try:
+            vne.vne_ctx_profile(ctx, profiled)
+            mat = vne.matrix_from_graph(ctx, g, fp64=fp64)
+            out.append([vne.vne_quadform_rational(ctx, mat, X[:, :k], None, num_shifts=5, opt=vne.options(panel=8))
+                        for k in (24, 56)])
+            vne.vne_matrix_destroy(mat)
+        finally:
+            vne.vne_ctx_destroy(ctx)
+    for two, one in zip(*out):
+        for a, b in zip(two, one):
+            assert np.array_equal(a, b)
