@@ -21,7 +21,8 @@ struct ColorJob {
     // internal
     cudaStream_t st = nullptr;
     ColorRound p{};
-    int32_t* ctr = nullptr;
+    uint64_t* key = nullptr;
+    int32_t *inv = nullptr, *ctr = nullptr;
     int32_t* h = nullptr;  // pinned host copy of the counters
     int r = 0;
     int64_t prev = 0;
@@ -56,31 +57,26 @@ void device_colorings(vne_matrix* M, std::vector<ColorJob>& jobs) {
         VNE_TRY_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         M->ball2 = h;
     }
+    // every buffer of every job first: their clearing is ordered on the context's
+    // stream, which the jobs' streams follow from here on
     for (int i = 0; i < nj; i++) {
         ColorJob& J = jobs[i];
-        J.st = i == 0 ? ctx->stream : ctx->color_streams[i - 1];
-        if (i > 0) {  // the job's stream follows the work enqueued on the context's stream
-            cudaEvent_t ev = ctx->color_events[2 * (i - 1)];
-            VNE_TRY_CUDA(ctx, cudaEventRecord(ev, ctx->stream));
-            VNE_TRY_CUDA(ctx, cudaStreamWaitEvent(J.st, ev, 0));
-        }
         const std::string w = "col" + std::to_string(i) + ".";
-        uint64_t* key = ws_get_t<uint64_t>(ctx, w + "key", n);
+        J.key = ws_get_t<uint64_t>(ctx, w + "key", n);
         int32_t* color = ws_get_t<int32_t>(ctx, w + "color", n);
         int32_t* blk = ws_get_t<int32_t>(ctx, w + "blk", n);
         int32_t* l0 = ws_get_t<int32_t>(ctx, w + "l0", n);
         int32_t* l1 = ws_get_t<int32_t>(ctx, w + "l1", n);
         J.ctr = ws_get_t<int32_t>(ctx, w + "ctr", 8, true);  // cnt[3], ncolors, overflow, bigcnt[2]
-        int32_t* inv = M->d_node_id ? ws_get_t<int32_t>(ctx, w + "inv", n) : nullptr;
+        J.inv = M->d_node_id ? ws_get_t<int32_t>(ctx, w + "inv", n) : nullptr;
         int32_t* tries = ws_get_t<int32_t>(ctx, w + "tries", n);
-        VNE_TRY_CUDA(ctx, launch_color_init(M->d_rowptr, M->d_node_id, n, key, inv, tries, color, blk, l0, J.st));
-        VNE_TRY_CUDA(ctx, cudaMemcpyAsync(J.ctr, &n32, sizeof(n32), cudaMemcpyHostToDevice, J.st));
+        J.out = ws_get_t<int32_t>(ctx, J.name, n);
         ColorRound& p = J.p;
         p = ColorRound{};
         p.rowptr = M->d_rowptr;
         p.col = M->d_col;
-        p.key = key;
-        p.inv = inv;
+        p.key = J.key;
+        p.inv = J.inv;
         p.color = color;
         p.blk = blk;
         p.tries = tries;
@@ -105,6 +101,30 @@ void device_colorings(vne_matrix* M, std::vector<ColorJob>& jobs) {
         J.r = 0;
         J.prev = n;
         J.done = J.overflow = false;
+    }
+    // the job's streams follow the work enqueued on the context's stream, and
+    // whatever happens they are idle before their buffers can be used again
+    struct Forked {
+        vne_ctx* ctx;
+        int nj;
+        ~Forked() {
+            if (!ctx->forked) return;  // joined
+            ctx->forked = false;
+            for (int i = 1; i < nj; i++) cudaStreamSynchronize(ctx->color_streams[i - 1]);
+        }
+    } region{ctx, nj};
+    ctx->forked = true;
+    for (int i = 0; i < nj; i++) {
+        ColorJob& J = jobs[i];
+        J.st = i == 0 ? ctx->stream : ctx->color_streams[i - 1];
+        if (i > 0) {
+            cudaEvent_t ev = ctx->color_events[2 * (i - 1)];
+            VNE_TRY_CUDA(ctx, cudaEventRecord(ev, ctx->stream));
+            VNE_TRY_CUDA(ctx, cudaStreamWaitEvent(J.st, ev, 0));
+        }
+        VNE_TRY_CUDA(ctx, launch_color_init(M->d_rowptr, M->d_node_id, n, J.key, J.inv, J.p.tries, J.p.color, J.p.blk,
+                                            J.p.list[0], J.st));
+        VNE_TRY_CUDA(ctx, cudaMemcpyAsync(J.ctr, &n32, sizeof(n32), cudaMemcpyHostToDevice, J.st));
     }
     for (;;) {
         bool any = false;
@@ -148,7 +168,6 @@ void device_colorings(vne_matrix* M, std::vector<ColorJob>& jobs) {
             J.rounds = 0;
             continue;
         }
-        J.out = ws_get_t<int32_t>(ctx, J.name, n);
         VNE_TRY_CUDA(ctx, launch_color_scatter(J.p.color, M->d_node_id, n, J.out, J.st));
         ctx->launches++;
         J.s = J.h[3];
@@ -160,6 +179,7 @@ void device_colorings(vne_matrix* M, std::vector<ColorJob>& jobs) {
         VNE_TRY_CUDA(ctx, cudaEventRecord(ev, jobs[i].st));
         VNE_TRY_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ev, 0));
     }
+    ctx->forked = false;
 }
 
 // Colours of M's graph in the caller's numbering, on the device; *rounds =

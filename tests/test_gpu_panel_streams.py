@@ -32,3 +32,23 @@ def test_first_rational_call_of_a_context(fp64):
     for two, one in zip(*out):
         for a, b in zip(two, one):
             assert np.array_equal(a, b)
+
+
+def test_first_colourings_of_a_context():
+    """The three colourings of the probing method run on a stream each.  On a fresh
+    context, and after its workspace grew, the colour counts and T values are
+    those of one colouring at a time."""
+    ctx = vne.vne_ctx_create(0)
+    try:
+        for n in (5000, 40000):
+            g = graphs.random_geometric(n, graphs.rgg_radius_for_degree(n, 6.0), 3)
+            mat = vne.matrix_from_graph(ctx, g, fp64=True, reorder="rcm")
+            est, rep = vne.vne_entropy_probing_auto(ctx, mat, 1e-3, 40)
+            one = {d: vne.vne_matrix_coloring(ctx, mat, g.n, d) for d in {1, 2, 3, rep["d"]}}
+            assert [one[d][1] for d in (1, 2, 3)] == rep["colors_d"]
+            # the same colours handed in, so that no colouring runs on the device
+            est1, rep1 = vne.vne_entropy_probing_auto(ctx, mat, 1e-3, 40, coloring=lambda d: one[d][0])
+            assert np.array_equal(rep["T"], rep1["T"]) and est == est1
+            vne.vne_matrix_destroy(mat)
+    finally:
+        vne.vne_ctx_destroy(ctx)
