@@ -165,7 +165,8 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     const int groups =
         panels >= 2 && !mixed && !ctx->profile && blk * sizeof(T) <= (size_t)16 << 20 ? 2 : 1;
     PanelRange grp[2];
-    if (groups > 1) init_streams(ctx, 3);  // a second group's stream, and one for the flags
+    const int streams = groups > 1 ? 3 : 1;  // a second group's, and one for the flags
+    init_streams(ctx, streams);
     for (int g = 0; g < groups; g++) {
         grp[g].stream = g == 0 ? st : ctx->aux[0];
         grp[g].begin = panels * g / groups;
@@ -267,18 +268,21 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
             if (done) break;
         }
     };
-    // the call's stream waits for the other group whatever happens, so that
-    // later work on it (and the reuse of the workspace) comes after
+    // the call's stream waits for the other group and for the flags' copies (the
+    // last may be under way when max_iter ends the loop) whatever happens, so
+    // that later work on it and the reuse of the workspace and of the pinned
+    // flags come after
     op_work<T>(ctx, P, ks, Kp);  // its clearing is ordered before the second group, too
-    fork_streams(ctx, st, groups);
+    fork_streams(ctx, st, streams);
     try {
         iterate();
     } catch (...) {
         ctx->forked = false;
-        if (groups > 1) cudaStreamSynchronize(ctx->aux[0]);
+        for (int g = 0; g + 1 < streams; g++) cudaStreamSynchronize(ctx->aux[g]);
+        cudaStreamSynchronize(st);
         throw;
     }
-    join_streams(ctx, st, groups);
+    join_streams(ctx, st, streams);
     // polynomial part: K_{n_inf+1}(A, c) by powers of A, or, with the
     // switching rule, K_k(A, c) by the seed residuals
     int kpoly = n_inf + 1;

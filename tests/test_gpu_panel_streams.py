@@ -52,3 +52,27 @@ def test_first_colourings_of_a_context():
             vne.vne_matrix_destroy(mat)
     finally:
         vne.vne_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("max_iter", [4, 5, 6, 7])
+def test_solve_after_one_that_was_stopped(fp64, max_iter):
+    """A solve that cg_max_iter ends with a copy of its activity flags under way,
+    followed at once by a full one: equal to the full one alone."""
+    g = graphs.watts_strogatz(20000, 6, 0.1, 2)
+    X = rng.rademacher(3, g.n, 0, 32)
+    opt = vne.options(panel=8)
+    ctx = vne.vne_ctx_create(0)
+    try:
+        mat = vne.matrix_from_graph(ctx, g, fp64=fp64)
+        want = vne.vne_quadform_rational(ctx, mat, X, None, num_shifts=4, opt=opt)
+        for _ in range(3):
+            _, its, _ = vne.vne_quadform_rational(ctx, mat, X, None, num_shifts=4,
+                                                  opt=vne.options(panel=8, cg_max_iter=max_iter))
+            assert its.max() == max_iter
+            got = vne.vne_quadform_rational(ctx, mat, X, None, num_shifts=4, opt=opt)
+            for a, b in zip(got, want):
+                assert np.array_equal(a, b)
+        vne.vne_matrix_destroy(mat)
+    finally:
+        vne.vne_ctx_destroy(ctx)
