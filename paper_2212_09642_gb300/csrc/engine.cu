@@ -29,8 +29,12 @@ cudaError_t dev_malloc(void** p, size_t bytes) {
     *p = nullptr;
     if (inject_failure()) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaSuccess) g_live_dev++;
-    else *p = nullptr;
+    if (e == cudaSuccess) {
+        g_live_dev++;
+    } else {
+        *p = nullptr;
+        cudaGetLastError();  // reported by the return value; a retry's launches are not to find it
+    }
     return e;
 }
 
@@ -44,8 +48,12 @@ cudaError_t pinned_malloc(void** p, size_t bytes) {
     *p = nullptr;
     if (inject_failure()) return cudaErrorMemoryAllocation;
     cudaError_t e = cudaMallocHost(p, bytes);
-    if (e == cudaSuccess) g_live_pinned++;
-    else *p = nullptr;
+    if (e == cudaSuccess) {
+        g_live_pinned++;
+    } else {
+        *p = nullptr;
+        cudaGetLastError();
+    }
     return e;
 }
 
@@ -84,6 +92,13 @@ void* ws_get(vne_ctx* ctx, const std::string& name, size_t bytes, bool zero) {
     }
     if (zero && bytes) VNE_TRY_CUDA(ctx, cudaMemsetAsync(b.ptr, 0, bytes, ctx->stream));
     return b.ptr;
+}
+
+void ws_drop(vne_ctx* ctx, const std::string& name) {
+    auto it = ctx->ws.find(name);
+    if (it == ctx->ws.end()) return;
+    dev_free(it->second.ptr);
+    ctx->ws.erase(it);
 }
 
 void* pinned_bytes(vne_ctx* ctx, const std::string& name, size_t bytes) {

@@ -248,6 +248,8 @@ void set_err(vne_ctx* ctx, const char* fmt, ...);
 // ordered on the context's stream only, so every buffer that work on another
 // stream uses is made before the fork (VNE_EDEVICE otherwise).
 void* ws_get(vne_ctx* ctx, const std::string& name, size_t bytes, bool zero = false);
+// Give a buffer back (nothing that uses it is in flight).
+void ws_drop(vne_ctx* ctx, const std::string& name);
 
 template <typename T>
 T* ws_get_t(vne_ctx* ctx, const std::string& name, size_t count, bool zero = false) {

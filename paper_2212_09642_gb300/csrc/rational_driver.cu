@@ -6,11 +6,24 @@
 
 namespace {
 
+// Residuals kept between two flushes: 32 make the flush's share of an iteration
+// about one vector per 8 live shifts; fewer when 33 slots would take more than
+// kRingBytes.  The ring of window + 1 slots lies in the buffer of the
+// orthonormalised basis (nb vectors), which is written after the iteration, so
+// the least window, nb - 1, costs no memory.
+constexpr size_t kRingBytes = (size_t)16 << 30;
+constexpr size_t kRetryBytes = (size_t)64 << 20;  // a solve is tried again for at least this much less memory
+int least_window(int nshift, int n_inf) { return std::max(2, (n_inf < 0 ? 1 : n_inf + 1) + nshift - 1); }
+int long_window(int nshift, int n_inf, size_t block_bytes) {
+    return std::max(least_window(nshift, n_inf), (int)std::min<size_t>(32, kRingBytes / block_bytes));
+}
+
 // Rational Krylov quadratic forms (poles -shifts[i] and n_inf poles at
-// infinity) of one start block, by multi-shift CG.
+// infinity) of one start block, by multi-shift CG with residuals kept over
+// `window` iterations.
 template <typename T>
 void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int ks, const double* shifts,
-                    int nshift, int n_inf, double tol, int max_iter, bool desing, int variant, double drop,
+                    int nshift, int n_inf, int window, double tol, int max_iter, bool desing, int variant, double drop,
                     double drop2, std::vector<double>& psi, std::vector<int>& iters, std::vector<double>& resid,
                     int* rank_min, double lam_min = 0.0, double lam_max = 0.0, int* kpoly_out = nullptr) {
     cudaStream_t st = ctx->stream;
@@ -59,14 +72,8 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     }
     // CG vectors.  Residuals go to a ring of window + 1 slots; every `window`
     // iterations one pass adds their combinations to the shifted iterates
-    // (rational.cu).  32 residuals make that pass's share of an iteration
-    // about one vector per 8 live shifts; fewer when 33 slots would take more
-    // than kRingBytes.  The ring lies in the buffer of the orthonormalised
-    // basis (nb vectors), which is written after the iteration.
-    constexpr size_t kRingBytes = (size_t)16 << 30;
+    // (rational.cu).
     const int nb_min = (mixed ? 1 : n_inf + 1) + nshift;
-    const int window = std::max({2, nb_min - 1,
-                                 (int)std::min<size_t>(32, kRingBytes / (blk * sizeof(T)))});
     const int slots = window + 1;
     const char* basis_tag = sizeof(T) == 8 ? "rat.V" : "rat.tw";
     T* ring = ws_get_t<T>(ctx, basis_tag, blk * std::max(slots, nb_min));
@@ -553,8 +560,23 @@ void rational_quadforms(vne_matrix* M, const vne_options* o, StartSource src, in
         std::vector<double> bp, br;
         std::vector<int> bi;
         int rmin = 0, kpoly = 0;
-        rational_block<T>(ctx, *P, s, K, sc.ks, shifts, nshift, n_inf, tol, maxit, M->desing, sc.variant, drop, drop2,
-                          bp, bi, br, &rmin, lam_min, lam_max, &kpoly);
+        auto solve = [&](int window) {
+            rational_block<T>(ctx, *P, s, K, sc.ks, shifts, nshift, n_inf, window, tol, maxit, M->desing, sc.variant,
+                              drop, drop2, bp, bi, br, &rmin, lam_min, lam_max, &kpoly);
+        };
+        const size_t block_bytes = (size_t)((K + sc.ks - 1) / sc.ks) * sc.ks * M->n * sizeof(T);
+        const int least = least_window(nshift, n_inf), window = long_window(nshift, n_inf, block_bytes);
+        try {
+            solve(window);
+        } catch (const Error& e) {
+            // out of memory with the long window: once more without it, if what
+            // it takes is worth speaking of
+            const size_t extra = (size_t)(window - least) * block_bytes;
+            if (e.code != VNE_ENOMEM || extra < kRetryBytes) throw;
+            VNE_TRY_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+            ws_drop(ctx, sizeof(T) == 8 ? "rat.V" : "rat.tw");
+            solve(least);
+        }
         ctx->last_poly_dim = std::max(ctx->last_poly_dim, kpoly);
         for (int c = 0; c < K; c++) psi[b0 + c] = bp[c];
         for (int i = 0; i < nshift; i++)
