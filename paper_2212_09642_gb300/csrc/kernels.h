@@ -369,7 +369,8 @@ struct ColorRound {
 cudaError_t launch_color_init(const int32_t* rowptr, const int32_t* node_id, int64_t n, uint64_t* key,
                               int32_t* inv, int32_t* tries, int32_t* color, int32_t* blk, int32_t* list,
                               cudaStream_t st);
-// *bound (zeroed) = an upper bound of the nodes within distance 2 of a node.
+// *bound (zeroed) = an upper bound of the nodes within distance 2 of a node, cut off where ball_table_bits no longer
+// depends on it.
 cudaError_t launch_ball2_bound(const int32_t* rowptr, const int32_t* col, int64_t n, int32_t* bound, cudaStream_t);
 int ball_table_bits(int d, int ball2);
 cudaError_t launch_color_round(const ColorRound& p, cudaStream_t st);
