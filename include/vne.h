@@ -224,7 +224,12 @@ vne_status vne_matrix_info(const vne_matrix *mat, int64_t *n, int64_t *nnz, doub
  *                 mode only.
  * With VNE_IS_LAPLACIAN (or a pattern matrix) each b is replaced by
  * b - mean(b) 1 (implicit desingularisation, Remark graph-laplacian-krylov),
- * which leaves b^T f(A) b unchanged. */
+ * which leaves b^T f(A) b unchanged.
+ * A column's value depends on the other columns of the call in its last bits:
+ * with the automatic schedule a small graph is given to one of two kernels
+ * by the number of columns (an explicit opt->panel keeps to one).  The
+ * seeded estimators below do not depend on it: a range of probes gives the
+ * bits of the whole. */
 #define VNE_VECTORS_DEVICE 0x1u
 vne_status vne_quadform_batch(vne_matrix *mat, const double *vectors, int32_t k, uint32_t vec_flags,
                               int32_t krylov_steps, const double *poles, int32_t num_poles,
@@ -243,7 +248,10 @@ vne_status vne_quadform_batch(vne_matrix *mat, const double *vectors, int32_t k,
  *   cg_iterations NULL or int32[num_shifts][k]: iterations until each shift converged
  *   residuals     NULL or double[num_shifts][k]: final recursive relative residuals
  * vne_quadform_batch and vne_entropy_probing take the same path when they
- * are given poles. */
+ * are given poles.  With opt->panel = 0 the panels of an FP32 matrix follow
+ * the number of columns, so the last bits of a column's psi, and with them
+ * its iteration counts, depend on it.  A block that does not find room for the
+ * residuals of 32 iterations is solved with fewer, to the same tolerance. */
 vne_status vne_quadform_rational(vne_matrix *mat, const double *vectors, int32_t k, uint32_t vec_flags,
                                  const double *shifts, int32_t num_shifts, const vne_options *opt, double *psi,
                                  int32_t *cg_iterations, double *residuals);

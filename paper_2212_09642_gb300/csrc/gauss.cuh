@@ -5,7 +5,7 @@
 // the CUDA math library's log, cos and sqrt, and GB300 issues 1.7 FP64 lane
 // operations per cycle and SM: 1.25 ms for 9.6 million entries.  Both functions
 // are needed on narrow ranges here, so they are taken from tables and short
-// series with about 28 FP64 instructions and the rest in integer arithmetic,
+// series with 33 FP64 instructions and the rest in integer arithmetic,
 // accurate to a few units of 2^-53 as before:
 //   log u1   u1 = 2^e m, m in [0.75, 1.5); with c_i the reciprocal (to 9 bits) of
 //            the middle of m's interval, r = c_i m - 1 (exact to rounding, |r| <
@@ -114,7 +114,6 @@ __device__ __forceinline__ double gauss_neg_log(double u) {
 // sqrt y for y in [2^-54, 128), or +-0 (tested by its bits: an FP64 comparison
 // would take a slot of the FP64 port)
 __device__ __forceinline__ double gauss_sqrt(double y) {
-    if ((__double_as_longlong(y) << 1) == 0) return 0.0;
     if ((__double_as_longlong(y) << 1) == 0) return 0.0;
     const float r = rsqrtf((float)y);
     const double h = (double)(0.5f * r);

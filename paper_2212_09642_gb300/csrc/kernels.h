@@ -284,6 +284,7 @@ struct CgFlush {
     int32_t n, K, nshift, panels;
     int32_t panel_base;   // first panel of the launch (panels: their number)
     int32_t rows;         // rows per CTA (set by the launcher)
+    int32_t sm_count;
     int32_t count;        // residuals in the window (<= CgState::window)
     int32_t first, last;  // first flush: x and p_s start from zero; last: p_s is not needed any more
     const T* r;           // residual slots, [slots][K / ks][n][ks]

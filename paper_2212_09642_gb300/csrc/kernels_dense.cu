@@ -173,7 +173,7 @@ __host__ __device__ inline bool symtri_qr_first_row(double* d, double* e, double
 // lane runs short independent chains:
 //  * theta_j by bisection on the Sturm count #{theta < z} (number of k with
 //    sign p_k(z) = sign p_{k-1}(z), p_k = det(z I - T_k) by the three-term
-//    recurrence, rescaled by powers of two every four steps; Wilkinson, The
+//    recurrence, rescaled by powers of two every eight steps; Wilkinson, The
 //    Algebraic Eigenvalue Problem, Ch. 5): FP32 counts first narrow the
 //    Gershgorin interval, FP64 counts check the bracket, a bracket that holds
 //    one eigenvalue goes to Newton's iteration on p_n, others are searched on
@@ -1029,7 +1029,7 @@ __global__ void __launch_bounds__(TqCfg<MAXM>::NT)
 // gamma_j = sum_{l != j} a_l b_l / (theta_j - theta_l),
 //   g_m(z) = sum_j a_j^2 b_j^2 f[theta_j, theta_j, z] + 2 a_j b_j gamma_j f[theta_j, z]
 // (divided differences of f, the limits at z = theta_j included; evaluated
-// stably, see dd_entropy), and ||c||^2 min / max of |g_m| over the
+// stably, see g_term), and ||c||^2 min / max of |g_m| over the
 // spectral interval bound the quadrature error from below / above; their
 // geometric mean is the paper's error estimate.  The minimum and maximum are
 // taken over `grid` geometrically and `grid` linearly spaced points of

@@ -17,8 +17,9 @@
 // M is the stored operator (the Laplacian L for a graph, kept implicit) and
 // A = scale * M; alpha and beta here belong to M and are scaled in FP64 by
 // the quadrature.  Inner products are accumulated per lane in the vector
-// precision over at most a few rows, then in FP64 across lanes, warps and
-// CTAs; the cross-CTA sums are done by the last CTA to arrive for each
+// precision over the lane's rows of a CTA (at most 16 with the default
+// schedules, in the step and in the update kernel), then in FP64 across lanes,
+// warps and CTAs; the cross-CTA sums are done by the last CTA to arrive for each
 // (panel, segment), in a fixed order, so results are bit-reproducible.
 #include "common.cuh"
 #include "gauss.cuh"

@@ -32,9 +32,11 @@ constexpr int kSmallWarps = kSmallThreads / 32;
 // Sum of one value per thread, fixed order; the result is valid in warp 0 only
 // (an FP64 operation of all 32 warps holds the port for 32 x 16 cycles, so the
 // scalars that follow are warp 0's too).  `pre`: 2^pre lanes are added in the
-// data precision first (FP32 sums of at most 16 products), then 128 threads, a
-// warp per sub-partition, add the rest in FP64, a shuffle tree and the four
-// warps in order.  Contains two barriers.
+// data precision first, as far as FP32 sums of 16 products allow; a thread's own
+// rows are one FP32 sum (up to 25 at the largest n that small_lanczos_wins
+// admits, and up to eight long rows more in the step, each on lane 0).  Then
+// 128 threads, a warp per sub-partition, add the rest in FP64, a shuffle tree and
+// the four warps in order.  Contains two barriers.
 template <typename T>
 __device__ __forceinline__ double block_sum(T x, int pre, T* s_part, double* s_red) {
     for (int k = 0; k < pre; k++) x += __shfl_xor_sync(0xffffffffu, x, 1 << k);

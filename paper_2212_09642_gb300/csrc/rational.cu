@@ -910,7 +910,7 @@ cudaError_t launch_cg_update(const CgVectors<T>& v, const CgState& st, int ks, i
 template <typename T, int KS>
 cudaError_t cg_flush_ks(CgFlush<T> f, cudaStream_t s) {
     // 1024 rows per CTA, 256 while that leaves SMs without one
-    f.rows = (int64_t)f.panels * f.n >= 1024 * 608 ? 1024 : 256;
+    f.rows = (int64_t)f.panels * f.n >= 4 * 1024 * (int64_t)f.sm_count ? 1024 : 256;
     const size_t smem = (size_t)f.count * kFlushShifts * 2 * KS * sizeof(T);
     if (smem + 4096 > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_cg_flush<T, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,

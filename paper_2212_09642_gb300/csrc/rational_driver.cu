@@ -140,6 +140,7 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     fl.n = n;
     fl.K = Kp;
     fl.nshift = nshift;
+    fl.sm_count = ctx->sm_count;
     fl.panels = panels;
     fl.r = ring;
     fl.slot_stride = blk;
