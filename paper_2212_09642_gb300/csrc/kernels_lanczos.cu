@@ -1306,6 +1306,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_apply(ReorthParams<T> p)
     }
     if (!NORM) return;
     __shared__ double red[VNE_WARPS][KS], tot[KS];
+    const double tau = p.seg[0].tau;  // on its way while the norm is added up
     double nd[V], part;
 #pragma unroll
     for (int e = 0; e < V; e++) nd[e] = (double)nrm[e];
@@ -1316,7 +1317,7 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_apply(ReorthParams<T> p)
         if (threadIdx.x < KS) {
             const int c = panel * KS + threadIdx.x;
             const double b = sqrt(tot[threadIdx.x]);
-            const bool stop = !(b > p.seg[0].tau) || p.norm_sig[c] == 0.0;
+            const bool stop = !(b > tau) || p.norm_sig[c] == 0.0;
             p.norm_beta[c] = stop ? 0.0 : b;
             p.norm_sig_next[c] = stop ? 0.0 : 1.0 / b;
         }
