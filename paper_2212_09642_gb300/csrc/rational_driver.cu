@@ -156,7 +156,12 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     T* rh = mixed ? ws_get_t<T>(ctx, "rat.rhist", blk * (kMixMax - 1)) : nullptr;  // r_1 .. r_{kMixMax-1}
     // the panels' activity flags arrive in pinned memory four iterations after
     // the copy is issued, so that the stream does not run dry while the host
-    // looks at them
+    // looks at them.  A solve may then run eight iterations too many, so the first
+    // kPrompt iterations look at the flags of the iteration itself (n = 200,000,
+    // 16 columns FP64, one pole, 13 iterations: 5.0 ms with 24, 4.5 with 16); the
+    // switching rule counts the first kMixMax of them
+    constexpr int kPrompt = 32;
+    static_assert(kPrompt >= kMixMax, "a short solve's iterations are counted");
     int32_t* any_host = (int32_t*)pinned_bytes(ctx, "rat.any", panels * sizeof(int32_t));
     VNE_REQUIRE(ctx, any_host, VNE_ENOMEM, "pinned allocation failed");
     struct Event {
@@ -264,9 +269,7 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
             }
             it++;
             bool done = it >= max_iter;
-            // the switching rule counts the iterations of a short solve, so it
-            // looks at the flags of the iteration itself
-            const bool lagged = !(mixed && it <= kMixMax);
+            const bool lagged = it > kPrompt;
             if (!done && lagged && (it & 7) == 4) ask();
             if (!done && (it & 7) == 0) {
                 if (!lagged) ask();

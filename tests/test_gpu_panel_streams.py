@@ -55,7 +55,7 @@ def test_first_colourings_of_a_context():
 
 
 @pytest.mark.parametrize("fp64", [False, True])
-@pytest.mark.parametrize("max_iter", [4, 5, 6, 7])
+@pytest.mark.parametrize("max_iter", [4, 7, 36, 37, 38, 39])
 def test_solve_after_one_that_was_stopped(fp64, max_iter):
     """A solve that cg_max_iter ends with a copy of its activity flags under way,
     followed at once by a full one: equal to the full one alone."""
@@ -73,6 +73,34 @@ def test_solve_after_one_that_was_stopped(fp64, max_iter):
             got = vne.vne_quadform_rational(ctx, mat, X, None, num_shifts=4, opt=opt)
             for a, b in zip(got, want):
                 assert np.array_equal(a, b)
+        vne.vne_matrix_destroy(mat)
+    finally:
+        vne.vne_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("tol", [1e-2, 1e-3, 1e-4, 1e-6, 1e-8])
+def test_short_solves_stop_at_the_next_look(fp64, tol):
+    """The conjugate gradients look at the activity flags every eight iterations; a
+    solve of at most 32 ends at the first look after its last shift converged:
+    as many launches as with cg_max_iter set to that iteration."""
+    g = graphs.watts_strogatz(3000, 6, 0.1, 2)
+    X = rng.rademacher(3, g.n, 0, 5)
+    ctx = vne.vne_ctx_create(0)
+
+    def launches(**kw):
+        before = vne.vne_ctx_stats(ctx)[0]
+        out = vne.vne_quadform_rational(ctx, mat, X, None, num_shifts=1, opt=vne.options(cg_tol=tol, **kw))
+        return vne.vne_ctx_stats(ctx)[0] - before, out
+
+    try:
+        mat = vne.matrix_from_graph(ctx, g, fp64=fp64)
+        launches()
+        n, (psi, its, _) = launches()
+        assert its.max() <= 32
+        want, (ref, _, _) = launches(cg_max_iter=(int(its.max()) + 7) // 8 * 8)
+        assert n == want
+        assert np.array_equal(psi, ref)
         vne.vne_matrix_destroy(mat)
     finally:
         vne.vne_ctx_destroy(ctx)
