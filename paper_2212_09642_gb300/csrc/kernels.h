@@ -98,9 +98,10 @@ struct ReorthParams {
     int32_t panel_base;   // first panel of this launch (panels: their number)
     int32_t jstride;      // basis vectors per panel in part (>= j)
     int32_t sub;          // update pass: CTAs per row tile
+    int32_t group, parts; // inner products: row tiles per CTA, CTAs per vector (set by the launcher)
     const RowTile* tiles;
     const SegInfo* seg;   // the matrix's segment (its breakdown threshold)
-    double* part;         // [panels][jstride][tiles][KS]
+    double* part;         // [panels][jstride][parts][KS]
     const double* coef;   // [j][K]
     const int32_t* panel_active;  // nullable: panels with no column to orthogonalise are skipped
     const uint8_t* sel;   // nullable [j][K]: a (panel, i) with no selected column is skipped
@@ -117,7 +118,7 @@ struct ReorthCoefParams {
     const double* sig;    // [j][K] sigma_i of each basis vector
     double* coef;
     int32_t j, K, panels, tiles_per_panel;
-    int32_t panel_base, jstride;  // as in ReorthParams
+    int32_t panel_base, jstride, parts;  // as in ReorthParams
     const uint8_t* sel;           // nullable [j][K]: orthogonalise column c against basis vector i
     const int32_t* panel_active;  // nullable, as in ReorthParams
 };

@@ -1067,18 +1067,19 @@ template <typename T, int KS>
 __global__ void __launch_bounds__(VNE_THREADS) k_reorth_dots(ReorthParams<T> p) {
     constexpr int V = Chunk16<T>::V, G = KS / V;
     static_assert(KS % V == 0 && VNE_THREADS % G == 0, "chunk layout");
-    // grid: panel * tiles * j ; each CTA: one tile, one i
+    // grid: panel * tile groups * j ; each CTA: p.group row tiles, one i
     const int i = blockIdx.x % p.j;
     const int pt = blockIdx.x / p.j;
-    const int panel = p.panel_base + pt / p.tiles_per_panel, tile = pt % p.tiles_per_panel;
+    const int panel = p.panel_base + pt / p.parts, tile = pt % p.parts;
     if (p.panel_active && !p.panel_active[panel]) return;
     if (!reorth_panel_uses<T, KS>(p, panel, i)) return;
-    const RowTile t = p.tiles[tile];
+    RowTile t = p.tiles[tile * p.group];
+    if (p.group > 1) t.row_end = p.tiles[min(p.tiles_per_panel, (tile + 1) * p.group) - 1].row_end;
     const size_t base = (size_t)panel * p.n_total * KS + (size_t)t.row_begin * KS;
     const T* Wi = p.basis + (size_t)i * p.slot_stride + base;
     const T* Wn = p.w + base;
     const int nchunks = (t.row_end - t.row_begin) * G;
-    const size_t opart = (((size_t)panel * p.jstride + i) * p.tiles_per_panel + tile) * KS;
+    const size_t opart = (((size_t)panel * p.jstride + i) * p.parts + tile) * KS;
     if constexpr (sizeof(T) == 8) {
         // FP64 inner products are bound by the FP64 pipe, so the partial sums
         // take as few FP64 additions as possible: each thread accumulates its
@@ -1157,7 +1158,18 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_dots(ReorthParams<T> p) 
     }
 }
 
-// Pass B: fixed-order sum of the tile partials -> coefficients.
+// Row tiles per CTA of k_reorth_dots.  FP32 tiles are short (1024 rows), so a CTA
+// of one spends a third of its time on its FP64 tail, and pass B adds the partials
+// of a vector one after another: four of them per CTA where the vectors and tiles
+// make CTAs enough (n = 10^6, 112 columns, 60 steps, full: 627 ms with one, 549 with
+// four; n = 5 10^5, 64: 184, 162; n = 3 10^5, 64, 100 steps: 288, 251).  The columns of the call do not count,
+// so that a range of probes gives the bits of the whole.
+template <typename T>
+int reorth_group(const ReorthParams<T>& p) {
+    return sizeof(T) == 4 && (int64_t)p.tiles_per_panel * p.j >= 2048 ? 4 : 1;
+}
+
+// Pass B: fixed-order sum of the partials of the tile groups -> coefficients.
 template <int KS>
 __global__ void k_reorth_coef(ReorthCoefParams p) {
     // one thread per (panel, i, c)
@@ -1171,8 +1183,7 @@ __global__ void k_reorth_coef(ReorthCoefParams p) {
         return;
     }
     double s = 0.0;
-    for (int t = 0; t < p.tiles_per_panel; t++)
-        s += p.part[(((size_t)panel * p.jstride + i) * p.tiles_per_panel + t) * KS + c];
+    for (int t = 0; t < p.parts; t++) s += p.part[(((size_t)panel * p.jstride + i) * p.parts + t) * KS + c];
     double sig = p.sig[(size_t)i * p.K + col];
     p.coef[(size_t)i * p.K + col] = sig * sig * s;
 }
@@ -1602,13 +1613,24 @@ cudaError_t launch_step_update_segj(const StepParams<T>& p, int ks, int panels, 
     return cudaGetLastError();
 }
 
+// The two passes that form the coefficients.
+template <typename T>
+static cudaError_t reorth_dots(ReorthParams<T> p, ReorthCoefParams c, int ks, cudaStream_t st) {
+    if (p.jstride < p.j || c.jstride != p.jstride) return cudaErrorInvalidValue;
+    p.group = reorth_group(p);
+    p.parts = c.parts = (p.tiles_per_panel + p.group - 1) / p.group;
+    VNE_DISPATCH_KS(T, ks, (k_reorth_dots<T, KS><<<dim3(p.panels * p.parts * p.j), VNE_THREADS, 0, st>>>(p)));
+    const int total = c.panels * c.j * ks;
+    VNE_DISPATCH_KS(T, ks, (k_reorth_coef<KS><<<dim3((total + 255) / 256), 256, 0, st>>>(c)));
+    return cudaSuccess;
+}
+
 template <typename T>
 cudaError_t launch_reorth(const ReorthParams<T>& p, const ReorthCoefParams& c, int ks, cudaStream_t st) {
     if (p.j <= 0) return cudaSuccess;
-    if (p.j > kReorthMaxJ || p.jstride < p.j || c.jstride != p.jstride) return cudaErrorInvalidValue;
-    VNE_DISPATCH_KS(T, ks, (k_reorth_dots<T, KS><<<dim3(p.panels * p.tiles_per_panel * p.j), VNE_THREADS, 0, st>>>(p)));
-    int total = c.panels * c.j * ks;
-    VNE_DISPATCH_KS(T, ks, (k_reorth_coef<KS><<<dim3((total + 255) / 256), 256, 0, st>>>(c)));
+    if (p.j > kReorthMaxJ) return cudaErrorInvalidValue;
+    const cudaError_t e = reorth_dots(p, c, ks, st);
+    if (e != cudaSuccess) return e;
     const dim3 ga(p.panels * p.tiles_per_panel * p.sub);
     if (p.norm_beta) VNE_DISPATCH_KS(T, ks, (k_reorth_apply<T, KS, true><<<ga, VNE_THREADS, 0, st>>>(p)));
     else VNE_DISPATCH_KS(T, ks, (k_reorth_apply<T, KS, false><<<ga, VNE_THREADS, 0, st>>>(p)));
@@ -1619,11 +1641,8 @@ cudaError_t launch_reorth(const ReorthParams<T>& p, const ReorthCoefParams& c, i
 template <typename T>
 cudaError_t launch_col_dots(const ReorthParams<T>& p, const ReorthCoefParams& c, int ks, cudaStream_t st) {
     if (p.j <= 0) return cudaSuccess;
-    if (p.jstride < p.j || c.jstride != p.jstride) return cudaErrorInvalidValue;
-    VNE_DISPATCH_KS(T, ks, (k_reorth_dots<T, KS><<<dim3(p.panels * p.tiles_per_panel * p.j), VNE_THREADS, 0, st>>>(p)));
-    int total = c.panels * c.j * ks;
-    VNE_DISPATCH_KS(T, ks, (k_reorth_coef<KS><<<dim3((total + 255) / 256), 256, 0, st>>>(c)));
-    return cudaGetLastError();
+    const cudaError_t e = reorth_dots(p, c, ks, st);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T>
