@@ -395,12 +395,13 @@ bool small_lanczos_wins(vne_matrix* M, Problem& P, int K, int m, int reorth) {
         if (m < 12) {
             // few steps: the column's way into the CTA, its basis and the fixed
             // cost of either form count.  Fitted to 1 .. 8 steps, n = 300 .. 12,000,
-            // 1 .. 256 columns (mine within 3 %, theirs within 6 %): n = 12,000, 8
+            // 1 .. 256 columns (mine within 3 %, theirs within 5 %): n = 12,000, 8
             // columns, 2 steps take 0.38 ms here and 0.19 there; n = 3,000, 8, 8 0.40
             // and 0.44
             const double mine = 0.081 + waves * (steps * (0.0070 + 1.28e-6 * nnz) + 2e-7 * gs + 2.45e-6 * n);
-            const double theirs = 0.078 + steps * (0.0407 + 8.2e-5 * (double)std::min<int64_t>(M->maxdeg, 256) +
-                                                   6.3e-7 * n + 6.8e-8 * n * K);
+            const double theirs = 0.082 + 1.2e-9 * gs * K +
+                                  steps * (0.0395 + 8.2e-5 * (double)std::min<int64_t>(M->maxdeg, 256) + 6.2e-7 * n +
+                                           5.8e-8 * n * K);
             if (0.95 * mine >= theirs) return false;  // else as with more steps
         }
         const double mine = 1.2 * (0.10 + waves * (steps * (0.0045 + 4.8e-7 * nnz) + gs / 3.36e6));
