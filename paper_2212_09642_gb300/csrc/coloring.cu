@@ -625,26 +625,21 @@ int ball_table_bits(int d, int ball2) {
 }
 
 template <int TB>
-static cudaError_t color_round_tb(const ColorRound& p, int64_t left, int ctas_per_sm, cudaStream_t st) {
+static cudaError_t color_round_tb(const ColorRound& p, int ctas_per_sm, cudaStream_t st) {
     const int smem = p.d >= 3 ? kCWarps * BallTable<TB>::kWords * (int)sizeof(int32_t) : 0;
     if (smem) {
         cudaError_t e = cudaFuncSetAttribute(k_color_round<TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    // a warp takes 32 nodes at a time, so no more CTAs than the nodes left fill:
-    // with 12 per SM in every round, the late rounds' idle CTAs made a WS graph of
-    // 10^5 nodes at d = 2 4 % slower than 8 per SM did
-    const int64_t filled = (left + kCWarps * 32 - 1) / (kCWarps * 32);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(filled, (int64_t)sm_count() * ctas_per_sm));
-    k_color_round<TB><<<grid, kCWarps * 32, smem, st>>>(p);
+    k_color_round<TB><<<sm_count() * ctas_per_sm, kCWarps * 32, smem, st>>>(p);
     return cudaGetLastError();
 }
 
-cudaError_t launch_color_round(const ColorRound& p, int64_t left, cudaStream_t st) {
-    if (p.d < 3) return color_round_tb<9>(p, left, 12, st);
-    if (p.table_bits == 9) return color_round_tb<9>(p, left, 12, st);
-    if (p.table_bits == 10) return color_round_tb<10>(p, left, 7, st);
-    return color_round_tb<11>(p, left, 4, st);
+cudaError_t launch_color_round(const ColorRound& p, cudaStream_t st) {
+    if (p.d < 3) return color_round_tb<9>(p, 12, st);
+    if (p.table_bits == 9) return color_round_tb<9>(p, 12, st);
+    if (p.table_bits == 10) return color_round_tb<10>(p, 7, st);
+    return color_round_tb<11>(p, 4, st);
 }
 
 int color_big_ctas() { return sm_count(); }

@@ -375,8 +375,7 @@ cudaError_t launch_color_init(const int32_t* rowptr, const int32_t* node_id, int
 // depends on it.
 cudaError_t launch_ball2_bound(const int32_t* rowptr, const int32_t* col, int64_t n, int32_t* bound, cudaStream_t);
 int ball_table_bits(int d, int ball2);
-// One round; at most `left` nodes are uncoloured.
-cudaError_t launch_color_round(const ColorRound& p, int64_t left, cudaStream_t st);
+cudaError_t launch_color_round(const ColorRound& p, cudaStream_t st);
 // d >= 3: the nodes of biglist, one CTA each, with a table in global memory.
 cudaError_t launch_color_big(const ColorRound& p, cudaStream_t st);
 int color_big_ctas();

@@ -136,7 +136,7 @@ void device_colorings(vne_matrix* M, std::vector<ColorJob>& jobs) {
             const int batch = J.prev > 4096 ? 4 : 16;
             for (int b = 0; b < batch; b++, J.r++) {
                 J.p.round = J.r;
-                VNE_TRY_CUDA(ctx, launch_color_round(J.p, J.prev, J.st));
+                VNE_TRY_CUDA(ctx, launch_color_round(J.p, J.st));
                 ctx->launches++;
                 if (J.p.biglist) {
                     VNE_TRY_CUDA(ctx, launch_color_big(J.p, J.st));
