@@ -154,14 +154,14 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     fl.live = cs.any_active + panels;
     const OpConsts op_s0 = op_consts(ctx, P, Kp, s0, "rat.op"), op_a = op_consts(ctx, P, Kp, 0.0, "rat.op0");
     T* rh = mixed ? ws_get_t<T>(ctx, "rat.rhist", blk * (kMixMax - 1)) : nullptr;  // r_1 .. r_{kMixMax-1}
-    // the panels' activity flags arrive in pinned memory four iterations after
-    // the copy is issued, so that the stream does not run dry while the host
-    // looks at them.  A solve may then run eight iterations too many, so the first
-    // kPrompt iterations look at the flags of the iteration itself (n = 200,000,
-    // 16 columns FP64, one pole, 13 iterations: 5.0 ms with 24, 4.5 with 16); the
-    // switching rule counts the first kMixMax of them
-    constexpr int kPrompt = 32;
-    static_assert(kPrompt >= kMixMax, "a short solve's iterations are counted");
+    // the panels' activity flags arrive in pinned memory and are looked at four
+    // iterations after they were asked for, so that the stream does not run dry
+    // meanwhile (a look at the iteration's own flags costs about 0.1 ms of an idle
+    // GPU in a small block).  They are asked for every four iterations at first, so
+    // that a short solve runs at most seven too many (every eight: n = 200,000, 16
+    // columns FP64, one pole took 5.0 ms, now 4.3), and every eight from
+    // kOften on (every four throughout: 2 to 4 % of a long solve of a small block)
+    constexpr int kOften = 64;
     int32_t* any_host = (int32_t*)pinned_bytes(ctx, "rat.any", panels * sizeof(int32_t));
     VNE_REQUIRE(ctx, any_host, VNE_ENOMEM, "pinned allocation failed");
     struct Event {
@@ -206,6 +206,7 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
     };
     const double vec = (double)n * K * sizeof(T);
     int it = 0, flushed = 0;
+    bool asked = false;  // flags of an earlier iteration are on their way
     auto flush = [&](bool last) {
         fl.count = it - flushed;
         fl.first = flushed == 0;
@@ -269,11 +270,16 @@ void rational_block(vne_ctx* ctx, Problem& P, const StartSource& src, int K, int
             }
             it++;
             bool done = it >= max_iter;
-            const bool lagged = it > kPrompt;
-            if (!done && lagged && (it & 7) == 4) ask();
-            if (!done && (it & 7) == 0) {
-                if (!lagged) ask();
-                done = finished();
+            if (!done && mixed && it <= kMixMax) {
+                // the switching rule counts the iterations of a short solve
+                if ((it & 7) == 0) {
+                    ask();
+                    done = finished();
+                }
+            } else if (!done && (it & 3) == 0) {
+                if (asked) done = finished();
+                asked = !done && (it < kOften || (it & 7) == 4);
+                if (asked) ask();
             }
             if (done || it - flushed == window) flush(done);
             if (done) break;
