@@ -1073,8 +1073,9 @@ __global__ void __launch_bounds__(VNE_THREADS) k_reorth_dots(ReorthParams<T> p) 
     const int panel = p.panel_base + pt / p.parts, tile = pt % p.parts;
     if (p.panel_active && !p.panel_active[panel]) return;
     if (!reorth_panel_uses<T, KS>(p, panel, i)) return;
-    RowTile t = p.tiles[tile * p.group];
-    if (p.group > 1) t.row_end = p.tiles[min(p.tiles_per_panel, (tile + 1) * p.group) - 1].row_end;
+    const int group = sizeof(T) == 4 ? p.group : 1;
+    RowTile t = p.tiles[tile * group];
+    if (group > 1) t.row_end = p.tiles[min(p.tiles_per_panel, (tile + 1) * group) - 1].row_end;
     const size_t base = (size_t)panel * p.n_total * KS + (size_t)t.row_begin * KS;
     const T* Wi = p.basis + (size_t)i * p.slot_stride + base;
     const T* Wn = p.w + base;
