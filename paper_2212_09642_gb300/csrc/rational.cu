@@ -30,7 +30,7 @@
 // live shift) / window instead of 6 + 4 per live shift.  Measured at n = 10^6,
 // 22 columns, 8 shifts, FP32, per iteration: update 88 us and flush 46 us
 // against 283 us for the update that touched every live x_s and p_s and 19 us
-// for its scalar kernels (estimate 397 -> 278 ms; update 53 and flush 33 us, 189
+// for its scalar kernels (estimate 397 -> 278 ms; update 53 and flush 33 us, 183
 // ms, with the shapes described at each kernel); FP64, n = 30,000, 12 columns:
 // 23 + 10 us against 51 + 15 us (88 -> 59 ms; 41 ms now).
 // Afterwards the basis W and A W are formed (A^j c by the step kernel,
